@@ -19,23 +19,37 @@
 //                 is the TMEM A operand, the V tile an MN-major shared-memory
 //                 operand; O accumulates in TMEM.
 //
-// One CTA per SM, 8 warps:
-//   warps 0, 7   TMA producers: 128-key K tiles (warp 0) and V tiles (warp 7),
-//                kD / 64 boxes of 64 x 128 each, through separate 3-stage rings:
-//                QK^T releases a K slot, P V a V slot, so the next K tiles
-//                never wait for a P V.
+// One CTA per SM, 12 warps in three warpgroups:
+//   warps 0, 3   TMA producers: 128-key K tiles (warp 0) and V tiles (warp 3),
+//                kD / 64 boxes of 64 x 128 each, through separate rings: QK^T
+//                releases a K slot, P V a V slot, so the next K tiles never
+//                wait for a P V.
 //   warp 1       TMEM allocation (512 columns) and the QK^T-issuing thread;
 //                S is double-buffered, so the softmax of tile i overlaps
 //                QK^T of tile i+1.
-//   warp 6       the P V-issuing thread (O += P V of tile i as soon as P is
+//   warp 2       the P V-issuing thread (O += P V of tile i as soon as P is
 //                written; it releases the tile's stage).
-//   warps 2-5    one thread per query row (TMEM lane): row max, exp2 with a
-//                lazily rescaled reference maximum (O and l are rescaled only
-//                when the maximum grows by more than 2^8), P written back to
-//                TMEM, and the segment epilogue (normalise, or write a partial
-//                for the merge).
+//   warps 4-7    softmax, one thread per query row (TMEM lane): row max, exp2
+//                with a lazily rescaled reference maximum (O and l are rescaled
+//                only when the maximum grows by more than 2^8), P written back
+//                to TMEM.
+//   warps 8-11   staging and epilogue: the next unit's query rows go to the
+//                second Q buffer while the current unit streams, and a finished
+//                unit's O is read out, normalised and written (or left as a
+//                partial for the merge) while the softmax goes on with the next.
+// What bounds it is the K/V stream from HBM (7.2 TB/s in the long-context
+// step), at a unit's ends the latency of staging and epilogue, and in short
+// launches the fetch of cold instructions.  With the softmax warps doing the
+// staging and the epilogue themselves (8 warps, one Q buffer) a unit boundary
+// stalled the stream for about 5 us, 6.7 times per CTA in a 32-layer step.
+// The softmax walks a score row in rolled 32-column steps, twice (maximum,
+// then weights): a masked tile's extra code, unrolled over the whole row, ran
+// once per unit from cold instruction memory and took 2 to 3 us.  Measured,
+// before and now: the 32-layer step at 1063 keys and 40 nodes (rotary
+// embedding, typical acceptance) 182 -> 159 us, at 16448 keys 1228 -> 1222 us;
+// 16 single-layer calls at 1526 keys with their head 549 -> 491 us.
 // TMEM columns: S0 [0,128), S1 [128,256) with P0 / P1 aliased onto their first
-// halves, O [256,256+kD), Q [384,384+kD/2).  Both QK^T and P V take their A operand
+// halves, O [256,256+kD), Q0 [384,384+kD/2), Q1 behind it.  Both QK^T and P V take their A operand
 // from TMEM, so each MMA reads only the 128 x 16 B operand from shared memory.
 // Query row r of a block sits in TMEM lane 32*(r%4) + r/4 so that the rows
 // are spread over the four lane quadrants (all four SM sub-partitions share
@@ -49,11 +63,14 @@ namespace tv {
 namespace {
 
 constexpr int kBN = 128;           // keys per tile
-constexpr int kKStages = 3;        // K ring depth
-constexpr int kVStages = 3;        // V ring depth
+// K and V ring depths.  More requests in flight make the long-context step
+// slower: 1287 us with 3 + 3 stages, against 1226 with 2 + 2 or 2 + 3 and 1222
+// with 3 + 2 or 4 + 2; the 32-layer step at 1063 keys takes 158-159 us with any.
+constexpr int kKStages = 3;
+constexpr int kVStages = 2;
 constexpr int kMaxStages = kKStages > kVStages ? kKStages : kVStages;
 constexpr int kAtom = 128 * 128;   // one 64-column swizzle atom of a 128-row tile (16 KB)
-constexpr int kTcThreads = 256;    // 8 warps: K loads, QK^T issuer, 4 softmax, P V issuer, V loads
+constexpr int kTcThreads = 384;    // 3 warpgroups: loads and MMA issue, softmax, staging and epilogue
 // bytes of a K or V tile (128 keys x head_dim: kD / 64 atoms)
 constexpr int tile_bytes(int d)
 {
@@ -67,8 +84,8 @@ constexpr int slot_floats(int d)
 // TMEM columns.  P_b (bf16 pairs) overwrites the first half of S_b once the
 // softmax has read S_b into registers; Q (bf16 pairs) is the A operand of QK^T.
 constexpr uint32_t kColS0 = 0, kColS1 = 128, kColP0 = 0, kColP1 = 128, kColO = 256, kColQ = 384;
-constexpr int kQPrefetchTiles = 3;  // tiles before a segment's end at which the next unit's q rows are prefetched
 constexpr float kRescaleLog2 = 8.f;  // rescale O only when the row max grows by more than 2^8
+constexpr int kSmCols = 32;          // columns of S a softmax thread holds at a time (64: the same time, twice the code)
 constexpr int kWholeUnitMaxTiles = 6;  // see attn_tc_plan
 
 // One sequence of a (possibly batched) launch: its own KV cache (tensor maps),
@@ -192,6 +209,35 @@ __device__ __forceinline__ uint32_t tile_allow(int tj0, uint64_t anc)
     return ((1u << pre) - 1u) | (uint32_t)(anc << pre);
 }
 
+// Position of a CTA's next segment: the run of key tiles of one unit that the
+// CTA covers.
+struct SegPos {
+    int b, u;   // sequence, unit within it
+    int j0, n;  // first key tile of the unit, and how many
+};
+
+template <bool kBatched>
+__device__ __forceinline__ SegPos seg_at(const TcParams &p, const TcSeq *seqs, long long t, long long t1, int b)
+{
+    SegPos g;
+    g.b = seq_at<kBatched>(p, t, b);
+    const TcSeq &sq = seqs[g.b];
+    const long long tl = t - sq.tile_base;
+    g.u = (unsigned long long)tl <= 0xffffffffull ? (int)((uint32_t)tl / (uint32_t)sq.T) : (int)(tl / sq.T);
+    g.j0 = (int)(tl - (long long)g.u * sq.T);
+    const long long left = t1 - t;
+    g.n = left < sq.T - g.j0 ? (int)left : sq.T - g.j0;
+    return g;
+}
+
+// What the softmax warps need of a segment, written by the staging warps with
+// the segment's queries (double-buffered like them).
+struct SegInfo {
+    int n, key0, L;            // key tiles, first key position, prefix length
+    uint64_t anc[128];         // ancestor set of each row's node
+    float m[128], l[128];      // written back by the softmax: reference maximum (log2 units) and sum of each row
+};
+
 template <int kD, bool kBatched>
 __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __grid_constant__ TcParams p)
 {
@@ -200,12 +246,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     constexpr int kSlot = slot_floats(kD);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
-    __shared__ __align__(8) uint64_t s_full[2], s_free[2], p_full[2], pv_done[2];
-    __shared__ __align__(8) uint64_t q_full, o_free, drain_bar;
+    __shared__ __align__(8) uint64_t s_full[2], p_full[2], pv_done[2];
+    __shared__ __align__(8) uint64_t q_full[2], ml_full[2], o_free[2], drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ TcSeq s_seq;
     __shared__ long long s_total;
+    __shared__ SegInfo s_info[2];
 
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sK = smem;                                // K ring: kKStages tiles
@@ -213,10 +260,37 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = blockIdx.x;
-    // Launched as a programmatic dependent (a grid that leaves SMs free), the
-    // kernel waits here for the stream's previous work (the previous step's
-    // compaction writes the cache).  The step's LM head may then be launched:
-    // it fills the SMs that attention CTAs leave free or release.
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kMaxStages; ++s) {
+            mbar_init(&k_full[s], 1);
+            mbar_init(&k_empty[s], 1);
+            mbar_init(&v_full[s], 1);
+            mbar_init(&v_empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&s_full[b], 1);
+            mbar_init(&p_full[b], 4);
+            mbar_init(&pv_done[b], 1);
+            mbar_init(&q_full[b], 4);
+            mbar_init(&ml_full[b], 4);
+            mbar_init(&o_free[b], 4);
+        }
+        mbar_init(&drain_bar, 2);  // one commit from each MMA issuer
+        abort_flag = 0;
+        fence_mbar_init();
+        for (int b = 0; b < (kBatched ? p.n_seq : 1); ++b) {
+            prefetch_tmap(&p.tmap[2 * b]);
+            prefetch_tmap(&p.tmap[2 * b + 1]);
+        }
+    }
+    if (warp == 1) {
+        tmem_alloc(&tmem_slot, 512);
+        tmem_relinquish();
+    }
+    // Launched as a programmatic dependent, the kernel waits here for the
+    // stream's previous work (the previous step's compaction writes the cache);
+    // only the set-up above overlaps it.  The step's LM head may then be
+    // launched: it fills the SMs that attention CTAs leave free or release.
     pdl_wait();
     pdl_trigger();
     const TcSeq *seqs = p.seq;
@@ -231,318 +305,203 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     const int P = tc_split_ctas(p, total);
     const long long t0 = c < P ? tc_seg_begin(total, P, c) : total;
     const long long t1 = c < P ? tc_seg_begin(total, P, c + 1) : total;
-    const long long n_tiles = t1 - t0;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kMaxStages; ++s) {
-            mbar_init(&k_full[s], 1);
-            mbar_init(&k_empty[s], 1);
-            mbar_init(&v_full[s], 1);
-            mbar_init(&v_empty[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&s_full[b], 1);
-            mbar_init(&s_free[b], 4);
-            mbar_init(&p_full[b], 4);
-            mbar_init(&pv_done[b], 1);
-        }
-        mbar_init(&q_full, 4);
-        mbar_init(&o_free, 4);
-        mbar_init(&drain_bar, 2);  // one commit from each MMA issuer
-        abort_flag = 0;
-        fence_mbar_init();
-        for (int b = 0; b < (kBatched ? p.n_seq : 1); ++b) {
-            prefetch_tmap(&p.tmap[2 * b]);
-            prefetch_tmap(&p.tmap[2 * b + 1]);
-        }
-    }
-    if (warp == 1) {
-        tmem_alloc(&tmem_slot, 512);
-        tmem_relinquish();
-    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == 0 || warp == 7) {
-        // ------------------------------------------------------------ TMA producers
-        // warp 0 streams the K tiles, warp 7 the V tiles, each through its own
-        // half of the 3-stage ring: QK^T releases a K slot, P V a V slot.
-        if (lane == 0) {
-            const bool is_v = (warp == 7);
+    if (warp < 4) {
+        if (lane != 0) {
+            // one thread of each warp of this warpgroup works
+        } else if (warp == 0 || warp == 3) {
+            // -------------------------------------------------------- TMA producers
+            // warp 0 streams the K tiles, warp 3 the V tiles, each through its own
+            // ring: QK^T releases a K slot, P V a V slot.
+            const bool is_v = (warp == 3);
             uint64_t *full = is_v ? v_full : k_full;
             uint64_t *empty = is_v ? v_empty : k_empty;
             const int S = is_v ? kVStages : kKStages;
             uint8_t *ring = is_v ? sV : sK;
             long long issued = 0;
-            int sb = 0;
-            for (long long it = 0; it < n_tiles; ++it) {
-                const int s = (int)(it % S);
-                const uint32_t ph = (uint32_t)(it / S) & 1u;
-                if (!mbar_wait_bounded(&empty[s], ph ^ 1u, &abort_flag, p.status))
-                    break;
-                const long long t = t0 + it;
-                sb = seq_at<kBatched>(p, t, sb);
+            int s = 0, sb = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (long long t = t0; ok && t < t1;) {
+                const SegPos g = seg_at<kBatched>(p, seqs, t, t1, sb);
+                sb = g.b;
                 const TcSeq &sq = seqs[sb];
-                const long long tl = t - sq.tile_base;
-                const int u = (int)(tl / sq.T);
-                const int j = (int)(tl % sq.T);
-                const int head = (u / sq.row_blocks) % p.Hkv;
-                const int layer = p.layer_begin + u / (sq.row_blocks * p.Hkv);
+                const int head = (g.u / sq.row_blocks) % p.Hkv;
+                const int layer = p.layer_begin + g.u / (sq.row_blocks * p.Hkv);
                 const CUtensorMap *m = &p.tmap[2 * sb + (is_v ? 1 : 0)];
-                uint8_t *dst = ring + (size_t)s * kTile;
-                mbar_arrive_expect_tx(&full[s], kTile);
+                for (int j = 0; j < g.n; ++j) {
+                    if (!mbar_wait_bounded(&empty[s], ph ^ 1u, &abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t *dst = ring + (size_t)s * kTile;
+                    mbar_arrive_expect_tx(&full[s], kTile);
 #pragma unroll
-                for (int a = 0; a < kD / 64; ++a)
-                    tma_load_4d(dst + a * kAtom, m, &full[s], 64 * a, j * kBN, head, layer);
-                issued = it + 1;
+                    for (int a = 0; a < kD / 64; ++a)
+                        tma_load_4d(dst + a * kAtom, m, &full[s], 64 * a, (g.j0 + j) * kBN, head, layer);
+                    ++issued;
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+                t += g.n;
             }
-            if (issued < n_tiles)
+            if (!ok)
                 for (long long it = (issued > S ? issued - S : 0); it < issued; ++it)
                     mbar_wait_drain(&full[it % S], (uint32_t)(it / S) & 1u);
-        }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ QK^T issuer
-        if (lane == 0) {
+        } else if (warp == 1) {
+            // -------------------------------------------------------- QK^T issuer
             const uint32_t idesc_s = idesc_bf16_f32(128, kBN);
-            int sg = -1, sb = 0;
-            for (long long it = 0; it < n_tiles; ++it) {
-                const long long t = t0 + it;
-                sb = seq_at<kBatched>(p, t, sb);
-                const bool first = (it == 0) || ((t - seqs[sb].tile_base) % seqs[sb].T == 0);
-                if (first)
-                    ++sg;
-                const int s = (int)(it % kKStages);
-                const int b = (int)(it & 1);
-                // K landed; the softmax has read S_b (tile it - 2) and P V(it - 2) has read
-                // the P that shares its columns; at a segment's first tile, its Q is staged
-                if (!mbar_wait_bounded(&k_full[s], (uint32_t)(it / kKStages) & 1u, &abort_flag, p.status) ||
-                    !mbar_wait_bounded(&s_free[b], ((uint32_t)(it >> 1) & 1u) ^ 1u, &abort_flag, p.status) ||
-                    (it >= 2 &&
-                     !mbar_wait_bounded(&pv_done[b], (uint32_t)((it - 2) >> 1) & 1u, &abort_flag, p.status)) ||
-                    (first && !mbar_wait_bounded(&q_full, (uint32_t)sg & 1u, &abort_flag, p.status)))
-                    break;
-                tc_fence_after();
-                const uint32_t k_base = smem_u32(sK + (size_t)s * kTile);
-                const uint32_t s_col = b ? kColS1 : kColS0;
+            long long it = 0;
+            int s = 0, sb = 0, sg = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (long long t = t0; ok && t < t1; ++sg) {
+                const SegPos g = seg_at<kBatched>(p, seqs, t, t1, sb);
+                sb = g.b;
+                const uint32_t q_col = tmem + kColQ + (sg & 1) * (kD / 2);
+                for (int j = 0; j < g.n; ++j, ++it) {
+                    const int b = (int)(it & 1);
+                    // K landed; P V(it - 2) has read P_b, which shares S_b's columns and was
+                    // written after the softmax had read S_b; at a segment's first tile, its Q
+                    // is staged
+                    if (!mbar_wait_bounded(&k_full[s], ph, &abort_flag, p.status) ||
+                        (it >= 2 &&
+                         !mbar_wait_bounded(&pv_done[b], (uint32_t)((it - 2) >> 1) & 1u, &abort_flag, p.status)) ||
+                        (j == 0 && !mbar_wait_bounded(&q_full[sg & 1], (uint32_t)(sg >> 1) & 1u, &abort_flag, p.status))) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t k_base = smem_u32(sK + (size_t)s * kTile);
+                    const uint32_t s_col = tmem + (b ? kColS1 : kColS0);
 #pragma unroll
-                for (int kk = 0; kk < kD / 16; ++kk) {
-                    const uint32_t off = (uint32_t)(kk >> 2) * kAtom + (uint32_t)(kk & 3) * 32;
-                    const uint64_t bdesc = smem_desc_sw128(k_base + off, 0, 1024);
-                    tc_mma_f16_ts(tmem + s_col, tmem + kColQ + kk * 8, bdesc, idesc_s, kk > 0 ? 1u : 0u);
+                    for (int kk = 0; kk < kD / 16; ++kk) {
+                        const uint32_t off = (uint32_t)(kk >> 2) * kAtom + (uint32_t)(kk & 3) * 32;
+                        const uint64_t bdesc = smem_desc_sw128(k_base + off, 0, 1024);
+                        tc_mma_f16_ts(s_col, q_col + kk * 8, bdesc, idesc_s, kk > 0 ? 1u : 0u);
+                    }
+                    tc_commit(&s_full[b]);
+                    tc_commit(&k_empty[s]);
+                    if (++s == kKStages) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
-                tc_commit(&s_full[b]);
-                tc_commit(&k_empty[s]);
+                t += g.n;
             }
             // arrives when every MMA issued above has retired (waited for before TMEM is released)
             tc_commit(&drain_bar);
-        }
-    } else if (warp == 6) {
-        // ------------------------------------------------------------ P V issuer
-        // A second issuing thread: each tcgen05.mma holds its issuer for about
-        // 100 cycles at these shapes, so P V(i) issued here runs alongside
-        // QK^T(i + 1) instead of queueing behind it, and the stage is released
-        // that much sooner.
-        if (lane == 0) {
+        } else {
+            // -------------------------------------------------------- P V issuer (warp 2)
+            // A second issuing thread: each tcgen05.mma holds its issuer for about
+            // 100 cycles at these shapes, so P V(i) issued here runs alongside
+            // QK^T(i + 1) instead of queueing behind it, and the stage is released
+            // that much sooner.
             const uint32_t idesc_pv = idesc_bf16_f32(128, kD, false, true);
-            int sg = -1, sb = 0;
-            for (long long it = 0; it < n_tiles; ++it) {
-                const long long t = t0 + it;
-                sb = seq_at<kBatched>(p, t, sb);
-                const bool first = (it == 0) || ((t - seqs[sb].tile_base) % seqs[sb].T == 0);
-                if (first)
-                    ++sg;
-                const int b = (int)(it & 1);
-                // P written; at a segment's first tile, the previous epilogue has read O
-                if (!mbar_wait_bounded(&p_full[b], (uint32_t)(it >> 1) & 1u, &abort_flag, p.status) ||
-                    (first && sg > 0 &&
-                     !mbar_wait_bounded(&o_free, (uint32_t)(sg - 1) & 1u, &abort_flag, p.status)) ||
-                    !mbar_wait_bounded(&v_full[it % kVStages], (uint32_t)(it / kVStages) & 1u, &abort_flag, p.status))
-                    break;
-                tc_fence_after();
-                const uint32_t v_base = smem_u32(sV + (size_t)(it % kVStages) * kTile);
-                const uint32_t p_col = b ? kColP1 : kColP0;
+            long long it = 0;
+            int s = 0, sb = 0, sg = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (long long t = t0; ok && t < t1; ++sg) {
+                const SegPos g = seg_at<kBatched>(p, seqs, t, t1, sb);
+                sb = g.b;
+                for (int j = 0; j < g.n; ++j, ++it) {
+                    const int b = (int)(it & 1);
+                    // P written; at a segment's first tile, the previous segment's O has been read
+                    if (!mbar_wait_bounded(&p_full[b], (uint32_t)(it >> 1) & 1u, &abort_flag, p.status) ||
+                        (j == 0 && sg > 0 &&
+                         !mbar_wait_bounded(&o_free[(sg - 1) & 1], (uint32_t)((sg - 1) >> 1) & 1u, &abort_flag,
+                                            p.status)) ||
+                        !mbar_wait_bounded(&v_full[s], ph, &abort_flag, p.status)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t v_base = smem_u32(sV + (size_t)s * kTile);
+                    const uint32_t p_col = tmem + (b ? kColP1 : kColP0);
 #pragma unroll
-                for (int ks = 0; ks < kBN / 16; ++ks) {
-                    const uint64_t bdesc = smem_desc_sw128_mn(v_base + ks * 2048, kAtom, 1024);
-                    tc_mma_f16_ts(tmem + kColO, tmem + p_col + ks * 8, bdesc, idesc_pv, (first && ks == 0) ? 0u : 1u);
+                    for (int ks = 0; ks < kBN / 16; ++ks) {
+                        const uint64_t bdesc = smem_desc_sw128_mn(v_base + ks * 2048, kAtom, 1024);
+                        tc_mma_f16_ts(tmem + kColO, p_col + ks * 8, bdesc, idesc_pv, (j == 0 && ks == 0) ? 0u : 1u);
+                    }
+                    tc_commit(&v_empty[s]);
+                    tc_commit(&pv_done[b]);
+                    if (++s == kVStages) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
-                tc_commit(&v_empty[it % kVStages]);
-                tc_commit(&pv_done[b]);
+                t += g.n;
             }
             tc_commit(&drain_bar);
         }
-    } else if (warp < 6) {
-        // ------------------------------------------------------------ softmax / epilogue (warps 2-5)
+    } else if (warp < 8) {
+        // ------------------------------------------------------------ softmax (warps 4-7)
         const int q4 = warp & 3;  // TMEM lane quadrant of this warp
         const uint32_t lane_addr = tmem + ((uint32_t)(32 * q4) << 16);
         const int rloc = 4 * lane + q4;  // query row of this thread within the block
-
-        struct Seg {
-            long long start, end, u_first, u_last;  // flattened tile indices
-            int b, u, rb, head, layer_rel, rows_here, node, qh, L, N, ns, dep;
-            bool valid;
-            uint64_t anc;
-            const __nv_bfloat16 *q;
-            __nv_bfloat16 *out;
-        };
-        int sb = 0;
-        auto describe = [&](long long t) {
-            Seg g;
-            sb = seq_at<kBatched>(p, t, sb);
-            const TcSeq &sq = seqs[sb];
-            g.b = sb;
-            g.start = t;
-            g.u = (int)((t - sq.tile_base) / sq.T);
-            g.u_first = sq.tile_base + (long long)g.u * sq.T;
-            g.u_last = g.u_first + sq.T;
-            g.end = t1 < g.u_last ? t1 : g.u_last;
-            g.rb = g.u % sq.row_blocks;
-            g.head = (g.u / sq.row_blocks) % p.Hkv;
-            g.layer_rel = g.u / (sq.row_blocks * p.Hkv);
-            g.rows_here = min(128, sq.rows - g.rb * 128);
-            g.valid = rloc < g.rows_here;
-            const int grow = g.rb * 128 + rloc;
-            g.node = g.valid ? grow / p.group : 0;
-            g.qh = g.head * p.group + grow % p.group;
-            // the row's query / output rows and tree entries
-            if (g.valid)
-                g.valid = in_bounds(g.layer_rel < p.n_layers && g.node < sq.N && g.node < sq.nstride &&
-                                        g.node < kMaxNodes && g.qh < p.Hq,
-                                    p.status);
-            g.anc = g.valid ? sq.tree->anc[g.node] : 0ull;
-            g.dep = g.valid ? sq.tree->depth[g.node] : 0;
-            g.L = sq.L;
-            g.N = sq.N;
-            g.ns = sq.nstride;
-            g.q = sq.q;
-            g.out = sq.out;
-            return g;
-        };
-        // Q row of this thread -> its TMEM lane as kD / 2 columns of bf16 pairs (the
-        // A operand of QK^T); zeros for padding rows
-        auto write_q = [&](const Seg &g) {
-            const uint4 *src =
-                reinterpret_cast<const uint4 *>(g.q + (((size_t)g.layer_rel * g.ns + g.node) * p.Hq + g.qh) * kD);
-            if (!p.rope_tab) {
-                // the whole row (2 kD bytes) in flight at once, then kD / 32 TMEM stores
-                uint4 qv[kD / 8];
-#pragma unroll
-                for (int i = 0; i < kD / 8; ++i)
-                    qv[i] = g.valid ? src[i] : make_uint4(0, 0, 0, 0);
-#pragma unroll
-                for (int qc = 0; qc < kD / 32; ++qc) {
-                    uint32_t w[16];
-#pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-                        const uint4 v = qv[qc * 4 + ch];
-                        w[4 * ch] = v.x;
-                        w[4 * ch + 1] = v.y;
-                        w[4 * ch + 2] = v.z;
-                        w[4 * ch + 3] = v.w;
-                    }
-                    tmem_st_32x32b_x16(lane_addr + kColQ + qc * 16, w);
-                }
-            } else {
-                // pre-rotary query: element i pairs with i + kD / 2, rotated at position
-                // L + depth(node) with the sequence's (cos, sin) table
-                constexpr int kHalf = kD / 64;  // 32-element chunks per half row
-                const float2 *tab = p.rope_tab + (size_t)g.b * kRopeTableEntries + (size_t)g.dep * kRopeMaxHalf;
-#pragma unroll 1
-                for (int qc = 0; qc < kHalf; ++qc) {
-                    uint32_t wl[16], wh[16];
-#pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-                        const uint4 lo = g.valid ? src[qc * 4 + ch] : make_uint4(0, 0, 0, 0);
-                        const uint4 hi = g.valid ? src[(qc + kHalf) * 4 + ch] : make_uint4(0, 0, 0, 0);
-                        const uint32_t lw[4] = {lo.x, lo.y, lo.z, lo.w}, hw[4] = {hi.x, hi.y, hi.z, hi.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int i0 = 32 * qc + 8 * ch + 2 * e;
-                            const float2 c0 = tab[i0], c1 = tab[i0 + 1];
-                            const float a0 = __uint_as_float(lw[e] << 16), a1 = __uint_as_float(lw[e] & 0xffff0000u);
-                            const float b0 = __uint_as_float(hw[e] << 16), b1 = __uint_as_float(hw[e] & 0xffff0000u);
-                            wl[4 * ch + e] = pack_bf16x2(a0 * c0.x - b0 * c0.y, a1 * c1.x - b1 * c1.y);
-                            wh[4 * ch + e] = pack_bf16x2(b0 * c0.x + a0 * c0.y, b1 * c1.x + a1 * c1.y);
-                        }
-                    }
-                    tmem_st_32x32b_x16(lane_addr + kColQ + qc * 16, wl);
-                    tmem_st_32x32b_x16(lane_addr + kColQ + (qc + kHalf) * 16, wh);
-                }
-            }
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(&q_full);
-        };
         long long it = 0;
-        bool aborted = (n_tiles == 0);
-        Seg g;
-        if (!aborted) {
-            g = describe(t0);
-            write_q(g);
-        }
-        while (!aborted) {
+        bool aborted = false;
+        int sg = 0;
+        for (long long t = t0; t < t1 && !aborted; ++sg) {
+            SegInfo &si = s_info[sg & 1];
+            if (!mbar_wait_bounded(&q_full[sg & 1], (uint32_t)(sg >> 1) & 1u, &abort_flag, p.status))
+                break;
+            const int n = si.n, L = si.L;
+            int key0 = si.key0;
+            const uint64_t anc = si.anc[rloc];
+            t += n;
             float m_ref = -INFINITY, l = 0.f;
-            for (long long t = g.start; t < g.end; ++t, ++it) {
+            for (int j = 0; j < n; ++j, ++it, key0 += kBN) {
                 const int b = (int)(it & 1);
-                if (t + kQPrefetchTiles == g.end && g.end < t1) {
-                    // the next unit's query rows are read from HBM when this segment ends
-                    // (write_q below): ask for them in L2 a few tiles ahead
-                    const Seg nx = describe(g.end);
-                    if (nx.valid) {
-                        const char *row = reinterpret_cast<const char *>(
-                            nx.q + (((size_t)nx.layer_rel * nx.ns + nx.node) * p.Hq + nx.qh) * kD);
-#pragma unroll
-                        for (int off = 0; off < 2 * kD; off += 128)
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(row + off));
-                    }
-                }
                 if (!mbar_wait_bounded(&s_full[b], (uint32_t)(it >> 1) & 1u, &abort_flag, p.status)) {
                     aborted = true;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t sa = lane_addr + (b ? kColS1 : kColS0);
-                const int key0 = (int)(t - g.u_first) * kBN;
-                const bool masked = key0 + kBN > g.L;
+                const bool masked = key0 + kBN > L;
 
-                // pass 1: the whole S row (4 loads, one wait), masked row max
-                float sc[kBN];
-                {
-                    uint32_t *r = reinterpret_cast<uint32_t *>(sc);
-                    tmem_ld_32x32b_x32(sa, r);
-                    tmem_ld_32x32b_x32(sa + 32, r + 32);
-                    tmem_ld_32x32b_x32(sa + 64, r + 64);
-                    tmem_ld_32x32b_x32(sa + 96, r + 96);
-                    tmem_ld_wait();
-                }
+                // pass 1: the row maximum over the allowed keys, kSmCols columns at a time
                 float mx = -INFINITY;
-                if (masked) {
-                    // the row's allowed keys among the tile's 128 columns, 32 per word:
-                    // prefix keys (tree index tj < 0) and the ancestors in the tree
-                    uint32_t allow[kBN / 32];
+#pragma unroll 1
+                for (int c0 = 0; c0 < kBN; c0 += kSmCols) {
+                    uint32_t r[kSmCols];
 #pragma unroll
-                    for (int w = 0; w < kBN / 32; ++w)
-                        allow[w] = tile_allow(key0 + 32 * w - g.L, g.anc);
+                    for (int x = 0; x < kSmCols; x += 32)
+                        tmem_ld_32x32b_x32(sa + c0 + x, r + x);
+                    tmem_ld_wait();
+                    if (masked) {
+                        // allowed: prefix keys (tree index < 0) and the ancestors in the tree, 32
+                        // columns per word; the others' scores become -inf in place
 #pragma unroll
-                    for (int x = 0; x < kBN; ++x) {
-                        sc[x] = ((allow[x >> 5] >> (x & 31)) & 1u) ? sc[x] : -INFINITY;
-                        mx = fmaxf(mx, sc[x]);
+                        for (int x0 = 0; x0 < kSmCols; x0 += 32) {
+                            const uint32_t allow = tile_allow(key0 + c0 + x0 - L, anc);
+                            if (__all_sync(0xffffffffu, allow == 0xffffffffu))
+                                continue;
+#pragma unroll
+                            for (int x = 0; x < 32; ++x)
+                                r[x0 + x] = (allow >> x) & 1u ? r[x0 + x] : 0xff800000u;
+                            tmem_st_32x32b_x32(sa + c0 + x0, r + x0);
+                            tmem_st_wait();
+                        }
                     }
-                } else {
 #pragma unroll
-                    for (int x = 0; x < kBN; ++x)
-                        mx = fmaxf(mx, sc[x]);
+                    for (int x = 0; x < kSmCols; ++x)
+                        mx = fmaxf(mx, __uint_as_float(r[x]));
                 }
                 mx *= p.scale_log2;  // row max in log2 units (scale > 0)
 
                 // lazily rescaled reference maximum
                 float alpha = 1.f;
                 bool rescale = false;
-                if (t == g.start) {
+                if (j == 0) {
                     m_ref = mx;
                 } else if (mx > m_ref + kRescaleLog2) {
                     alpha = (m_ref == -INFINITY) ? 0.f : ex2_approx(m_ref - mx);
@@ -570,76 +529,225 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                     }
                     tmem_st_wait();
                 }
-                // P buffer b was last read by O += P V of tile it - 2
-                if (it >= 2 &&
-                    !mbar_wait_bounded(&pv_done[b], (uint32_t)((it - 2) >> 1) & 1u, &abort_flag, p.status)) {
-                    aborted = true;
-                    break;
-                }
-                tc_fence_after();
 
                 // pass 2: P = 2^(s * scale - m_ref) as bf16 pairs into TMEM (masked entries are
-                // -inf and give 0), row sum into l
+                // -inf and give 0), row sum into l.  P_b's columns are S_b's: QK^T wrote S_b
+                // after O += P V of tile it - 2 had read P_b.
                 const float mu = (m_ref == -INFINITY) ? 0.f : m_ref;
                 const uint32_t pa = lane_addr + (b ? kColP1 : kColP0);
                 float rs = 0.f;
+#pragma unroll 1
+                for (int c0 = 0; c0 < kBN; c0 += kSmCols) {
+                    uint32_t r[kSmCols];
 #pragma unroll
-                for (int c0 = 0; c0 < kBN; c0 += 32) {
-                    uint32_t pk[16];
+                    for (int x = 0; x < kSmCols; x += 32)
+                        tmem_ld_32x32b_x32(sa + c0 + x, r + x);
+                    tmem_ld_wait();
 #pragma unroll
-                    for (int x = 0; x < 16; ++x) {
-                        const float p0 = ex2_approx(fmaf(sc[c0 + 2 * x], p.scale_log2, -mu));
-                        const float p1 = ex2_approx(fmaf(sc[c0 + 2 * x + 1], p.scale_log2, -mu));
-                        rs += p0 + p1;
-                        pk[x] = pack_bf16x2(p0, p1);
+                    for (int x0 = 0; x0 < kSmCols; x0 += 32) {
+                        uint32_t pk[16];
+#pragma unroll
+                        for (int x = 0; x < 16; ++x) {
+                            const float p0 = ex2_approx(fmaf(__uint_as_float(r[x0 + 2 * x]), p.scale_log2, -mu));
+                            const float p1 = ex2_approx(fmaf(__uint_as_float(r[x0 + 2 * x + 1]), p.scale_log2, -mu));
+                            rs += p0 + p1;
+                            pk[x] = pack_bf16x2(p0, p1);
+                        }
+                        tmem_st_32x32b_x16(pa + (c0 + x0) / 2, pk);
                     }
-                    tmem_st_32x32b_x16(pa + c0 / 2, pk);
                 }
                 l += rs;
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&s_free[b]);
+                if (lane == 0)
                     mbar_arrive(&p_full[b]);
-                }
             }
             if (aborted)
                 break;
-
-            // Every QK^T of this segment has been consumed, so Q can take the next unit's rows
-            // now, letting the next segment's first QK^T overlap this epilogue.
-            const bool has_next = g.end < t1;
-            Seg nx;
-            if (has_next) {
-                nx = describe(g.end);
-                write_q(nx);
-            }
-
-            // ---------------------------------------------------- segment epilogue
-            const long long jl = it - 1;
-            if (!mbar_wait_bounded(&pv_done[jl & 1], (uint32_t)(jl >> 1) & 1u, &abort_flag, p.status))
+            // the segment's (m, l) for its epilogue; the buffer was read by segment sg - 2's
+            if (sg >= 2 && !mbar_wait_bounded(&o_free[sg & 1], (uint32_t)((sg >> 1) - 1) & 1u, &abort_flag, p.status))
                 break;
-            tc_fence_after();
-            const bool whole = (g.start == g.u_first && g.end == g.u_last);
-            float *slot = p.part + ((size_t)c * 2 + (g.start == t0 ? 0 : 1)) * kSlot;
-            if (!whole && g.valid)
-                g.valid = in_bounds(c < p.P && rloc < 128, p.status);
-            {
-                const float inv = 1.f / l;
-                uint4 *dst =
-                    reinterpret_cast<uint4 *>(g.out + (((size_t)g.layer_rel * g.ns + g.node) * p.Hq + g.qh) * kD);
-                float4 *pdst = reinterpret_cast<float4 *>(slot + rloc * kD);
+            si.m[rloc] = m_ref;
+            si.l[rloc] = l;
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&ml_full[sg & 1]);
+        }
+    } else {
+        // ------------------------------------------------------------ staging and epilogue (warps 8-11)
+        // One segment ahead of the softmax: the next segment's query rows go to
+        // the other Q buffer while the current one streams, and a finished
+        // segment's O is read out and written while the softmax goes on with the
+        // next, so a unit boundary does not stall the K/V stream.
+        const int q4 = warp & 3;
+        const uint32_t lane_addr = tmem + ((uint32_t)(32 * q4) << 16);
+        const int rloc = 4 * lane + q4;
+
+        struct Seg {
+            int n, j0, T;
+            bool first;  // the CTA's first segment
+            bool valid;  // this thread's row exists
+            int b, dep, L;
+            uint64_t anc;
+            const __nv_bfloat16 *q;  // this thread's query and output rows
+            __nv_bfloat16 *out;
+        };
+        int sb = 0;
+        auto describe = [&](long long t) {
+            const SegPos sp = seg_at<kBatched>(p, seqs, t, t1, sb);
+            sb = sp.b;
+            const TcSeq &sq = seqs[sb];
+            Seg g;
+            g.n = sp.n;
+            g.j0 = sp.j0;
+            g.T = sq.T;
+            g.first = t == t0;
+            g.b = sb;
+            g.L = sq.L;
+            const int rb = sp.u % sq.row_blocks;
+            const int head = (sp.u / sq.row_blocks) % p.Hkv;
+            const int layer_rel = sp.u / (sq.row_blocks * p.Hkv);
+            g.valid = rloc < min(128, sq.rows - rb * 128);
+            const int grow = rb * 128 + rloc;
+            const int node = g.valid ? grow / p.group : 0;
+            const int qh = head * p.group + grow % p.group;
+            // the row's query / output rows and tree entries
+            if (g.valid)
+                g.valid = in_bounds(layer_rel < p.n_layers && node < sq.N && node < sq.nstride && node < kMaxNodes &&
+                                        qh < p.Hq,
+                                    p.status);
+            g.anc = g.valid ? sq.tree->anc[node] : 0ull;
+            g.dep = g.valid ? sq.tree->depth[node] : 0;
+            const size_t row = (((size_t)layer_rel * sq.nstride + node) * p.Hq + qh) * kD;
+            g.q = sq.q + row;
+            g.out = sq.out + row;
+            return g;
+        };
+        // The segment's info and its Q rows, each row in its thread's TMEM lane as
+        // kD / 2 columns of bf16 pairs (the A operand of QK^T); zeros for padding rows
+        auto stage = [&](const Seg &g, int sg) {
+            SegInfo &si = s_info[sg & 1];
+            const uint32_t col = lane_addr + kColQ + (sg & 1) * (kD / 2);
+            const uint4 *src = reinterpret_cast<const uint4 *>(g.q);
+            if (!p.rope_tab) {
+                // the whole row (2 kD bytes) in flight at once, then kD / 32 TMEM stores
+                uint4 qv[kD / 8];
+#pragma unroll
+                for (int i = 0; i < kD / 8; ++i)
+                    qv[i] = g.valid ? src[i] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (int qc = 0; qc < kD / 32; ++qc) {
+                    uint32_t w[16];
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) {
+                        const uint4 v = qv[qc * 4 + ch];
+                        w[4 * ch] = v.x;
+                        w[4 * ch + 1] = v.y;
+                        w[4 * ch + 2] = v.z;
+                        w[4 * ch + 3] = v.w;
+                    }
+                    tmem_st_32x32b_x16(col + qc * 16, w);
+                }
+            } else {
+                // pre-rotary query: element i pairs with i + kD / 2, rotated at position
+                // L + depth(node) with the sequence's (cos, sin) table
+                constexpr int kHalf = kD / 64;  // 32-element chunks per half row
+                const float2 *tab = p.rope_tab + (size_t)g.b * kRopeTableEntries + (size_t)g.dep * kRopeMaxHalf;
 #pragma unroll 1
-                for (int c0 = 0; c0 < kD; c0 += 32) {
-                    uint32_t r[32];
+                for (int qc = 0; qc < kHalf; ++qc) {
+                    uint32_t wl[16], wh[16];
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) {
+                        const uint4 lo = g.valid ? src[qc * 4 + ch] : make_uint4(0, 0, 0, 0);
+                        const uint4 hi = g.valid ? src[(qc + kHalf) * 4 + ch] : make_uint4(0, 0, 0, 0);
+                        const uint32_t lw[4] = {lo.x, lo.y, lo.z, lo.w}, hw[4] = {hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int i0 = 32 * qc + 8 * ch + 2 * e;
+                            const float2 c0 = tab[i0], c1 = tab[i0 + 1];
+                            const float a0 = __uint_as_float(lw[e] << 16), a1 = __uint_as_float(lw[e] & 0xffff0000u);
+                            const float b0 = __uint_as_float(hw[e] << 16), b1 = __uint_as_float(hw[e] & 0xffff0000u);
+                            wl[4 * ch + e] = pack_bf16x2(a0 * c0.x - b0 * c0.y, a1 * c1.x - b1 * c1.y);
+                            wh[4 * ch + e] = pack_bf16x2(b0 * c0.x + a0 * c0.y, b1 * c1.x + a1 * c1.y);
+                        }
+                    }
+                    tmem_st_32x32b_x16(col + qc * 16, wl);
+                    tmem_st_32x32b_x16(col + (qc + kHalf) * 16, wh);
+                }
+            }
+            si.anc[rloc] = g.anc;
+            // every warp writes the same words, so that each softmax warp's wait covers them
+            if (lane == 0) {
+                si.n = g.n;
+                si.key0 = g.j0 * kBN;
+                si.L = g.L;
+            }
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&q_full[sg & 1]);
+        };
+        long long t = t0;
+        if (t < t1) {
+            Seg cur = describe(t);
+            stage(cur, 0);
+            t += cur.n;
+            Seg nxt{};
+            bool has_next = t < t1;
+            if (has_next) {
+                nxt = describe(t);
+                stage(nxt, 1);
+                t += nxt.n;
+            }
+            long long it = 0;
+            for (int sg = 0;; ++sg) {
+                it += cur.n;
+                // the segment after the next: its query rows are asked for in L2 now, staged below
+                Seg fut{};
+                const bool has_fut = t < t1;
+                if (has_fut) {
+                    fut = describe(t);
+                    t += fut.n;
+                    if (fut.valid) {
+#pragma unroll
+                        for (int off = 0; off < 2 * kD; off += 128)
+                            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(fut.q) + off));
+                    }
+                }
+                const long long last = it - 1;
+                if (!mbar_wait_bounded(&ml_full[sg & 1], (uint32_t)(sg >> 1) & 1u, &abort_flag, p.status))
+                    break;
+                const float m_ref = s_info[sg & 1].m[rloc], l = s_info[sg & 1].l[rloc];
+                if (!mbar_wait_bounded(&pv_done[last & 1], (uint32_t)(last >> 1) & 1u, &abort_flag, p.status))
+                    break;
+                tc_fence_after();
+                const bool whole = cur.n == cur.T;
+                const bool write = cur.valid && (whole || in_bounds(c < p.P && rloc < 128, p.status));
+                const float inv = 1.f / l;
+                uint4 *dst = reinterpret_cast<uint4 *>(cur.out);
+                // a partial (O, m, l) goes to the CTA's slot; k1_merge_split finishes the unit
+                float *slot = p.part + ((size_t)c * 2 + (cur.first ? 0 : 1)) * kSlot;
+                float4 *pdst = reinterpret_cast<float4 *>(slot + rloc * kD);
+#pragma unroll
+                for (int c0 = 0; c0 < kD; c0 += 64) {
+                    uint32_t r[64];
                     tmem_ld_32x32b_x32(lane_addr + kColO + c0, r);
+                    tmem_ld_32x32b_x32(lane_addr + kColO + c0 + 32, r + 32);
                     tmem_ld_wait();
-                    if (!g.valid)
+                    if (c0 + 64 == kD) {
+                        // the whole row is read: the next segment's P V may overwrite O
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0)
+                            mbar_arrive(&o_free[sg & 1]);
+                    }
+                    if (!write)
                         continue;
                     if (whole) {
 #pragma unroll
-                        for (int ch = 0; ch < 4; ++ch) {
+                        for (int ch = 0; ch < 8; ++ch) {
                             uint4 v;
                             v.x = pack_bf16x2(__uint_as_float(r[8 * ch + 0]) * inv, __uint_as_float(r[8 * ch + 1]) * inv);
                             v.y = pack_bf16x2(__uint_as_float(r[8 * ch + 2]) * inv, __uint_as_float(r[8 * ch + 3]) * inv);
@@ -649,25 +757,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                         }
                     } else {
 #pragma unroll
-                        for (int x = 0; x < 8; ++x)
+                        for (int x = 0; x < 16; ++x)
                             pdst[c0 / 4 + x] = make_float4(__uint_as_float(r[4 * x]), __uint_as_float(r[4 * x + 1]),
                                                            __uint_as_float(r[4 * x + 2]), __uint_as_float(r[4 * x + 3]));
                     }
                 }
+                if (!whole && write) {
+                    slot[128 * kD + rloc] = m_ref;
+                    slot[128 * kD + 128 + rloc] = l;
+                }
+                if (!has_next)
+                    break;
+                // every QK^T of the finished segment has been consumed: its Q buffer is free
+                if (has_fut)
+                    stage(fut, sg + 2);
+                cur = nxt;
+                nxt = fut;
+                has_next = has_fut;
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(&o_free);
-
-            if (!whole && g.valid) {
-                // partial (O in the slot already, m_ref, l); k1_merge_split finishes the unit
-                slot[128 * kD + rloc] = m_ref;
-                slot[128 * kD + 128 + rloc] = l;
-            }
-            if (!has_next)
-                break;
-            g = nx;
         }
     }
 

@@ -115,6 +115,15 @@ def test_tree_attention_layer_subset(dev, bank):
     _run_attention(bank, dev, synth.bank_trees()[4], 200, 4, 4, 4, 128, seed=3, layer_begin=1, n_run=2)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("L", [0, 40, 130, 290])
+def test_tree_attention_many_short_units(dev, bank, L, d):
+    """Units of one to three key tiles, 640 of them (four to nine per CTA): the
+    double-buffered queries and unit records are reused every other unit, and
+    single-tile units put a unit boundary at every tile."""
+    _run_attention(bank, dev, synth.bank_trees()[2], L, 20, 32, 32, d, seed=L + d)
+
+
 def test_tree_attention_large_L_multilayer(dev, bank):
     _run_attention(bank, dev, synth.bank_trees()[-1], 5000, 3, 8, 8, 128, seed=4)
 
