@@ -11,7 +11,8 @@ import numpy as np
 import pytest
 
 import oracle
-from helpers import ATT_MAX, STAT_TOL, bits, check_attention, gap_filtered_hidden, make_case, to_dev
+from helpers import (ATT_MAX, STAT_TOL, abs_bits, bits, check_attention, check_attention_fuzz, gap_filtered_hidden,
+                     make_case, to_dev)
 from paper_2606_27550_gb300 import synth
 
 torch = pytest.importorskip("torch")
@@ -40,7 +41,8 @@ def _ws(dev, rows, d, V):
     return tv.make_workspace(tv.tb_workspace_size(rows, 1, 1, 1, d, V, 0), dev)
 
 
-def _run_attention(bank, dev, parent, L, n_layers, Hq, Hkv, d, seed, layer_begin=0, n_run=None, L_cap=None):
+def _run_attention(bank, dev, parent, L, n_layers, Hq, Hkv, d, seed, layer_begin=0, n_run=None, L_cap=None,
+                   derived=False):
     parent = np.asarray(parent, np.int32)
     N = len(parent)
     bid, order = bank.add(parent)
@@ -59,7 +61,12 @@ def _run_attention(bank, dev, parent, L, n_layers, Hq, Hkv, d, seed, layer_begin
     got = out.float().cpu().numpy()
     for li in range(n_run):
         ref = oracle.tree_attention(q[layer_begin + li], k[layer_begin + li], v[layer_begin + li], L, parent)
-        check_attention(got[li], ref, f"layer {layer_begin + li}")
+        if derived:  # short prefixes: the bound the bf16 roundings give, above 1e-2 for outputs past 2.4
+            ref_abs_v = oracle.tree_attention(q[layer_begin + li], k[layer_begin + li], abs_bits(v[layer_begin + li]),
+                                              L, parent)
+            check_attention_fuzz(got[li], ref, ref_abs_v, f"layer {layer_begin + li}")
+        else:
+            check_attention(got[li], ref, f"layer {layer_begin + li}")
     # the workspace counters are back at zero: a second call gives the same bytes
     out2 = torch.empty_like(out)
     tv.tree_attention(bank, bid, kv, qd, out2, ws, layer_begin, n_run)
@@ -121,7 +128,7 @@ def test_tree_attention_many_short_units(dev, bank, L, d):
     """Units of one to three key tiles, 640 of them (four to nine per CTA): the
     double-buffered queries and unit records are reused every other unit, and
     single-tile units put a unit boundary at every tile."""
-    _run_attention(bank, dev, synth.bank_trees()[2], L, 20, 32, 32, d, seed=L + d)
+    _run_attention(bank, dev, synth.bank_trees()[2], L, 20, 32, 32, d, seed=L + d, derived=True)
 
 
 def test_tree_attention_large_L_multilayer(dev, bank):
