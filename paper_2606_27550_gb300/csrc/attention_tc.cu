@@ -9,7 +9,9 @@
 // (k1_merge_split, one warp per query row) combines them by log-sum-exp after
 // the first one has finished (in a verification step, beside the acceptance
 // kernel at the end of the step: nothing in the step reads the attention
-// output):
+// output).  A call of its own on a small problem (one layer of a model) gives
+// each unit to a cluster of CTAs instead, which combine their (O, m, l) through
+// shared memory at the end: no partials in memory and no second kernel.
 //
 //   S   = Q K^T   tcgen05.mma kind::f16, M = 128 query rows, N = 128 keys,
 //                 K = kD = head_dim; Q (bf16) is the TMEM A operand, the K
@@ -56,6 +58,8 @@
 // the softmax).
 #include <string.h>
 
+#include <atomic>
+
 #include "kernels.cuh"
 
 namespace tv {
@@ -85,6 +89,7 @@ constexpr int slot_floats(int d)
 // softmax has read S_b into registers; Q (bf16 pairs) is the A operand of QK^T.
 constexpr uint32_t kColS0 = 0, kColS1 = 128, kColP0 = 0, kColP1 = 128, kColO = 256, kColQ = 384;
 constexpr float kRescaleLog2 = 8.f;  // rescale O only when the row max grows by more than 2^8
+constexpr int kMaxCluster = 8;          // CTAs that may share a unit (the portable cluster size)
 constexpr int kSmCols = 32;          // columns of S a softmax thread holds at a time (64: the same time, twice the code)
 constexpr int kWholeUnitMaxTiles = 6;  // see attn_tc_plan
 
@@ -117,6 +122,7 @@ struct TcParams {
     int n_rungs, n_layers, L_cap;
     int max_rows;  // query rows of the largest row block (the split merge's grid)
     int d;         // head_dim: the kernels' kD (host side: picks the instantiation)
+    int cluster;   // > 1: a cluster of that many CTAs shares each unit (one sequence; see attn_tc_clusters)
     // rotary embedding (null: the queries are already rotated): per sequence a
     // table of (cos, sin) at position L + depth for every pair of head elements
     const float2 *rope_tab;
@@ -238,12 +244,37 @@ struct SegInfo {
     float m[128], l[128];      // written back by the softmax: reference maximum (log2 units) and sum of each row
 };
 
-template <int kD, bool kBatched>
+// Loads from the shared memory of any CTA of the cluster.
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(addr)
+                 : "memory");
+    return v;
+}
+
+// kCluster: the p.cluster CTAs of a cluster share one unit's key tiles, leave
+// their (O, m, l) in shared memory and combine them there (log-sum-exp, in rank
+// order), every CTA a share of the rows: no partials in global memory and no
+// second kernel.  For problems small enough that all their clusters run at
+// once (attn_tc_clusters).
+template <int kD, bool kBatched, bool kCluster>
 __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __grid_constant__ TcParams p)
 {
     static_assert(kD == 64 || kD == 128, "head_dim 64 or 128");
     constexpr int kTile = tile_bytes(kD);
     constexpr int kSlot = slot_floats(kD);
+    constexpr int kClusterLd = kD + 4;  // row stride of O in shared memory (floats): conflict-free row writes
+    static_assert(!(kCluster && kBatched), "clusters: one sequence");
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
     __shared__ __align__(8) uint64_t s_full[2], p_full[2], pv_done[2];
@@ -302,9 +333,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         seqs = &s_seq;
         total = s_total;
     }
-    const int P = tc_split_ctas(p, total);
-    const long long t0 = c < P ? tc_seg_begin(total, P, c) : total;
-    const long long t1 = c < P ? tc_seg_begin(total, P, c + 1) : total;
+    long long t0, t1;
+    if constexpr (kCluster) {
+        // every rank has a tile: the host takes no more CTAs than tiles
+        const int T = seqs[0].T, rank = c % p.cluster;
+        const long long first = (long long)(c / p.cluster) * T;
+        t0 = first + (long long)T * rank / p.cluster;
+        t1 = first + (long long)T * (rank + 1) / p.cluster;
+    } else {
+        const int P = tc_split_ctas(p, total);
+        t0 = c < P ? tc_seg_begin(total, P, c) : total;
+        t1 = c < P ? tc_seg_begin(total, P, c + 1) : total;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -723,13 +763,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                 if (!mbar_wait_bounded(&pv_done[last & 1], (uint32_t)(last >> 1) & 1u, &abort_flag, p.status))
                     break;
                 tc_fence_after();
-                const bool whole = cur.n == cur.T;
+                const bool whole = !kCluster && cur.n == cur.T;
                 const bool write = cur.valid && (whole || in_bounds(c < p.P && rloc < 128, p.status));
                 const float inv = 1.f / l;
                 uint4 *dst = reinterpret_cast<uint4 *>(cur.out);
                 // a partial (O, m, l) goes to the CTA's slot; k1_merge_split finishes the unit
                 float *slot = p.part + ((size_t)c * 2 + (cur.first ? 0 : 1)) * kSlot;
                 float4 *pdst = reinterpret_cast<float4 *>(slot + rloc * kD);
+                if constexpr (kCluster)  // the rings are drained: every tile has been consumed
+                    pdst = reinterpret_cast<float4 *>(smem + (size_t)rloc * kClusterLd * 4);
 #pragma unroll
                 for (int c0 = 0; c0 < kD; c0 += 64) {
                     uint32_t r[64];
@@ -762,7 +804,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                                                            __uint_as_float(r[4 * x + 2]), __uint_as_float(r[4 * x + 3]));
                     }
                 }
-                if (!whole && write) {
+                if (!kCluster && !whole && write) {
                     slot[128 * kD + rloc] = m_ref;
                     slot[128 * kD + 128 + rloc] = l;
                 }
@@ -786,6 +828,67 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             mbar_wait_drain(&drain_bar, 0);
         __syncwarp();
         tmem_dealloc(tmem, 512);
+    }
+    if constexpr (kCluster) {
+        cluster_barrier();  // every CTA's (O, m, l) is in its shared memory
+        const TcSeq &sq = seqs[0];
+        const int n_cta = p.cluster, rank = c % n_cta, u = c / n_cta;
+        const int rb = u % sq.row_blocks;
+        const int head = (u / sq.row_blocks) % p.Hkv;
+        const int layer_rel = u / (sq.row_blocks * p.Hkv);
+        const int rows_here = abort_flag ? 0 : min(128, sq.rows - rb * 128);
+        // this CTA's rows are rank, rank + n_cta, ..: at most 64, so that their weights
+        // (one per row and rank, then 1 / l) fit the unused second unit record
+        const int n_rows = (rows_here - rank + n_cta - 1) / n_cta;
+        float *s_w = reinterpret_cast<float *>(s_info[1].anc), *s_inv = s_info[1].l;
+        if ((int)threadIdx.x < n_rows) {
+            const int r = threadIdx.x * n_cta + rank;
+            const uint32_t m_addr = smem_u32(&s_info[0].m[r]), l_addr = smem_u32(&s_info[0].l[r]);
+            float m[kMaxCluster], l[kMaxCluster], M = -INFINITY, lsum = 0.f;
+#pragma unroll
+            for (int k = 0; k < kMaxCluster; ++k) {
+                m[k] = k < n_cta ? ld_cluster_f32(cluster_map(m_addr, k)) : -INFINITY;
+                l[k] = k < n_cta ? ld_cluster_f32(cluster_map(l_addr, k)) : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < kMaxCluster; ++k)
+                M = fmaxf(M, m[k]);
+#pragma unroll
+            for (int k = 0; k < kMaxCluster; ++k) {
+                const float w = m[k] == -INFINITY ? 0.f : ex2_approx(m[k] - M);
+                lsum += w * l[k];
+                if (k < n_cta)
+                    s_w[threadIdx.x * n_cta + k] = w;
+            }
+            s_inv[threadIdx.x] = 1.f / lsum;
+        }
+        __syncthreads();
+        constexpr int kVec = kD / 4;  // 4-column pieces of a row
+        const uint32_t o_base = smem_u32(smem);
+        for (int x = threadIdx.x; x < n_rows * kVec; x += kTcThreads) {
+            const int i = x / kVec, col = 4 * (x % kVec), r = i * n_cta + rank;
+            const uint32_t o_addr = o_base + (uint32_t)(r * kClusterLd + col) * 4;
+            float4 v[kMaxCluster];
+#pragma unroll
+            for (int k = 0; k < kMaxCluster; ++k)
+                if (k < n_cta)
+                    v[k] = ld_cluster_f32x4(cluster_map(o_addr, k));
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < kMaxCluster; ++k)
+                if (k < n_cta) {
+                    const float w = s_w[i * n_cta + k];
+                    acc.x += w * v[k].x, acc.y += w * v[k].y, acc.z += w * v[k].z, acc.w += w * v[k].w;
+                }
+            const float inv = s_inv[i];
+            const int grow = rb * 128 + r;
+            const int node = grow / p.group;
+            const int qh = head * p.group + grow % p.group;
+            if (in_bounds(layer_rel < p.n_layers && node < sq.nstride && qh < p.Hq, p.status))
+                *reinterpret_cast<uint2 *>(sq.out + (((size_t)layer_rel * sq.nstride + node) * p.Hq + qh) * kD + col) =
+                    make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
+        }
+        cluster_barrier();  // no CTA leaves while another reads its shared memory
     }
 }
 
@@ -967,7 +1070,7 @@ static cudaError_t merge_launch_d(const TcParams &p, bool batched, cudaStream_t 
 // has work).  Scheduled mode plans on the device: assumed so.
 static bool any_split(const TcParams &p)
 {
-    if (p.P <= 1)
+    if (p.P <= 1 || p.cluster > 1)
         return false;
     if (p.sched)
         return true;
@@ -992,21 +1095,61 @@ static cudaError_t merge_launch(const TcParams &p, bool batched, cudaStream_t st
 }
 
 // The attention kernel for p.d, one CTA per SM (each holds 512 TMEM columns).
-template <int kD, bool kBatched>
+static size_t attn_smem(int d)
+{
+    return (size_t)(kKStages + kVStages) * tile_bytes(d) + 1024;
+}
+
+template <int kD, bool kBatched, bool kCluster>
 static cudaError_t attn_kernel_launch_d(const TcParams &p, cudaStream_t stream, bool pdl)
 {
     cudaError_t e;
-    if ((e = allow_max_smem((const void *)k1_tree_attention_tc<kD, kBatched>)) != cudaSuccess)
+    if ((e = allow_max_smem((const void *)k1_tree_attention_tc<kD, kBatched, kCluster>)) != cudaSuccess)
         return e;
-    const size_t smem = (size_t)(kKStages + kVStages) * tile_bytes(kD) + 1024;
-    return launch_kernel(k1_tree_attention_tc<kD, kBatched>, dim3(p.P), dim3(kTcThreads), smem, stream, pdl, p);
+    return launch_kernel_cluster(k1_tree_attention_tc<kD, kBatched, kCluster>, dim3(p.P), dim3(kTcThreads),
+                                 attn_smem(kD), stream, pdl, kCluster ? p.cluster : 1, p);
 }
 
 static cudaError_t attn_kernel_launch(const TcParams &p, bool batched, cudaStream_t stream, bool pdl)
 {
+    if (p.cluster > 1)
+        return p.d == 64 ? attn_kernel_launch_d<64, false, true>(p, stream, pdl)
+                         : attn_kernel_launch_d<128, false, true>(p, stream, pdl);
     if (p.d == 64)
-        return batched ? attn_kernel_launch_d<64, true>(p, stream, pdl) : attn_kernel_launch_d<64, false>(p, stream, pdl);
-    return batched ? attn_kernel_launch_d<128, true>(p, stream, pdl) : attn_kernel_launch_d<128, false>(p, stream, pdl);
+        return batched ? attn_kernel_launch_d<64, true, false>(p, stream, pdl)
+                       : attn_kernel_launch_d<64, false, false>(p, stream, pdl);
+    return batched ? attn_kernel_launch_d<128, true, false>(p, stream, pdl)
+                   : attn_kernel_launch_d<128, false, false>(p, stream, pdl);
+}
+
+// Clusters of `size` CTAs of the attention kernel that can be resident at once
+// on the current device (cached; 0 if none).
+template <int kD>
+static int attn_max_clusters(int size)
+{
+    static std::atomic<int> cache[kMaxCluster + 1];  // 0: not queried yet, else clusters + 1
+    const int v = cache[size].load(std::memory_order_relaxed);
+    if (v > 0)
+        return v - 1;
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = attn_smem(kD);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (allow_max_smem((const void *)k1_tree_attention_tc<kD, false, true>) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k1_tree_attention_tc<kD, false, true>, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        n = 0;
+    }
+    cache[size].store(n + 1, std::memory_order_relaxed);
+    return n;
 }
 
 // The attention launch's parameters, kept for a split-unit merge enqueued later.
@@ -1045,6 +1188,37 @@ AttnPlan attn_tc_plan(int L, int N, int Hq, int Hkv, int n_layers, int n_sm)
     return pl;
 }
 
+// CTAs per unit of a stand-alone attention call of one sequence (1: no
+// clusters): as many as fit the SMs with every unit's cluster resident at once;
+// units of a few tiles run whole (32 q / 8 kv heads x 128, 64 nodes at 100 and
+// 400 keys: 8.5 and 10.4 us whole, 10.9 and 11.1 in clusters).
+// The clusters save the partials' round trip through memory and the merge
+// launch, but leave SMs idle when the units do not divide them.  At head_dim
+// 128 three quarters of the SMs still saturate HBM, and the clusters win at
+// any length.  Otherwise they win while the longest CTA has at most about
+// `size` tiles more than an even split over all SMs would give it.  Measured on
+// GB300, one layer, clusters / even split: 32 kv heads x 128, 26 nodes at 700,
+// 1500, 24000 keys 11.0 / 13.8, 12.7 / 16.0, 64.1 / 67.9 us; 8 heads x 128 at
+// 12000 and 24000 keys 20.9 / 21.6 and 33.1 / 29.2; 64 heads x 64 at 3000 and
+// 6000 keys 20.7 / 21.9 and 32.6 / 32.2.
+static int attn_tc_clusters(const AttnPlan &pl, int d, int n_sm)
+{
+    if (pl.total <= n_sm && (pl.T <= 2 || (pl.T <= 4 && pl.rows > 64)))
+        return 1;
+    int size = n_sm / pl.n_units;
+    size = size < kMaxCluster ? size : kMaxCluster;
+    size = size < pl.T ? size : pl.T;
+    for (; size > 1; --size)
+        if (pl.n_units <= (d == 64 ? attn_max_clusters<64>(size) : attn_max_clusters<128>(size)))
+            break;
+    if (size <= 1)
+        return 1;
+    if (d == 128 && 4 * pl.n_units * size >= 3 * n_sm)
+        return size;
+    const long long longest = (pl.T + size - 1) / size, even = pl.total / n_sm;
+    return longest - even <= size ? size : 1;
+}
+
 size_t attn_tc_slot_floats(int d)
 {
     return (size_t)slot_floats(d);
@@ -1060,7 +1234,7 @@ int attn_tc_units(const AttnSeq *seqs, int n_seq, int Hq, int Hkv, int n_layers)
 
 cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin, int n_layers, int Hq, float *part,
                                  int *status, int n_sm, cudaStream_t stream, const char **err,
-                                 const float2 *rope_tab, AttnMerge *merge_later)
+                                 const float2 *rope_tab, AttnMerge *merge_later, bool alone)
 {
     if (n_seq < 1 || n_seq > kMaxSeqPerLaunch) {
         *err = "too many sequences for one attention launch";
@@ -1119,23 +1293,34 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     p.rope_tab = rope_tab;
     p.max_rows = max_rows;
     const bool batched = n_seq > 1;
+    // a call of its own, not part of a step: clusters share the units of a small problem
+    p.cluster = 1;
+    if (n_seq == 1 && alone) {
+        const AttnPlan pl = attn_tc_plan(seqs[0].kv->L, seqs[0].N, Hq, Hkv, n_layers, n_sm);
+        p.cluster = attn_tc_clusters(pl, d, n_sm);
+        if (p.cluster > 1)
+            p.P = pl.n_units * p.cluster;
+    }
     cudaError_t e;
-    // A grid that takes every SM starts when the stream's previous work is done,
-    // so that all its CTAs start together (its work split is static); a grid
-    // capped beside a longer LM head (merge_later->pdl_launch) is launched as a
-    // programmatic dependent and its CTAs wait on SMs that are free already.
-    const bool pdl = merge_later && merge_later->pdl_launch;
+    // In a step, a grid that takes every SM starts when the stream's previous
+    // work is done, so that all its CTAs start together (its work split is
+    // static) and before the LM head's; a grid capped beside a longer LM head
+    // (merge_later) is launched as a programmatic dependent and its CTAs wait on
+    // SMs that are free already.  A call of its own is launched as a programmatic
+    // dependent too, and so is its merge: only the set-up overlaps what runs
+    // before, each kernel waiting for the one it follows.
+    const bool pdl = alone || merge_later;
     if ((e = attn_kernel_launch(p, batched, stream, pdl)) != cudaSuccess)
         return e;
     if (merge_later) {
         stash_merge(p, batched, merge_later);
         return cudaSuccess;
     }
-    // A plain dependent of the attention: launched as a programmatic one, its
-    // CTAs would take the SMs that attention CTAs release and hold them until
+    // In a step, a plain dependent of the attention: launched as a programmatic
+    // one, its CTAs would take the SMs that attention CTAs release and hold them until
     // the whole grid is done, away from an LM head beside it on another stream
     // (measured on GB300: the ragged batch's step 20 us longer).
-    return merge_launch(p, batched, stream, false, false);
+    return merge_launch(p, batched, stream, alone, false);
 }
 
 cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *status, int n_sm,
@@ -1195,11 +1380,12 @@ cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *
 
 cudaError_t attn_tc_launch(const tb_kv *kv, const TreeDesc *d_tree, int N, int layer_begin, int n_layers,
                            const void *q, int Hq, void *out, float *part, int *status, int n_sm,
-                           cudaStream_t stream, const char **err, const float2 *rope_tab, AttnMerge *merge_later)
+                           cudaStream_t stream, const char **err, const float2 *rope_tab, AttnMerge *merge_later,
+                           bool alone)
 {
     AttnSeq one{kv, d_tree, N, q, out};
     return attn_tc_launch_batch(&one, 1, layer_begin, n_layers, Hq, part, status, n_sm, stream, err, rope_tab,
-                                merge_later);
+                                merge_later, alone);
 }
 
 cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream, bool after_step)

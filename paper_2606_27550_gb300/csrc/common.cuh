@@ -219,6 +219,14 @@ __device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank)
     return r;
 }
 
+// As cluster_addr, from a shared::cta address.
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
 // As mbar_try_wait, acquiring at cluster scope: for a barrier that another CTA
 // of the cluster arrives on (release at cluster scope) after storing data
 // into this CTA's shared memory.

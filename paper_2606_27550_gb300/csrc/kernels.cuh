@@ -139,7 +139,6 @@ int attn_tc_units(const AttnSeq *seqs, int n_seq, int Hq, int Hkv, int n_layers)
 // stream's previous kernel: after the LM head, or (after_step) after the
 // acceptance kernel, beside which it runs.
 struct AttnMerge {
-    bool pdl_launch;  // set by the caller: launch the attention itself as a programmatic dependent
     bool pending;
     bool batched;
     alignas(64) unsigned char params[8192];
@@ -147,10 +146,14 @@ struct AttnMerge {
 cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream, bool after_step);
 // rope_tab: null, or the (cos, sin) tables of rope.cu: the queries are then
 // pre-rotary and are rotated at L + depth while they are staged
-// merge_later: the split-unit merge is not enqueued but kept there
+// merge_later: the split-unit merge is not enqueued but kept there, and the
+// attention is launched as a programmatic dependent; alone: a call of its own,
+// not part of a verification step (clusters may share its units, and its
+// launches are programmatic dependents)
 cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin, int n_layers, int Hq, float *part,
                                  int *status, int n_sm, cudaStream_t stream, const char **err,
-                                 const float2 *rope_tab = nullptr, AttnMerge *merge_later = nullptr);
+                                 const float2 *rope_tab = nullptr, AttnMerge *merge_later = nullptr,
+                                 bool alone = false);
 bool attn_tc_supported(int d);
 AttnPlan attn_tc_plan(int L, int N, int Hq, int Hkv, int n_layers, int n_sm);
 size_t attn_tc_slot_floats(int d);  // floats per partial slot (two slots per CTA)
@@ -170,7 +173,7 @@ cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *
 cudaError_t attn_tc_launch(const tb_kv *kv, const TreeDesc *d_tree, int N, int layer_begin, int n_layers,
                            const void *q, int Hq, void *out, float *part, int *status, int n_sm,
                            cudaStream_t stream, const char **err, const float2 *rope_tab = nullptr,
-                           AttnMerge *merge_later = nullptr);
+                           AttnMerge *merge_later = nullptr, bool alone = false);
 
 // acceptance + compaction (accept.cu)
 struct AcceptParams {

@@ -7,18 +7,21 @@
 // positions; the prefix keys were rotated when they entered the cache.
 //
 //   k0_rope_tree_k  one launch: a CTA per (tree node, 64 or 128 (layer, kv
-//                   head) rows of it).  Every thread first loads its 8 pairs
-//                   of two rows (16 bytes from each half: the long-context
-//                   step's 1024 CTAs are about one wave), then 64 threads form the
-//                   (cos, sin) of (L + depth) * theta_i for the node's depth
-//                   while the loads are in flight: the angle is formed and
-//                   reduced to [-pi, pi] in double (positions reach 10^4-10^5
-//                   rad), sin and cos are taken in float.  The rotated pairs
-//                   are written back to the bf16 cache in place.  The first
-//                   node of each depth (canonical order: depths do not
+//                   head) rows of it).  64 threads form the (cos, sin) of
+//                   (L + depth) * theta_i for the node's depth: the angle is
+//                   formed and reduced to [-pi, pi] in double (positions reach
+//                   10^4-10^5 rad), sin and cos are taken in float.  That part
+//                   depends on the topology and L only and runs before the wait
+//                   for the stream's previous kernel (the launch is a
+//                   programmatic dependent of it).  Then every thread loads its
+//                   8 pairs of two rows (16 bytes from each half: the
+//                   long-context step's 1024 CTAs are about one wave), rotates
+//                   them and writes them back to the bf16 cache in place.  The
+//                   first node of each depth (canonical order: depths do not
 //                   decrease with the id) also writes its table row to the
 //                   workspace for the query rotation.  head_dim 64 or 128
-//                   (template kD: kD / 16 threads per row).
+//                   (template kD: kD / 16 threads per row).  What bounds it is
+//                   launch and load latency (16.8 MB at 32 layers).
 // The queries are rotated inside the attention kernel as they are staged
 // into tensor memory (attention_tc.cu), with the same table.
 #include <cuda_bf16.h>
@@ -46,6 +49,7 @@ __global__ void __launch_bounds__(kRopeThreads) k0_rope_tree_k(const __grid_cons
     const TreeDesc *tree = sq.tree;
     int L = sq.L;
     if (p.sched) {
+        pdl_wait();
         const int rung = p.sched[0], Ls = p.sched[1];
         if (rung < 0 || rung >= p.n_rungs || Ls < 0 || Ls + p.rung_tree[rung]->n > p.L_cap)
             return;  // no work this step (the acceptance kernel reports it)
@@ -53,10 +57,23 @@ __global__ void __launch_bounds__(kRopeThreads) k0_rope_tree_k(const __grid_cons
         L = Ls;
     }
     const int j = blockIdx.x;
-    if (j >= tree->n)
-        return;
-    const int dep = tree->depth[j];
     constexpr int kHalf = kD / 2;  // pairs of a row
+    const bool here = j < tree->n;
+    const int dep = here ? tree->depth[j] : 0;
+    // The angles depend on the topology and L only: they are formed before the
+    // wait for the stream's previous work.
+    float2 cn = make_float2(1.f, 0.f);
+    if (here && threadIdx.x < kHalf) {
+        constexpr double kTwoPi = 6.283185307179586476925286766559;
+        const double a = (double)(L + dep) * p.inv_freq[threadIdx.x];
+        const double red = a - kTwoPi * rint(a * (1.0 / kTwoPi));
+        sincosf((float)red, &cn.y, &cn.x);
+        cs[threadIdx.x] = cn;
+    }
+    pdl_wait();
+    pdl_trigger();  // the attention may be launched: it waits for this grid to complete
+    if (!here)
+        return;
     const int ch = (threadIdx.x % kTpr) * 8;
     __nv_bfloat16 *row[kRopeRowsPerThread];
     uint4 lo[kRopeRowsPerThread], hi[kRopeRowsPerThread];  // elements [ch, ch + 8) and [kHalf + ch, kHalf + ch + 8)
@@ -73,17 +90,8 @@ __global__ void __launch_bounds__(kRopeThreads) k0_rope_tree_k(const __grid_cons
             hi[k] = *reinterpret_cast<const uint4 *>(row[k] + kHalf + ch);
         }
     }
-    if (threadIdx.x < kHalf) {
-        const int i = threadIdx.x;
-        constexpr double kTwoPi = 6.283185307179586476925286766559;
-        const double a = (double)(L + dep) * p.inv_freq[i];
-        const double red = a - kTwoPi * rint(a * (1.0 / kTwoPi));
-        float sn, cn;
-        sincosf((float)red, &sn, &cn);
-        cs[i] = make_float2(cn, sn);
-        if (blockIdx.y == 0 && (j == 0 || tree->depth[j - 1] != dep))
-            p.table[(size_t)blockIdx.z * kRopeTableEntries + dep * kRopeMaxHalf + i] = make_float2(cn, sn);
-    }
+    if (threadIdx.x < kHalf && blockIdx.y == 0 && (j == 0 || tree->depth[j - 1] != dep))
+        p.table[(size_t)blockIdx.z * kRopeTableEntries + dep * kRopeMaxHalf + threadIdx.x] = cn;
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kRopeRowsPerThread; ++k) {
@@ -116,13 +124,8 @@ cudaError_t rope_launch(const RopeParams &p, int n_seq, int max_nodes, int n_lay
     const int per_cta = rope_rows_per_cta(p.d);
     const dim3 grid(max_nodes, (n_rows + per_cta - 1) / per_cta, n_seq);
     if (p.d == 64)
-        k0_rope_tree_k<64><<<grid, kRopeThreads, 0, stream>>>(p, n_rows);
-    else
-        k0_rope_tree_k<128><<<grid, kRopeThreads, 0, stream>>>(p, n_rows);
-    const cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess)
-        count_launch();
-    return e;
+        return launch_kernel(k0_rope_tree_k<64>, grid, dim3(kRopeThreads), 0, stream, true, p, n_rows);
+    return launch_kernel(k0_rope_tree_k<128>, grid, dim3(kRopeThreads), 0, stream, true, p, n_rows);
 }
 
 TB_BOUNDS_COUNTER(bounds_violations_rope)

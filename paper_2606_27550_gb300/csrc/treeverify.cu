@@ -272,11 +272,10 @@ class StepStreams {
             lk_ = std::unique_lock<std::mutex>(bank_->fork_mu);
     }
     bool chain() const { return chain_; }
-    // the split-unit merge is kept for finish() in the chain, enqueued right
-    // after the attention otherwise
+    // the split-unit merge is kept for merge() in the chain (whose attention is
+    // a programmatic dependent of the kernel before), enqueued right after the
+    // attention otherwise
     AttnMerge *merge_later() { return chain_ ? &merge_ : nullptr; }
-    // an attention grid capped beside a longer LM head is itself a programmatic dependent
-    void attention_pdl(bool pdl) { merge_.pdl_launch = chain_ && pdl; }
     // called between the rotary launch and the attention launch
     tb_status before_attention(const char *fn)
     {
@@ -749,7 +748,7 @@ static tb_status attn_enqueue(const AttnArgs &a, uint8_t *ws, size_t part_off, c
         attn_tc_launch(a.kv, a.bank->d_desc + a.bank_id, N, a.layer_begin, a.n_layers, a.q, a.Hq, a.out,
                        reinterpret_cast<float *>(ws + part_off), reinterpret_cast<int *>(ws),
                        a.max_ctas > 0 && a.max_ctas < nsm ? a.max_ctas : nsm, stream, &err,
-                       rope ? rope_table(ws) : nullptr, merge_later);
+                       rope ? rope_table(ws) : nullptr, merge_later, ss == nullptr);
     if (e == cudaErrorInvalidValue && err[0])
         return fail(TB_EINVAL, "%s: %s", fn, err);
     if (e != cudaSuccess)
@@ -1070,7 +1069,6 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
     a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
     // the structure of verify_step, with the walk between the LM head and the compaction
     StepStreams ss(bank, s, a.max_ctas > 0);
-    ss.attention_pdl(kv->rope_theta == 0.f);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, kPartBase + attn_bytes,
@@ -1151,7 +1149,6 @@ static tb_status verify_step_impl(const tb_bank *bank, int bank_id, const tb_kv 
     // the step's structure: see StepStreams
     a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
     StepStreams ss(bank, s, a.max_ctas > 0);
-    ss.attention_pdl(kv->rope_theta == 0.f);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, kPartBase + attn_bytes,

@@ -131,6 +131,21 @@ def test_tree_attention_many_short_units(dev, bank, L, d):
     _run_attention(bank, dev, synth.bank_trees()[2], L, 20, 32, 32, d, seed=L + d, derived=True)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("Hq,Hkv,tree,L", [
+    (64, 64, 5, 640), (40, 40, 5, 900), (32, 32, 5, 1500), (20, 20, 0, 1023),  # 2, 3, 4 and 7 CTAs a unit
+    (8, 8, 4, 400), (8, 8, 5, 1019),                      # 8; as many as the unit's 4 tiles, then an uneven split
+    (2, 2, 0, 3000), (32, 8, 7, 1100), (32, 4, 3, 2500),  # one query row; two row blocks; 64 rows
+    (8, 4, 7, 3), (16, 4, 7, 450), (32, 8, 5, 513),       # around the limit below which units run whole
+])
+def test_tree_attention_clusters(dev, bank, Hq, Hkv, tree, L, d):
+    """One layer alone: the CTAs of a cluster share a unit's key tiles and
+    combine their partials through shared memory, for every cluster size that
+    the SM count gives, uneven tile counts, a masked last tile that a rank holds
+    alone, and row counts from 1 to 256."""
+    _run_attention(bank, dev, synth.bank_trees()[tree], L, 1, Hq, Hkv, d, seed=L + d, derived=True)
+
+
 def test_tree_attention_large_L_multilayer(dev, bank):
     _run_attention(bank, dev, synth.bank_trees()[-1], 5000, 3, 8, 8, 128, seed=4)
 
