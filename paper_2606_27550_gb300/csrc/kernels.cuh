@@ -215,9 +215,10 @@ struct AcceptParams {
 cudaError_t accept_launch(const AcceptParams &p, int n_sm, cudaStream_t stream, bool pdl = false);
 cudaError_t accept_launch_batch(const AcceptParams *ps, int n, int n_sm, cudaStream_t stream, bool pdl = false);
 
-// speculative sampling on the tree (sample.cu): one CTA walks the tree
+// speculative sampling on the tree (sample.cu)
 struct SampleParams {
     const TreeDesc *tree;
+    int n;                // its nodes
     const int32_t *draft;
     const float *logits;  // [N][V]
     const float *logz_t;  // [N]: ln sum_v e^(z_v / T)

@@ -22,25 +22,31 @@
 // every later child is rejected and the draw returns the last token, as the
 // sequential update does.
 //
-// k4_spec_sample_cluster (vocabularies up to 131072): a cluster of 8 CTAs x
-// 1024 threads, each thread holding E consecutive vocabulary entries of p_u
-// and q_u in registers (loaded once per node), so a rejection costs a block
-// reduction and one cluster barrier.  What the decisions read -- for every
-// non-root node c with parent u, p_u(t_c), q_u(t_c) and unif[c] -- depends on
-// the tree and the drafts only, so every CTA gathers all of it at the start
-// (one round of dependent loads for the whole walk) and the slices of a node
-// are loaded only when a child of it is rejected or the draw happens there.
-// The control flow -- the children tried, the decisions, the number of
-// cluster barriers -- depends only on those values (the same read-only words,
-// turned into the same numbers by the same instructions in every CTA) and on
-// the cluster sums (the same eight CTA partials added in the same order
-// everywhere), so every CTA takes the same decisions and the same barriers
-// whatever the inputs hold.
+// k4_spec_sample_cluster (vocabularies up to 262144): a cluster of 8 or 16 CTAs
+// x 1024 threads, each thread holding E consecutive vocabulary entries of p_u
+// and q_u in registers (loaded once per node), so a rejection costs one cluster
+// barrier: every warp hands its sum to every CTA, and each warp adds all of
+// them.  What the decisions read -- for every non-root node c with parent u,
+// p_u(t_c), q_u(t_c) and unif[c] -- depends on the tree and the drafts only, so
+// every CTA gathers all of it at the start (one round of dependent loads for
+// the whole walk, beside the root's slices) and the slices of another node are
+// loaded only when a child of it is rejected or the draw happens there.  The
+// control flow -- the children tried, the decisions, the number of cluster
+// barriers -- depends only on those values (the same read-only words, turned
+// into the same numbers by the same instructions in every CTA) and on the
+// cluster sums (the same warp sums added in the same order everywhere), so
+// every CTA takes the same decisions and the same barriers whatever the inputs
+// hold.  Latency bounds it: the gather (two dependent loads), then one barrier
+// and two warp reductions (about 1.2 us) per rejection.  Measured on 64-node
+// walks: 5.8-8.4 us at V 32000 or less (7.0-9.6 with a block reduction in each
+// CTA before the exchange); 11-17 us at V 150004, where one CTA took 28-100.
 //
 // k4_spec_sample (larger vocabularies): one CTA of 1024 threads; the residual
 // is kept explicitly in the scratch row, one read-modify-write pass per
 // rejection.
 #include <math.h>
+
+#include <atomic>
 
 #include "kernels.cuh"
 
@@ -130,6 +136,8 @@ __global__ void __launch_bounds__(kSampleThreads) k4_spec_sample(const __grid_co
     __shared__ int s_par[kMaxNodes];
     __shared__ int s_draft[kMaxNodes];
     __shared__ int s_tok;
+    pdl_wait();
+    pdl_trigger();
     const TreeDesc *t = p.tree;
     const int n = t->n;
     const int tid = threadIdx.x;
@@ -245,68 +253,66 @@ __global__ void __launch_bounds__(kSampleThreads) k4_spec_sample(const __grid_co
 
 // ------------------------------------------------------------ cluster walk
 
-constexpr int kWalkCtas = 8;  // portable cluster size
 constexpr int kWalkThreads = kSampleThreads;
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
+constexpr int kWalkWarps = kWalkThreads / 32;
 
 // All threads of all CTAs of the cluster; orders shared and global memory at
 // cluster scope (writes before it are visible to every CTA after it).  The
 // non-.aligned form: the threads of a warp need not be converged here.
+__device__ __forceinline__ void cluster_arrive()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+
+__device__ __forceinline__ void cluster_wait()
+{
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 __device__ __forceinline__ void cluster_sync()
 {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
-// The address of the shared variable at p in the shared memory of CTA `rank`.
-__device__ __forceinline__ uint32_t dsmem(const void *p, uint32_t rank)
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v)
 {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-    return r;
-}
-
-__device__ __forceinline__ float ld_dsmem_f32(uint32_t a)
-{
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
 // Atomic minimum on a 32-bit shared variable of another CTA of the cluster
 // (ordered for the others by the next cluster barrier).
-__device__ __forceinline__ void red_min_dsmem_s32(uint32_t a, int v)
+__device__ __forceinline__ void red_min_cluster_s32(uint32_t a, int v)
 {
     asm volatile("red.relaxed.cluster.shared::cluster.min.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-// Sum of x over the cluster.  Every thread of every CTA gets the same bits:
-// the CTA partials are added in rank order by a butterfly, and a butterfly's
-// partners add the same two values (addition commutes exactly).
-__device__ float cluster_sum(float x, float *red, float *part_slot)
+// Hands this warp's value x to every CTA of the cluster: entry rank * 32 + warp
+// of each one's vals.  Readable after the next cluster barrier.
+template <int kCtas>
+__device__ __forceinline__ void cluster_publish(float x, uint32_t rank, float *vals)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane < kCtas)
+        st_cluster_f32(cluster_addr(vals + rank * kWalkWarps + warp, lane), x);
+}
+
+// Sum of x over the cluster.  Every warp of every CTA adds the same warp sums
+// in the same order (and a butterfly's partners add the same two values:
+// addition commutes exactly), so every thread gets the same bits.
+template <int kCtas>
+__device__ float cluster_sum(float x, uint32_t rank, float *vals)
+{
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1)
         x += __shfl_xor_sync(0xffffffffu, x, m);
-    if (lane == 0)
-        red[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        float t = red[lane];
-#pragma unroll
-        for (int m = 16; m >= 1; m >>= 1)
-            t += __shfl_xor_sync(0xffffffffu, t, m);
-        if (lane == 0)
-            *part_slot = t;
-    }
+    cluster_publish<kCtas>(x, rank, vals);
     cluster_sync();
-    float y = lane < kWalkCtas ? ld_dsmem_f32(dsmem(part_slot, lane)) : 0.f;
+    float y = 0.f;
+#pragma unroll
+    for (int r = 0; r < kCtas; ++r)
+        y += vals[r * kWalkWarps + lane];
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1)
         y += __shfl_xor_sync(0xffffffffu, y, m);
@@ -348,39 +354,42 @@ __device__ __forceinline__ void load_slice(const float *z, const float *q, int v
     }
 }
 
-template <int E>
-__global__ void __cluster_dims__(kWalkCtas, 1, 1) __launch_bounds__(kWalkThreads, 1)
-    k4_spec_sample_cluster(const __grid_constant__ SampleParams p)
+template <int E, int kCtas>
+__global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const __grid_constant__ SampleParams p)
 {
-    __shared__ float red[32];
-    __shared__ float s_part[2];             // this CTA's partial of the last two cluster sums
+    __shared__ __align__(16) float s_vals[2][kCtas * kWalkWarps];  // the cluster's warp sums of the last two exchanges
     __shared__ uint64_t l_kids[kMaxNodes];  // the children of each node (bitset)
+    __shared__ uint64_t l_anc[kMaxNodes];
     __shared__ int l_ok[kMaxNodes];         // per non-root node c with parent u: draft token in [0, V),
     __shared__ float l_pt[kMaxNodes];       // ... p_u(t_c), q_u(t_c) and the uniform deciding c
     __shared__ float l_qt[kMaxNodes], l_uf[kMaxNodes];
+    __shared__ float l_off[kMaxNodes];      // log2(e) logZ_u of each node
     __shared__ int s_tok;                   // rank 0: the drawn token (minimum over the claiming threads)
 
     constexpr float kLog2e = 1.4426950408889634f;
+    cluster_arrive();  // every CTA has started: waited for before the first remote access
     const float scale = p.inv_t * kLog2e;
-    const uint32_t rank = cluster_rank();
-    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t rank = cluster_ctarank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TreeDesc *t = p.tree;
-    const int n = t->n;
-    if (!in_bounds(n >= 1 && n <= kMaxNodes, const_cast<int *>(p.ws_status)))
-        return;  // the same tree in every CTA: the whole cluster returns before its first barrier
+    const int n = p.n;
     if (tid < kMaxNodes)
         l_kids[tid] = 0;
     if (tid == 0)
         s_tok = 0x7fffffff;
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    const bool vec = (p.V & 3) == 0 && ((reinterpret_cast<uintptr_t>(p.logits) | reinterpret_cast<uintptr_t>(p.q)) & 15) == 0;
+    const int v0 = (static_cast<int>(rank) * kWalkThreads + tid) * E;
     // every CTA gathers what every decision of the walk reads: they depend on
     // the tree and the drafts only, so all of them are loaded at once, up front
-    // (no CTA reads another's shared memory before the first cluster barrier)
-    if (tid > 0 && tid < n && tid < kMaxNodes) {
-        const int c = tid, pa = t->parent[c];
-        if (pa >= 0 && pa < c) {  // canonical order: a parent precedes its children
+    if (tid < n && in_bounds(n <= kMaxNodes && t->n == n, const_cast<int *>(p.ws_status))) {
+        const int c = tid, pa = t->parent[c], tok = c > 0 ? p.draft[c] : 0;
+        l_anc[c] = t->anc[c];
+        l_off[c] = p.logz_t[c] * kLog2e;
+        if (c > 0 && pa >= 0 && pa < c) {  // canonical order: a parent precedes its children
             atomicOr(reinterpret_cast<unsigned long long *>(&l_kids[pa]), 1ull << c);
-            const int tok = p.draft[c];
             const bool ok = tok >= 0 && tok < p.V;
             const float zt = ok ? p.logits[(size_t)pa * p.V + tok] : 0.f;
             l_ok[c] = ok;
@@ -389,19 +398,19 @@ __global__ void __cluster_dims__(kWalkCtas, 1, 1) __launch_bounds__(kWalkThreads
             l_uf[c] = p.unif[c];
         }
     }
-    __syncthreads();
-
-    const bool vec = (p.V & 3) == 0 && ((reinterpret_cast<uintptr_t>(p.logits) | reinterpret_cast<uintptr_t>(p.q)) & 15) == 0;
-    const int v0 = (static_cast<int>(rank) * kWalkThreads + tid) * E;
+    // the root's slices, while the gather's dependent loads are in flight
     float pv[E], qv[E];
+    load_slice<E>(p.logits, p.q, v0, p.V, vec, scale, p.logz_t[0] * kLog2e, pv, qv);
+    __syncthreads();
+    cluster_wait();
+
     int u = 0, nsum = 0;
-    bool bad = false, first = true, zero = false, have = false;  // have: pv, qv hold node u's slices
+    bool bad = false, first = true, zero = false, have = true;  // have: pv, qv hold node u's slices
     float cc = 0.f, S = 1.f;
     for (int hop = 0; hop < kMaxNodes; ++hop) {
         uint64_t kids = l_kids[u];
         first = true;
         zero = false;
-        have = false;
         cc = 0.f;
         S = 1.f;
         int next = -1;
@@ -417,8 +426,7 @@ __global__ void __cluster_dims__(kWalkCtas, 1, 1) __launch_bounds__(kWalkThreads
             }
             // rejected: c <- c + S, S <- sum_v max(0, p - c q) over node u's slices
             if (!have) {
-                load_slice<E>(p.logits + (size_t)u * p.V, p.q + (size_t)u * p.V, v0, p.V, vec, scale,
-                              p.logz_t[u] * kLog2e, pv, qv);
+                load_slice<E>(p.logits + (size_t)u * p.V, p.q + (size_t)u * p.V, v0, p.V, vec, scale, l_off[u], pv, qv);
                 have = true;
             }
             cc += S;
@@ -426,7 +434,7 @@ __global__ void __cluster_dims__(kWalkCtas, 1, 1) __launch_bounds__(kWalkThreads
 #pragma unroll
             for (int j = 0; j < E; ++j)
                 part += fmaxf(fmaf(-cc, qv[j], pv[j]), 0.f);
-            S = cluster_sum(part, red, &s_part[nsum & 1]);
+            S = cluster_sum<kCtas>(part, rank, s_vals[nsum & 1]);
             ++nsum;
             zero = !(S > 0.f);
             first = false;
@@ -434,35 +442,51 @@ __global__ void __cluster_dims__(kWalkCtas, 1, 1) __launch_bounds__(kWalkThreads
         if (next <= u)  // none accepted (ids of children exceed their parent's)
             break;
         u = next;
+        have = false;
     }
     if (!have)
-        load_slice<E>(p.logits + (size_t)u * p.V, p.q + (size_t)u * p.V, v0, p.V, vec, scale, p.logz_t[u] * kLog2e,
-                      pv, qv);
+        load_slice<E>(p.logits + (size_t)u * p.V, p.q + (size_t)u * p.V, v0, p.V, vec, scale, l_off[u], pv, qv);
+    const float uf = p.unif[n + u];
 
-    // inverse CDF of max(0, p - c q) (p itself before any rejection) at u
+    // inverse CDF of max(0, p - c q) (p itself before any rejection) at u: this
+    // thread's sum, its prefix in the warp, then the warp's prefix in the cluster
     float loc = 0.f;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         pv[j] = first ? pv[j] : (zero ? 0.f : fmaxf(fmaf(-cc, qv[j], pv[j]), 0.f));
         loc += pv[j];
     }
-    float cta_total;
-    const float before = block_exclusive_scan(loc, red, &cta_total);
-    if (tid == 0)
-        s_part[nsum & 1] = cta_total;
-    cluster_sync();
-    // the CTA totals in rank order: base = those of the lower ranks, grand = all
-    const float tot = lane < kWalkCtas ? ld_dsmem_f32(dsmem(&s_part[nsum & 1], lane)) : 0.f;
-    float base = 0.f, grand = 0.f;
+    float inc = loc;
 #pragma unroll
-    for (int r = 0; r < kWalkCtas; ++r) {
-        const float x = __shfl_sync(0xffffffffu, tot, r);
-        if (r == static_cast<int>(rank))
-            base = grand;
-        grand += x;
+    for (int d = 1; d < 32; d <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d)
+            inc += y;
     }
-    const float thr = p.unif[n + u] * grand;
-    const float c0 = base + before;
+    float *vals = s_vals[nsum & 1];
+    cluster_publish<kCtas>(__shfl_sync(0xffffffffu, inc, 31), rank, vals);
+    cluster_sync();
+    // lane l adds the totals of the cluster's warps [l * kCtas, (l + 1) * kCtas)
+    const int mine = static_cast<int>(rank) * kWalkWarps + warp;
+    float sum = 0.f, part = 0.f;  // part: of those before this warp
+#pragma unroll
+    for (int r = 0; r < kCtas; ++r) {
+        const float x = vals[lane * kCtas + r];
+        if (r == mine % kCtas)
+            part = sum;
+        sum += x;
+    }
+    float incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d)
+            incl += y;
+    }
+    const float grand = __shfl_sync(0xffffffffu, incl, 31);
+    const float base = __shfl_sync(0xffffffffu, incl - sum + part, mine / kCtas);
+    const float thr = uf * grand;
+    const float c0 = base + (inc - loc);
     if (loc > 0.f && c0 <= thr && thr < c0 + loc) {
         float cum = c0;
         int pick = -1, last = -1;
@@ -476,41 +500,83 @@ __global__ void __cluster_dims__(kWalkCtas, 1, 1) __launch_bounds__(kWalkThreads
             }
         }
         // into rank 0's s_tok (rounding can let two neighbouring chunks claim the threshold)
-        red_min_dsmem_s32(dsmem(&s_tok, 0), pick >= 0 ? pick : last);
+        red_min_cluster_s32(cluster_addr(&s_tok, 0), pick >= 0 ? pick : last);
     }
     cluster_sync();  // every claim has reached rank 0; no CTA touches another's shared memory after it
-    if (rank == 0 && tid == 0) {
-        const int tok = s_tok;
+    if (rank == 0 && tid < kMaxNodes) {
         tb_result *res = p.result;
-        const uint64_t anc = t->anc[u];
+        const uint64_t anc = l_anc[u];
         const int len = __popcll(anc);
-        int pos = 0;
-        for (int i = 0; i < kMaxNodes; ++i)
-            if ((anc >> i) & 1ull)
-                res->path[pos++] = i;
-        for (int i = pos; i < kMaxNodes; ++i)
-            res->path[i] = -1;
-        res->accept_len = len;
-        res->bonus_token = tok == 0x7fffffff ? p.V - 1 : tok;  // threshold at the total: the last token
-        res->new_L = p.L + len;
-        const int ws = p.ws_status ? *p.ws_status : 0;
-        res->status = (ws & kStatusTimeout) ? TB_ETIMEOUT
-                                            : ((bad || (ws & (kStatusBadToken | kStatusBounds))) ? TB_EINVAL : TB_OK);
+        if ((anc >> tid) & 1ull)
+            res->path[__popcll(anc & ((1ull << tid) - 1ull))] = tid;
+        if (tid >= len)
+            res->path[tid] = -1;
+        if (tid == 0) {
+            const int tok = s_tok;
+            res->accept_len = len;
+            res->bonus_token = tok == 0x7fffffff ? p.V - 1 : tok;  // threshold at the total: the last token
+            res->new_L = p.L + len;
+            const int ws = p.ws_status ? *p.ws_status : 0;
+            res->status = (ws & kStatusTimeout)
+                              ? TB_ETIMEOUT
+                              : ((bad || (ws & (kStatusBadToken | kStatusBounds))) ? TB_EINVAL : TB_OK);
+        }
     }
 }
 
+// Whether a cluster of kCtas CTAs can be resident (cached; 16 is above the
+// portable cluster size).
+template <int E, int kCtas>
+static bool walk_fits()
+{
+    static std::atomic<int> cache{0};  // 0: not queried yet, 1: no, 2: yes
+    int v = cache.load(std::memory_order_relaxed);
+    if (v == 0) {
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kCtas);
+        cfg.blockDim = dim3(kWalkThreads);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kCtas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if ((kCtas > 8 && cudaFuncSetAttribute(k4_spec_sample_cluster<E, kCtas>,
+                                               cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&n, k4_spec_sample_cluster<E, kCtas>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        v = n >= 1 ? 2 : 1;
+        cache.store(v, std::memory_order_relaxed);
+    }
+    return v == 2;
+}
+
+template <int E, int kCtas>
+static cudaError_t walk_launch(const SampleParams &p, cudaStream_t stream)
+{
+    return launch_kernel_cluster(k4_spec_sample_cluster<E, kCtas>, dim3(kCtas), dim3(kWalkThreads), 0, stream, true,
+                                 kCtas, p);
+}
+
+// The cluster by vocabulary: 8 CTAs up to 32768 (its barrier is the cheaper
+// one: 8.4 us at V 32000 against 10.8 for 16 CTAs), 16 CTAs with as few
+// entries per thread as cover it above (10.7 us at V 131072 against 13.4 for 8
+// CTAs with 16 entries), one CTA past 16 x 1024 x 16.
 cudaError_t sample_launch(const SampleParams &p, cudaStream_t stream)
 {
-    if (p.V <= kWalkCtas * kWalkThreads * 4)
-        k4_spec_sample_cluster<4><<<kWalkCtas, kWalkThreads, 0, stream>>>(p);
-    else if (p.V <= kWalkCtas * kWalkThreads * 16)
-        k4_spec_sample_cluster<16><<<kWalkCtas, kWalkThreads, 0, stream>>>(p);
-    else
-        k4_spec_sample<<<1, kSampleThreads, 0, stream>>>(p);
-    const cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess)
-        count_launch();
-    return e;
+    if (p.V <= 8 * kWalkThreads * 4)
+        return walk_launch<4, 8>(p, stream);
+    if (p.V <= 16 * kWalkThreads * 8 && walk_fits<8, 16>())
+        return walk_launch<8, 16>(p, stream);
+    if (p.V <= 8 * kWalkThreads * 16)
+        return walk_launch<16, 8>(p, stream);
+    if (p.V <= 16 * kWalkThreads * 16 && walk_fits<16, 16>())
+        return walk_launch<16, 16>(p, stream);
+    return launch_kernel(k4_spec_sample, dim3(1), dim3(kSampleThreads), 0, stream, true, p);
 }
 
 TB_BOUNDS_COUNTER(bounds_violations_sample)

@@ -994,6 +994,7 @@ static tb_status sample_enqueue(const tb_bank *bank, int bank_id, const int32_t 
 {
     SampleParams sp{};
     sp.tree = bank->d_desc + bank_id;
+    sp.n = bank->h_desc[bank_id].n;
     sp.draft = draft;
     sp.logits = logits;
     sp.logz_t = logz_t;
@@ -1085,7 +1086,7 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
         p.from_path = result->path;
         p.from_len = &result->accept_len;
         add_compaction(p, kv);
-        cudaError_t e = accept_launch(p, sm_count(bank->device), s, ss.accept_pdl());
+        cudaError_t e = accept_launch(p, sm_count(bank->device), s, true);  // a programmatic dependent of the walk
         if (e != cudaSuccess)
             return cuda_fail(e, fn);
     }

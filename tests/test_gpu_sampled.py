@@ -108,6 +108,22 @@ def test_walk_vocab_paths(dev, V):
     b.close()
 
 
+@pytest.mark.parametrize("V", [131075, 262144, 262145])
+def test_walk_large_vocab_paths(dev, V):
+    """Past the 8-CTA cluster's slices: unaligned rows on the 16-CTA cluster, the
+    largest vocabulary it holds (16 x 1024 threads x 16 entries: every slice
+    full), and one token more (the one-CTA walk)."""
+    b = tv.Bank(4, 0)
+    g = synth.rng(34 + V % 97)
+    for trial, parent in enumerate([synth.bank_trees()[-1], synth.bank_trees()[3]]):
+        z, q = _spiky_rows(g, len(parent), V, 4, T)
+        draft, unif, want = _draw_case(g, parent, z, q, T)
+        r = _walk_on_gpu(dev, b, parent, draft, z, q, unif, T, L=trial)
+        assert (r["accept_len"], r["path"], r["bonus_token"], r["new_L"], r["status"]) == (
+            want[0], want[1], want[2], trial + want[0], 0), (V, trial)
+    b.close()
+
+
 def test_walk_is_lossless_on_the_gpu(dev):
     """Root with three children drawn from q: the first emitted token follows p."""
     b = tv.Bank(4, 0)
