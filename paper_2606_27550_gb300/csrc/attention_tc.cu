@@ -101,7 +101,8 @@ struct TcSeq {
     const __nv_bfloat16 *q;  // [n_layers][nstride][Hq][head_dim]
     __nv_bfloat16 *out;      // same layout
     const TreeDesc *tree;
-    int L, N, rows, row_blocks, T;
+    int L, N, rows, row_blocks, T;  // row_blocks: 128-row blocks in the unit index (1 when row_split is 2)
+    int row_split;           // 2: the CTAs 2c and 2c + 1 take the two row blocks of the same units
     int nstride;             // nodes per layer in q / out (N, or the largest tree of a scheduled loop)
 };
 
@@ -120,13 +121,24 @@ struct TcParams {
     const int32_t *sched;
     const TreeDesc *rung_tree[8];
     int n_rungs, n_layers, L_cap;
-    int max_rows;  // query rows of the largest row block (the split merge's grid)
+    int max_rows;  // rows the split merge's grid covers: of the largest row block, or of both (row_split)
     int d;         // head_dim: the kernels' kD (host side: picks the instantiation)
     int cluster;   // > 1: a cluster of that many CTAs shares each unit (one sequence; see attn_tc_clusters)
     // rotary embedding (null: the queries are already rotated): per sequence a
     // table of (cos, sin) at position L + depth for every pair of head elements
     const float2 *rope_tab;
 };
+
+// Two row blocks per kv head (grouped queries, 129 to 256 rows) and more than a
+// wave of tiles: neighbouring CTAs walk the same key tiles side by side, one
+// row block each, so that the second reading of a tile comes from L2.  As units
+// of their own the two blocks are read a whole unit apart: at 32 layers, 32 q /
+// 8 kv heads, 64 nodes at 8192 keys that streams K and V from HBM twice, and
+// the step took 487 us, now MEASURED.
+__host__ __device__ inline bool split_rows(int row_blocks, long long total, int n_ctas)
+{
+    return row_blocks == 2 && total >= n_ctas && n_ctas >= 2;
+}
 
 // Scheduled mode: the sequence of this step from the device state.  An
 // out-of-range rung or a prefix that does not fit the cache gives no work
@@ -145,6 +157,8 @@ __device__ void sched_plan(const TcParams &p, TcSeq *sq, long long *total)
     sq->rows = N * p.group;
     sq->row_blocks = (sq->rows + 127) / 128;
     sq->T = (sq->L + N + kBN - 1) / kBN;
+    sq->row_split = split_rows(sq->row_blocks, (long long)p.n_layers * p.Hkv * sq->row_blocks * sq->T, p.P) ? 2 : 1;
+    sq->row_blocks /= sq->row_split;
     *total = (ok && L + N <= p.L_cap) ? (long long)p.n_layers * p.Hkv * sq->row_blocks * sq->T : 0;
 }
 
@@ -162,14 +176,16 @@ __device__ __forceinline__ int seq_at(const TcParams &p, long long t, int b)
     }
 }
 
-// CTAs the tile space is split over.  The host plans at most one CTA per
+// Ranges the tile space is split over: one per CTA, or per pair of CTAs with
+// the same tiles and a row block each (row_split = 2).  The host plans at most one CTA per
 // tile; scheduled mode plans on the device with a grid of one CTA per SM, and
 // a step with fewer tiles than that splits them over its first `total` CTAs
 // only (the others get nothing), so that no CTA range inside the split is
 // empty: the split merge combines the partials of consecutive CTAs.
-__device__ __forceinline__ int tc_split_ctas(const TcParams &p, long long total)
+__device__ __forceinline__ int tc_split_ctas(const TcParams &p, long long total, int row_split)
 {
-    return (p.sched && total < p.P) ? (int)(total > 0 ? total : 1) : p.P;
+    const int n = p.P / row_split;
+    return (p.sched && total < n) ? (int)(total > 0 ? total : 1) : n;
 }
 
 // First flattened tile of CTA c's range (the ranges split the tile space
@@ -341,9 +357,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         t0 = first + (long long)T * rank / p.cluster;
         t1 = first + (long long)T * (rank + 1) / p.cluster;
     } else {
-        const int P = tc_split_ctas(p, total);
-        t0 = c < P ? tc_seg_begin(total, P, c) : total;
-        t1 = c < P ? tc_seg_begin(total, P, c + 1) : total;
+        const int rs = kBatched ? 1 : seqs[0].row_split;
+        const int P = tc_split_ctas(p, total, rs), r = c / rs;
+        t0 = r < P ? tc_seg_begin(total, P, r) : total;
+        t1 = r < P ? tc_seg_begin(total, P, r + 1) : total;
     }
     tc_fence_before();
     __syncthreads();
@@ -645,7 +662,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             g.first = t == t0;
             g.b = sb;
             g.L = sq.L;
-            const int rb = sp.u % sq.row_blocks;
+            const int rb = sp.u % sq.row_blocks + (kBatched || kCluster ? 0 : c % sq.row_split);
             const int head = (sp.u / sq.row_blocks) % p.Hkv;
             const int layer_rel = sp.u / (sq.row_blocks * p.Hkv);
             g.valid = rloc < min(128, sq.rows - rb * 128);
@@ -953,7 +970,8 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
         seqs = &s_seq;
         total = s_total;
     }
-    const int P = tc_split_ctas(p, total);
+    const int rs = kBatched ? 1 : seqs[0].row_split;
+    const int P = tc_split_ctas(p, total, rs);
     const int cb = blockIdx.x + 1;  // CTA range starting at tile t_c
     if (cb >= P)
         return;
@@ -972,12 +990,12 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
     if (cb != c_lo + 1)
         return;  // an earlier boundary inside this unit handles it
     const int nseg = c_hi - c_lo + 1;
-    const int rb = u % sq.row_blocks;
     const int head = (u / sq.row_blocks) % p.Hkv;
     const int layer_rel = u / (sq.row_blocks * p.Hkv);
-    const int rows_here = min(128, sq.rows - rb * 128);
-    const int r = blockIdx.y * 8 + warp;
-    if (r >= rows_here)
+    const int r_all = blockIdx.y * 8 + warp;  // row of the unit: of both row blocks when split between two CTAs
+    const int half = rs == 2 ? r_all / 128 : 0;
+    const int r = r_all - 128 * half, rb = u % sq.row_blocks + half;
+    if (r >= min(128, sq.rows - rb * 128))
         return;
     {
         const int grow = rb * 128 + r;
@@ -991,7 +1009,7 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
     for (int j0 = 0; j0 < nseg; j0 += 32) {
         const int cc = c_lo + j0 + lane;
         if (j0 + lane < nseg) {
-            const float *sl = p.part + ((size_t)cc * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
+            const float *sl = p.part + ((size_t)(cc * rs + half) * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
             M = fmaxf(M, __ldcg(sl + 128 * kD + r));
         }
     }
@@ -1005,7 +1023,7 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
         const float *sl = p.part;
         float w = 0.f;
         if (j0 + lane < nseg) {
-            sl = p.part + ((size_t)cc * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
+            sl = p.part + ((size_t)(cc * rs + half) * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
             const float ms = __ldcg(sl + 128 * kD + r);
             w = (ms == -INFINITY) ? 0.f : ex2_approx(ms - M);
             lsum += w * __ldcg(sl + 128 * kD + 128 + r);
@@ -1058,7 +1076,8 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
 template <int kD>
 static cudaError_t merge_launch_d(const TcParams &p, bool batched, cudaStream_t stream, bool pdl, bool after_step)
 {
-    const dim3 grid(p.P - 1, (p.max_rows + 7) / 8);
+    // scheduled mode chooses row_split on the device: the grid covers both choices
+    const dim3 grid((p.sched ? p.P : p.P / p.seq[0].row_split) - 1, (p.max_rows + 7) / 8);
     if (batched)
         return after_step ? launch_kernel(k1_merge_split<kD, true, true>, grid, dim3(256), 0, stream, pdl, p)
                           : launch_kernel(k1_merge_split<kD, true, false>, grid, dim3(256), 0, stream, pdl, p);
@@ -1075,8 +1094,9 @@ static bool any_split(const TcParams &p)
     if (p.sched)
         return true;
     int b = 0;
-    for (int c = 1; c < p.P; ++c) {
-        const long long t = (long long)((unsigned long long)c * (unsigned long long)p.total / (unsigned long long)p.P);
+    const int n = p.P / p.seq[0].row_split;
+    for (int c = 1; c < n; ++c) {
+        const long long t = (long long)((unsigned long long)c * (unsigned long long)p.total / (unsigned long long)n);
         while (b + 1 < p.n_seq && t >= p.seq[b + 1].tile_base)
             ++b;
         if ((t - p.seq[b].tile_base) % p.seq[b].T != 0)
@@ -1184,6 +1204,11 @@ AttnPlan attn_tc_plan(int L, int N, int Hq, int Hkv, int n_layers, int n_sm)
     // GB300: whole units faster up to 5 tiles, even at 6-7).
     if (pl.total <= n_sm && pl.T <= kWholeUnitMaxTiles)
         P = pl.n_units;
+    pl.row_split = 1;
+    if (split_rows(pl.row_blocks, pl.total, n_sm)) {
+        pl.row_split = 2;
+        P &= ~1ll;
+    }
     pl.P = (int)P;
     return pl;
 }
@@ -1272,6 +1297,7 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
         sq.row_blocks = pl.row_blocks;
         sq.T = pl.T;
         sq.nstride = seqs[b].N;
+        sq.row_split = 1;
         tiles += pl.total;
         max_rows = pl.rows < 128 ? (pl.rows > max_rows ? pl.rows : max_rows) : 128;
     }
@@ -1282,10 +1308,25 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     p.layer_begin = layer_begin;
     p.n_layers = n_layers;
     p.total = tiles;
-    // one sequence: its plan (whole units for a short one-wave problem); a batch
-    // splits its tiles evenly (units of different lengths)
-    p.P = n_seq == 1 ? attn_tc_plan(seqs[0].kv->L, seqs[0].N, Hq, Hkv, n_layers, n_sm).P
-                     : (int)(tiles < n_sm ? tiles : n_sm);
+    // a batch splits its tiles evenly (units of different lengths)
+    p.P = (int)(tiles < n_sm ? tiles : n_sm);
+    p.cluster = 1;
+    if (n_seq == 1) {
+        // one sequence: its plan (whole units for a short one-wave problem), or in a call of its
+        // own, not part of a step, clusters that share the units of a small problem
+        const AttnPlan pl = attn_tc_plan(seqs[0].kv->L, seqs[0].N, Hq, Hkv, n_layers, n_sm);
+        p.P = pl.P;
+        if (alone)
+            p.cluster = attn_tc_clusters(pl, d, n_sm);
+        if (p.cluster > 1) {
+            p.P = pl.n_units * p.cluster;
+        } else if (pl.row_split == 2) {
+            p.seq[0].row_split = 2;
+            p.seq[0].row_blocks = 1;
+            p.total = tiles / 2;
+            max_rows = pl.rows;
+        }
+    }
     p.d = d;
     p.scale_log2 = 1.4426950408889634f / sqrtf((float)d);
     p.part = part;
@@ -1293,14 +1334,6 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     p.rope_tab = rope_tab;
     p.max_rows = max_rows;
     const bool batched = n_seq > 1;
-    // a call of its own, not part of a step: clusters share the units of a small problem
-    p.cluster = 1;
-    if (n_seq == 1 && alone) {
-        const AttnPlan pl = attn_tc_plan(seqs[0].kv->L, seqs[0].N, Hq, Hkv, n_layers, n_sm);
-        p.cluster = attn_tc_clusters(pl, d, n_sm);
-        if (p.cluster > 1)
-            p.P = pl.n_units * p.cluster;
-    }
     cudaError_t e;
     // In a step, a grid that takes every SM starts when the stream's previous
     // work is done, so that all its CTAs start together (its work split is
@@ -1350,6 +1383,7 @@ cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *
     sq.nstride = sc.N_max;
     sq.T = 1;
     sq.row_blocks = 1;
+    sq.row_split = 1;
     p.n_seq = 1;
     p.Hq = Hq;
     p.Hkv = kv->n_kv_heads;
@@ -1367,7 +1401,7 @@ cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *
     p.n_rungs = sc.n_rungs;
     for (int r = 0; r < sc.n_rungs; ++r)
         p.rung_tree[r] = sc.rung_tree[r];
-    p.max_rows = sc.N_max * p.group < 128 ? sc.N_max * p.group : 128;
+    p.max_rows = sc.N_max * p.group;
     cudaError_t e;
     if ((e = attn_kernel_launch(p, false, stream, false)) != cudaSuccess)
         return e;

@@ -124,6 +124,7 @@ constexpr int kMaxSeqPerLaunch = TB_MAX_BATCH;
 // 128-key tiles each, over P persistent CTAs.
 struct AttnPlan {
     int group, rows, row_blocks, T, n_units, P;
+    int row_split;  // 2: pairs of CTAs share their key tiles, one row block each
     long long total;
 };
 struct AttnSeq {
