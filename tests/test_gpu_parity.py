@@ -146,6 +146,19 @@ def test_tree_attention_clusters(dev, bank, Hq, Hkv, tree, L, d):
     _run_attention(bank, dev, synth.bank_trees()[tree], L, 1, Hq, Hkv, d, seed=L + d, derived=True)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("Hq,Hkv,tree,L,layers", [
+    (32, 8, 7, 700, 4),   # 256 rows: both row blocks full
+    (32, 8, 6, 500, 5),   # 160 rows: 32 in the second block
+    (16, 2, 5, 1300, 8),  # 208 rows
+    (8, 2, 7, 0, 40),     # single-tile units, more than a wave of them
+])
+def test_tree_attention_row_blocks_side_by_side(dev, bank, Hq, Hkv, tree, L, layers, d):
+    """Two row blocks per kv head and more than a wave of tiles: pairs of CTAs
+    take the same key tiles, one row block each, and the split merge covers both."""
+    _run_attention(bank, dev, synth.bank_trees()[tree], L, layers, Hq, Hkv, d, seed=L + d, derived=True)
+
+
 def test_tree_attention_large_L_multilayer(dev, bank):
     _run_attention(bank, dev, synth.bank_trees()[-1], 5000, 3, 8, 8, 128, seed=4)
 
