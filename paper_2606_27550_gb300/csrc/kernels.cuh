@@ -53,6 +53,7 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 // LM head (lm_head.cu)
 struct LmPlan {
     int R_pad, n_tiles, n_kblocks, stages, acc_cols;
+    int tile_rows;    // vocab entries per tile and CTA
     int ctas_per_sm;  // 2 when two rings fit side by side, else 1
     bool pair;        // CTA pairs share each MMA (M = 256); tiles are then 256 vocab entries
     int units;        // the tile split's units: CTAs, or CTA pairs
@@ -60,11 +61,14 @@ struct LmPlan {
     int n_slots;      // per-tile partials: one per tile and CTA (two per pair tile)
     int n_counters;   // workspace counters used (the tile counter)
     size_t smem_bytes;
-    size_t ws_bytes;  // per-tile partials, 256-byte aligned
+    size_t ws_bytes;  // the least room for per-tile partials that a call needs, 256-byte aligned
 };
-// n_sm: the SMs the launch may use; max_pairs: the clusters of two that can
-// be resident at once (-1: n_sm / 2), which bounds the pairs of a pair plan.
-LmPlan lm_plan(int R, int D, int V, int n_sm, int max_pairs = -1);
+// n_sm: the SMs the launch may use; parts_bytes: the room for per-tile
+// partials; max_pairs: the clusters of two that can be resident at once (-1:
+// n_sm / 2), which bounds the pairs of a pair plan.
+LmPlan lm_plan(int R, int D, int V, int n_sm, size_t parts_bytes, int max_pairs = -1);
+// Room for the partials of every plan of up to R rows.
+size_t lm_parts_bytes(int R, int V, int n_sm);
 // typical-acceptance inputs produced by the same pass: per-row statistics at
 // temperature T and the draft-token logit of every tree edge j, written to
 // seq[b].out[j] for edges whose parent row row_base + parent[j] is in [0, R)
@@ -89,7 +93,7 @@ struct LmTypical {
 // verification step's attention); the LM head does not wait for it, but
 // completes only after it
 cudaError_t lm_head_launch(const void *hidden, int R, const void *W, int D, int V, int32_t *argmax, float *top1,
-                           float *entropy, void *parts, int *counters, int *status, int n_sm, cudaStream_t stream,
+                           float *entropy, void *parts, size_t parts_bytes, int *counters, int *status, int n_sm, cudaStream_t stream,
                            const char **err, int expire_wait = 0, const LmTypical *typ = nullptr, bool pdl = false);
 
 // rotary embedding at the tree's position offsets (rope.cu)

@@ -38,7 +38,8 @@ struct LmParams {
     CUtensorMap tmap_w;  // (d_model, vocab), box (64, 128), 128B swizzle
     CUtensorMap tmap_h;  // (d_model, rows),  box (64, R_pad) (R_pad / 2 for CTA pairs), 128B swizzle
     int R, R_pad, D, V;
-    int n_tiles, nk, stages, acc_cols;  // tiles of 128 vocab entries (256 for CTA pairs)
+    int n_tiles, nk, stages, acc_cols;
+    int tile_rows;       // vocab entries per tile and CTA: up to 128 (128 in a pair, whose tiles are two of them)
     int units;           // the tile split's units: CTAs, or CTA pairs
     int n_slots;         // per-tile partials: one per tile (two per pair tile, one per CTA)
     float4 *part_tile;   // [n_slots][R_pad]  (max, argmax bits, s, t)
@@ -220,7 +221,8 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
     const int S = p.stages;
     // one 64-column box of this CTA's tree rows (half of them in a pair)
     const uint32_t hb = (uint32_t)(kPair ? p.R_pad / 2 : p.R_pad) * 128u;
-    const uint32_t stage_bytes = 16384u + hb;
+    const uint32_t stage_bytes = 16384u + hb;                               // a ring slot
+    const uint32_t stage_tx = (uint32_t)p.tile_rows * 128u + hb;            // what its loads bring
     uint8_t *ring = smem;
     float *chunk = reinterpret_cast<float *>(smem + (size_t)S * stage_bytes);  // [kLmChunk][kChunkLd]
 
@@ -283,6 +285,7 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
             uint32_t ph = 0;
             long long g = 0;    // the current tile's first k-block in the CTA's sequence
             long long g_end = 0;
+            const uint64_t w_policy = l2_evict_first();  // W is read once: it should not push out what is reused
             bool ok = true;
             // tile scheduler (warp 0 of the even CTA): entry i + 1 of the queue is
             // published while tile i streams; its tile was fetched a tile earlier
@@ -325,15 +328,16 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
                     if constexpr (kPair) {
                         // the stage's four boxes (W and tree rows of both CTAs) complete on the even CTA's barrier
                         if (leader)
-                            mbar_arrive_expect_tx(&full_bar[s], 2 * stage_bytes);
+                            mbar_arrive_expect_tx(&full_bar[s], 2 * stage_tx);
                         const uint32_t fb = cluster_addr(&full_bar[s], 0);
-                        tma_load_2d_pair(ring + (size_t)s * stage_bytes, &p.tmap_w, fb, kb * 64,
-                                         tile * 256 + (int)rank * 128);
+                        tma_load_2d_pair_hint(ring + (size_t)s * stage_bytes, &p.tmap_w, fb, kb * 64,
+                                              tile * 256 + (int)rank * 128, w_policy);
                         tma_load_2d_pair(ring + (size_t)s * stage_bytes + 16384, &p.tmap_h, fb, kb * 64,
                                          (int)rank * (p.R_pad / 2));
                     } else {
-                        mbar_arrive_expect_tx(&full_bar[s], stage_bytes);
-                        tma_load_2d(ring + (size_t)s * stage_bytes, &p.tmap_w, &full_bar[s], kb * 64, tile * 128);
+                        mbar_arrive_expect_tx(&full_bar[s], stage_tx);
+                        tma_load_2d_hint(ring + (size_t)s * stage_bytes, &p.tmap_w, &full_bar[s], kb * 64,
+                                         tile * p.tile_rows, w_policy);
                         tma_load_2d(ring + (size_t)s * stage_bytes + 16384, &p.tmap_h, &full_bar[s], kb * 64, 0);
                     }
                     g_end = g + j + 1;
@@ -452,7 +456,8 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
                 break;
             tc_fence_after();
             // this CTA's 128 vocab entries (the odd CTA of a pair's last tile may have none)
-            const int v0 = kPair ? tile * 256 + (int)rank * 128 : tile * 128, nvalid = min(128, p.V - v0);
+            const int v0 = kPair ? tile * 256 + (int)rank * 128 : tile * p.tile_rows;
+            const int nvalid = min(p.tile_rows, p.V - v0);
             const int slot = kPair ? 2 * tile + (int)rank : tile;  // this CTA's partial of the tile
             if constexpr (kTyp) {
                 // the tree edges whose draft token lies in this tile
@@ -589,7 +594,7 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
             const long long mine = threadIdx.x, gl = s_gend[mine], go = s_peer_gend[mine];
             for (long long it = gl; it < go; ++it)
                 if ((it & 1) == mine)
-                    mbar_arrive_expect_tx(&full_bar[it % S], stage_bytes);
+                    mbar_arrive_expect_tx(&full_bar[it % S], stage_tx);
             const long long ge = gl > go ? gl : go;
             if (abort_flag || gl != go)
                 for (long long it = (ge > S ? ge - S : 0); it < ge; ++it)
@@ -746,7 +751,10 @@ static int ceil_div(int a, int b)
     return (a + b - 1) / b;
 }
 
-LmPlan lm_plan(int R, int D, int V, int n_sm, int max_pairs)
+// Bytes of one (max, argmax, s, t) and one (sT, tT) partial.
+constexpr size_t kPartBytes = 16 + 8;
+
+LmPlan lm_plan(int R, int D, int V, int n_sm, size_t parts_bytes, int max_pairs)
 {
     LmPlan pl{};
     if (n_sm < 1)
@@ -758,21 +766,24 @@ LmPlan lm_plan(int R, int D, int V, int n_sm, int max_pairs)
         cols *= 2;
     pl.acc_cols = cols;
     const size_t fixed = (size_t)kLmChunk * kChunkLd * 4;  // the epilogue's chunk buffer
-    // Two CTAs share an SM when each still gets a ring of at least three stages
+    // Two CTAs can share an SM when each still gets a ring of at least three stages
     // in half of its shared memory and four accumulators fit in TMEM: two
     // independent TMA pipelines per SM stream W faster than one deeper ring.
     const size_t pad = 1024 + 1024;  // alignment pad, static shared memory
     const size_t half = 112 * 1024;
     const size_t stage1 = 16384 + (size_t)pl.R_pad * 128;
     const int st2 = half > fixed + pad ? (int)((half - fixed - pad) / stage1) : 0;
-    pl.ctas_per_sm = (st2 >= 3 && 4 * cols <= 512) ? 2 : 1;
+    const bool two = st2 >= 3 && 4 * cols <= 512;
+    // Over many rounds of tiles one CTA with a ring twice as deep is faster: 26
+    // rows x 4096, V 128256 160 us against 166, V 100000 x 1024 39.5 against
+    // 40.0; V 80000 108 against 106, V 32000 51 against 46.
+    pl.ctas_per_sm = two && ceil_div(V, 128) <= 5 * n_sm ? 2 : 1;
     // Otherwise (wide rows, one CTA per SM) CTA pairs share each MMA: each CTA
     // stages half of the rows, so the rows cross each SM's shared memory once
     // per 256 vocab entries instead of once per 128.
     if (max_pairs < 0)
         max_pairs = n_sm / 2;
-    pl.pair = pl.ctas_per_sm == 1 && max_pairs >= 1;
-    pl.n_tiles = ceil_div(V, pl.pair ? 256 : 128);
+    pl.pair = !two && max_pairs >= 1;
     const size_t stage_bytes = 16384 + (size_t)(pl.pair ? pl.R_pad / 2 : pl.R_pad) * 128;
     const size_t budget = (pl.ctas_per_sm == 2 ? half : 227 * 1024) - fixed - pad;
     pl.stages = (int)(budget / stage_bytes);
@@ -780,31 +791,48 @@ LmPlan lm_plan(int R, int D, int V, int n_sm, int max_pairs)
         pl.stages = 8;
     if (pl.stages < 2)
         pl.stages = 2;
-    if (pl.pair) {
-        pl.units = max_pairs < pl.n_tiles ? max_pairs : pl.n_tiles;
-        pl.P = 2 * pl.units;
-    } else {
-        const int slots = pl.ctas_per_sm * n_sm;
-        pl.P = slots < pl.n_tiles ? slots : pl.n_tiles;
-        pl.units = pl.P;
+    // tiles of 128 vocab entries (256 for a pair)
+    pl.tile_rows = 128;
+    pl.n_tiles = ceil_div(V, pl.pair ? 256 : 128);
+    const int slots = pl.pair ? max_pairs : pl.ctas_per_sm * n_sm;
+    if (!pl.pair) {
+        // Lower tiles where they spread several rounds of the vocabulary evenly over
+        // the CTAs, in as many rounds as 128-entry tiles take, and the workspace has
+        // room for their partials: V 40000 59 us against 72, V 80000 106 against
+        // 120, V 64000 87 against 86 (26 and 64 rows x 4096).  A single round is
+        // left alone (V 32000 46.7 against 46.1): HBM is busy either way.
+        const int rounds = ceil_div(pl.n_tiles, slots);
+        const int rows = ceil_div(V, rounds * slots);
+        const int tiles = ceil_div(V, rows);
+        if (rounds > 1 && (size_t)tiles * pl.R_pad * kPartBytes <= parts_bytes) {
+            pl.tile_rows = rows;
+            pl.n_tiles = tiles;
+        }
     }
+    pl.units = slots < pl.n_tiles ? slots : pl.n_tiles;
+    pl.P = pl.pair ? 2 * pl.units : pl.units;
     // per-tile partials: one per tile and CTA, merged by k2_lm_merge
     pl.n_slots = pl.pair ? 2 * pl.n_tiles : pl.n_tiles;
     pl.smem_bytes = (size_t)pl.stages * stage_bytes + fixed + 1024;
-    // (max, argmax, s, t) and (sT, tT) partials.  The workspace also covers the
-    // plan without pairs, which a launch takes when no cluster of two can be
-    // resident.
-    const int slots1 = ceil_div(V, 128);
-    const int parts = pl.n_slots > slots1 ? pl.n_slots : slots1;
     pl.n_counters = 1;  // the tile counter
-    pl.ws_bytes = ((size_t)parts * pl.R_pad * (16 + 8) + 255) / 256 * 256;
+    // What a call needs: the partials of 128-entry tiles (two per pair tile), or
+    // of the plan without pairs, which a launch takes when no cluster of two can
+    // be resident.
+    const int slots1 = ceil_div(V, 128), slots2 = 2 * ceil_div(V, 256);
+    pl.ws_bytes = ((size_t)(pl.pair && slots2 > slots1 ? slots2 : slots1) * pl.R_pad * kPartBytes + 255) / 256 * 256;
     return pl;
+}
+
+size_t lm_parts_bytes(int R, int V, int n_sm)
+{
+    // lower tiles add at most one tile per CTA (two CTAs per SM) to those of 128 entries
+    return ((size_t)(ceil_div(V, 128) + 1 + 2 * n_sm) * (ceil_div(R, 16) * 16) * kPartBytes + 255) / 256 * 256;
 }
 
 // Clusters of two CTAs of k2_lm_head<kTyp, true> with `smem` bytes each that
 // can be resident at once (cached per shared-memory size; 0 if none).
 template <bool kTyp>
-static int lm_max_pairs(size_t smem, int n_sm)
+static int lm_max_pairs(size_t smem)
 {
     static std::atomic<int> cache[24];  // by smem / 16 KB; 0: not queried yet, else pairs + 1
     const size_t slot = smem / 16384 < 24 ? smem / 16384 : 23;
@@ -813,7 +841,7 @@ static int lm_max_pairs(size_t smem, int n_sm)
         return v - 1;
     int pairs = 0;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * (n_sm / 2 > 0 ? n_sm / 2 : 1));
+    cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(kLmThreads);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
@@ -828,8 +856,6 @@ static int lm_max_pairs(size_t smem, int n_sm)
         (void)cudaGetLastError();
         pairs = 0;
     }
-    if (pairs > n_sm / 2)
-        pairs = n_sm / 2;
     cache[slot].store(pairs + 1, std::memory_order_relaxed);
     return pairs;
 }
@@ -856,18 +882,19 @@ static cudaError_t lm_launch_as(LmParams &p, const LmPlan &pl, cudaStream_t stre
 }
 
 cudaError_t lm_head_launch(const void *hidden, int R, const void *W, int D, int V, int32_t *argmax, float *top1,
-                           float *entropy, void *parts, int *counters, int *status, int n_sm, cudaStream_t stream,
+                           float *entropy, void *parts, size_t parts_bytes, int *counters, int *status, int n_sm, cudaStream_t stream,
                            const char **err, int expire_wait, const LmTypical *typ, bool pdl)
 {
-    LmPlan pl = lm_plan(R, D, V, n_sm);
+    LmPlan pl = lm_plan(R, D, V, n_sm, parts_bytes);
     if (pl.pair) {
         // as many pairs as can be resident at once (the SMs of a cluster share a GPC)
-        const int mp = typ ? lm_max_pairs<true>(pl.smem_bytes, n_sm) : lm_max_pairs<false>(pl.smem_bytes, n_sm);
+        int mp = typ ? lm_max_pairs<true>(pl.smem_bytes) : lm_max_pairs<false>(pl.smem_bytes);
+        mp = mp < n_sm / 2 ? mp : n_sm / 2;
         if (mp != pl.units || mp < 1)
-            pl = lm_plan(R, D, V, n_sm, mp);
+            pl = lm_plan(R, D, V, n_sm, parts_bytes, mp);
     }
     LmParams p{};
-    if (!make_tmap_2d(&p.tmap_w, W, (uint64_t)D, (uint64_t)V, (uint64_t)D * 2, 64, 128, err))
+    if (!make_tmap_2d(&p.tmap_w, W, (uint64_t)D, (uint64_t)V, (uint64_t)D * 2, 64, (uint32_t)pl.tile_rows, err))
         return cudaErrorInvalidValue;
     if (!make_tmap_2d(&p.tmap_h, hidden, (uint64_t)D, (uint64_t)R, (uint64_t)D * 2, 64,
                       (uint32_t)(pl.pair ? pl.R_pad / 2 : pl.R_pad), err))
@@ -877,6 +904,7 @@ cudaError_t lm_head_launch(const void *hidden, int R, const void *W, int D, int 
     p.D = D;
     p.V = V;
     p.n_tiles = pl.n_tiles;
+    p.tile_rows = pl.tile_rows;
     p.nk = pl.n_kblocks;
     p.stages = pl.stages;
     p.acc_cols = pl.acc_cols;

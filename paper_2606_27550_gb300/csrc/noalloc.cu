@@ -90,7 +90,7 @@ extern "C" tb_status lm_head_stats_noalloc(const void *hidden, int n_rows, const
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return record_error(TB_ECUDA, "%s: no current device", fn);
     const char *err = "";
-    e = lm_head_launch(hidden, n_rows, lm_head, d_model, vocab, argmax, top1, entropy, parts, counters,
+    e = lm_head_launch(hidden, n_rows, lm_head, d_model, vocab, argmax, top1, entropy, parts, kNoAllocScratchBytes, counters,
                        counters + kNoAllocStatusWord, n_sm, (cudaStream_t)stream, &err,
                        (flags & TB_DEBUG_EXPIRE_WAIT) ? 1 : 0);
     if (e != cudaSuccess)

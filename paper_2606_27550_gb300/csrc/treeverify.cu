@@ -525,7 +525,7 @@ extern "C" size_t tb_workspace_size(int max_rows, int n_layers, int n_kv_heads, 
     if (head_dim > 0)
         bytes += attn_part_bytes(nsm, head_dim);
     if (max_rows > 0 && vocab > 0)  // batched calls run the LM head in chunks of 256 rows
-        bytes += align256(lm_plan(max_rows < 256 ? max_rows : 256, 64, vocab, nsm).ws_bytes);
+        bytes += align256(lm_parts_bytes(max_rows < 256 ? max_rows : 256, vocab, nsm));
     return bytes;
 }
 
@@ -769,20 +769,20 @@ tb_status tv::lm_validate(const void *hidden, int R, const void *W, int D, int V
         return fail(TB_EINVAL, "%s: d_model %d must be a positive multiple of 8", fn, D);
     if (V < 1)
         return fail(TB_EINVAL, "%s: vocab %d", fn, V);
-    *plan = lm_plan(R, D, V, sm_count(current_device()));
+    *plan = lm_plan(R, D, V, sm_count(current_device()), 0);
     if (plan->n_counters > kMaxLmCounters)
         return fail(TB_EUNSUPPORTED, "%s: vocab %d too large", fn, V);
     return TB_OK;
 }
 
 static tb_status lm_enqueue(const void *hidden, int R, const void *W, int D, int V, int32_t *am, float *t1, float *en,
-                            uint8_t *ws, size_t part_off, cudaStream_t stream, const char *fn, int expire_wait = 0,
-                            const LmTypical *typ = nullptr, bool pdl = false)
+                            uint8_t *ws, size_t ws_bytes, size_t part_off, cudaStream_t stream, const char *fn,
+                            int expire_wait = 0, const LmTypical *typ = nullptr, bool pdl = false, int n_sm = 0)
 {
     const char *err = "";
-    cudaError_t e = lm_head_launch(hidden, R, W, D, V, am, t1, en, ws + part_off,
+    cudaError_t e = lm_head_launch(hidden, R, W, D, V, am, t1, en, ws + part_off, ws_bytes - part_off,
                                    reinterpret_cast<int *>(ws + kLmCounterOff), reinterpret_cast<int *>(ws),
-                                   sm_count(current_device()), stream, &err, expire_wait, typ, pdl);
+                                   n_sm > 0 ? n_sm : sm_count(current_device()), stream, &err, expire_wait, typ, pdl);
     if (e == cudaErrorInvalidValue && err[0])
         return fail(TB_EINVAL, "%s: %s", fn, err);
     if (e != cudaSuccess)
@@ -882,7 +882,7 @@ extern "C" tb_status lm_head_stats(const void *hidden, int n_rows, const void *l
     if ((st = check_ws(workspace, workspace_bytes, kPartBase + plan.ws_bytes, fn)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, n_rows, lm_head, d_model, vocab, argmax, top1, entropy,
-                         static_cast<uint8_t *>(workspace), kPartBase, (cudaStream_t)stream, fn)) != TB_OK)
+                         static_cast<uint8_t *>(workspace), workspace_bytes, kPartBase, (cudaStream_t)stream, fn)) != TB_OK)
         return st;
     return ok();
 }
@@ -933,7 +933,7 @@ extern "C" tb_status lm_head_stats_typical(const tb_bank *bank, int bank_id, con
     lt.gather.n_seq = 1;
     lt.gather.seq[0] = LmGatherSeq{bank->d_desc + bank_id, draft_tokens, draft_logit, 0, N};
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, static_cast<uint8_t *>(workspace),
-                         kPartBase, (cudaStream_t)stream, fn, 0, &lt)) != TB_OK)
+                         workspace_bytes, kPartBase, (cudaStream_t)stream, fn, 0, &lt)) != TB_OK)
         return st;
     return ok();
 }
@@ -974,10 +974,14 @@ extern "C" tb_status typical_accept(const tb_bank *bank, int bank_id, const int3
 // size and the step runs as the same chain: both start at once, and the
 // programmatic launches hide the launch latencies (the tiny step: 60-65 k
 // verify-steps/s against 47-57 k with the LM head forked).  0: no cap.
+static int lm_sms_beside_attn(const LmPlan &lp)
+{
+    return (lp.P + lp.ctas_per_sm - 1) / lp.ctas_per_sm;
+}
+
 static int attn_ctas_beside_lm(const AttnPlan &ap, const LmPlan &lp, int d_model, int vocab, int n_sm)
 {
-    const int lm_sms = (lp.P + lp.ctas_per_sm - 1) / lp.ctas_per_sm;
-    const int free_sms = n_sm - lm_sms;
+    const int free_sms = n_sm - lm_sms_beside_attn(lp);
     if (free_sms < 1 || ap.total < 1)
         return 0;
     if (ap.P <= free_sms)
@@ -1068,12 +1072,13 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
     lt.ent_t = tr.ent_t;
     lt.logits_out = logits;
     a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
+    const int lm_sms = a.max_ctas > 0 ? lm_sms_beside_attn(lplan) : 0;
     // the structure of verify_step, with the walk between the LM head and the compaction
     StepStreams ss(bank, s, a.max_ctas > 0);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
-    if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, kPartBase + attn_bytes,
-                         ss.lm_stream(), fn, 0, &lt, ss.lm_pdl())) != TB_OK)
+    if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, workspace_bytes,
+                         kPartBase + attn_bytes, ss.lm_stream(), fn, 0, &lt, ss.lm_pdl(), lm_sms)) != TB_OK)
         return st;
     if ((st = ss.before_accept(fn)) != TB_OK)
         return st;
@@ -1149,12 +1154,13 @@ static tb_status verify_step_impl(const tb_bank *bank, int bank_id, const tb_kv 
     }
     // the step's structure: see StepStreams
     a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
+    const int lm_sms = a.max_ctas > 0 ? lm_sms_beside_attn(lplan) : 0;
     StepStreams ss(bank, s, a.max_ctas > 0);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
-    if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, kPartBase + attn_bytes,
-                         ss.lm_stream(), fn, (flags & TB_DEBUG_EXPIRE_WAIT) ? 1 : 0, typ ? &lt : nullptr,
-                         ss.lm_pdl())) != TB_OK)
+    if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, workspace_bytes,
+                         kPartBase + attn_bytes, ss.lm_stream(), fn, (flags & TB_DEBUG_EXPIRE_WAIT) ? 1 : 0,
+                         typ ? &lt : nullptr, ss.lm_pdl(), lm_sms)) != TB_OK)
         return st;
     if ((st = ss.before_accept(fn)) != TB_OK)
         return st;
@@ -1307,8 +1313,8 @@ static tb_status verify_step_batched_impl(const tb_bank *bank, int batch, const 
         }
         // the chunks share the partials and counters: only the first overlaps the attention
         if ((st = lm_enqueue(h8 + (size_t)r0 * d_model * 2, rc, lm_head, d_model, vocab, argmax + r0, top1 + r0,
-                             entropy + r0, ws, kPartBase + attn_bytes, ss.lm_stream(), fn, 0, typ ? &lt : nullptr,
-                             ss.lm_pdl() && r0 == 0)) != TB_OK)
+                             entropy + r0, ws, workspace_bytes, kPartBase + attn_bytes, ss.lm_stream(), fn, 0,
+                             typ ? &lt : nullptr, ss.lm_pdl() && r0 == 0)) != TB_OK)
             return st;
     }
     if ((st = ss.before_accept(fn)) != TB_OK)
@@ -1474,7 +1480,7 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
         if (e != cudaSuccess)
             return cuda_fail(e, fn);
         if ((st = lm_enqueue(hidden, N_max, lm_head, d_model, vocab, argmax, top1, entropy, ws,
-                             kPartBase + attn_bytes, ss.lm_stream(), fn, 0, nullptr, ss.lm_pdl())) != TB_OK)
+                             workspace_bytes, kPartBase + attn_bytes, ss.lm_stream(), fn, 0, nullptr, ss.lm_pdl())) != TB_OK)
             return st;
         if ((st = ss.merge(fn, false)) != TB_OK)
             return st;
