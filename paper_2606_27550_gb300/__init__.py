@@ -139,23 +139,41 @@ def load(path: str = LIB_PATH):
 
 
 def _check(rc: int, where: str):
-    if rc != TB_OK:
+    if rc:
         raise TreeVerifyError(rc, where, load().tb_last_error().decode())
 
 
 def _ptr(t) -> int | None:
-    if t is None:
-        return None
-    if isinstance(t, np.ndarray):
-        return t.ctypes.data
-    return t.data_ptr()
+    try:
+        return t.data_ptr()  # a tensor, on every call's path: no checks first
+    except AttributeError:
+        return None if t is None else t.ctypes.data
+
+
+_current_stream = None
+
+
+def _find_current_stream():
+    """A function that returns the raw handle of torch's current stream: torch's
+    own raw getter where it has one (a Stream object per call costs 1 us)."""
+    import torch
+
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None or not torch.cuda.is_initialized():
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
 
 
 def _stream(stream) -> int | None:
     if stream is None:
-        import torch
+        global _current_stream
+        if _current_stream is None:
+            import torch
 
-        return torch.cuda.current_stream().cuda_stream
+            torch.cuda.current_stream()  # initialises CUDA, as the getter expects
+            _current_stream = _find_current_stream()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -234,9 +252,10 @@ class KvCache:
     rope_theta: float = 0.0  # > 0: the call rotary-embeds q and the tree keys at L + depth
 
     def as_c(self) -> TbKv:
-        n_layers, n_kv_heads, L_cap, head_dim = self.k.shape
-        s = self.k.stride()
-        return TbKv(self.k.data_ptr(), self.v.data_ptr(), s[0], s[1], n_layers, n_kv_heads, head_dim, self.L, L_cap,
+        k = self.k
+        n_layers, n_kv_heads, L_cap, head_dim = k.shape
+        s = k.stride()
+        return TbKv(k.data_ptr(), self.v.data_ptr(), s[0], s[1], n_layers, n_kv_heads, head_dim, self.L, L_cap,
                     float(self.rope_theta))
 
 

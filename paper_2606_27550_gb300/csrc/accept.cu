@@ -70,8 +70,11 @@ __device__ __forceinline__ void copy_rows(uint8_t *base, const int *path, int k,
     }
 }
 
+// One launch's sequences: a launch of one sequence passes one entry's worth of
+// parameters.
+template <int kSeqs>
 struct AcceptBatch {
-    AcceptParams seq[TB_MAX_BATCH];
+    AcceptParams seq[kSeqs];
 };
 
 // A warp's registers with the tree of a step: lane l holds nodes l and l + 32
@@ -168,7 +171,8 @@ __device__ void policy_step(const AcceptParams &p, int rung, int L, int len, int
 }
 
 // blockIdx.y selects the sequence; every CTA of a sequence recomputes its acceptance.
-__global__ void __launch_bounds__(256) k3_accept_compact(const __grid_constant__ AcceptBatch pb)
+template <int kSeqs>
+__global__ void __launch_bounds__(256) k3_accept_compact(const __grid_constant__ AcceptBatch<kSeqs> pb)
 {
     const AcceptParams &p = pb.seq[blockIdx.y];
     __shared__ int s_path[kMaxNodes];
@@ -396,10 +400,8 @@ cudaError_t accept_launch_batch(const AcceptParams *ps, int n, int n_sm, cudaStr
 {
     if (n < 1 || n > TB_MAX_BATCH)
         return cudaErrorInvalidValue;
-    AcceptBatch pb{};
     int grid = 1;
-    for (int b = 0; b < n; ++b) {
-        pb.seq[b] = ps[b];
+    for (int b = 0; b < n; ++b)
         if (ps[b].n_layers > 0) {
             const int units = ps[b].n_layers * ps[b].n_kv_heads * 2;
             int gx = (units + 7) / 8;
@@ -409,8 +411,17 @@ cudaError_t accept_launch_batch(const AcceptParams *ps, int n, int n_sm, cudaStr
             if (gx > grid)
                 grid = gx;
         }
+    if (n == 1) {
+        AcceptBatch<1> one;
+        one.seq[0] = ps[0];
+        return launch_kernel(k3_accept_compact<1>, dim3(grid), dim3(256), 0, stream, pdl, one);
     }
-    return launch_kernel(k3_accept_compact, dim3(grid, n), dim3(256), 0, stream, pdl, pb);
+    AcceptBatch<TB_MAX_BATCH> pb;
+    for (int b = 0; b < n; ++b)
+        pb.seq[b] = ps[b];
+    for (int b = n; b < TB_MAX_BATCH; ++b)
+        pb.seq[b] = AcceptParams{};
+    return launch_kernel(k3_accept_compact<TB_MAX_BATCH>, dim3(grid, n), dim3(256), 0, stream, pdl, pb);
 }
 
 cudaError_t accept_launch(const AcceptParams &p, int n_sm, cudaStream_t stream, bool pdl)

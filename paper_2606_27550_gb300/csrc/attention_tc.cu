@@ -106,9 +106,7 @@ struct TcSeq {
     int nstride;             // nodes per layer in q / out (N, or the largest tree of a scheduled loop)
 };
 
-struct TcParams {
-    CUtensorMap tmap[2 * kMaxSeqPerLaunch];  // K, V of each sequence: (head_dim, L + N, Hkv, layers), box (64, 128, 1, 1)
-    TcSeq seq[kMaxSeqPerLaunch];
+struct TcCommon {
     int n_seq, Hq, Hkv, group, layer_begin;
     long long total;
     int P;
@@ -129,6 +127,18 @@ struct TcParams {
     const float2 *rope_tab;
 };
 
+// The launch's parameters for up to kSeqs sequences.  A launch of one sequence
+// passes 0.5 KB of them rather than 5.4: every launch copies its parameters to
+// the device.
+template <int kSeqs>
+struct TcParamsOf : TcCommon {
+    CUtensorMap tmap[2 * kSeqs];  // K, V of each sequence: (head_dim, L + N, Hkv, layers), box (64, 128, 1, 1)
+    TcSeq seq[kSeqs];
+};
+using TcParams = TcParamsOf<kMaxSeqPerLaunch>;
+template <bool kBatched>
+using TcKernelParams = TcParamsOf<kBatched ? kMaxSeqPerLaunch : 1>;
+
 // Two row blocks per kv head (grouped queries, 129 to 256 rows) and more than a
 // wave of tiles: neighbouring CTAs walk the same key tiles side by side, one
 // row block each, so that the second reading of a tile comes from L2.  As units
@@ -143,9 +153,9 @@ __host__ __device__ inline bool split_rows(int row_blocks, long long total, int 
 // Scheduled mode: the sequence of this step from the device state.  An
 // out-of-range rung or a prefix that does not fit the cache gives no work
 // (the acceptance kernel reports it).
-__device__ void sched_plan(const TcParams &p, TcSeq *sq, long long *total)
+__device__ void sched_plan(const TcCommon &p, const TcSeq &first, TcSeq *sq, long long *total)
 {
-    *sq = p.seq[0];
+    *sq = first;
     sq->tile_base = 0;
     const int rung = p.sched[0], L = p.sched[1];
     const bool ok = rung >= 0 && rung < p.n_rungs && L >= 0;
@@ -165,7 +175,7 @@ __device__ void sched_plan(const TcParams &p, TcSeq *sq, long long *total)
 // Sequence holding flattened tile t, searching forward from `b` (tiles are
 // visited in increasing order by every role).  kBatched = false: sequence 0.
 template <bool kBatched>
-__device__ __forceinline__ int seq_at(const TcParams &p, long long t, int b)
+__device__ __forceinline__ int seq_at(const TcKernelParams<kBatched> &p, long long t, int b)
 {
     if constexpr (!kBatched) {
         return 0;
@@ -182,7 +192,7 @@ __device__ __forceinline__ int seq_at(const TcParams &p, long long t, int b)
 // a step with fewer tiles than that splits them over its first `total` CTAs
 // only (the others get nothing), so that no CTA range inside the split is
 // empty: the split merge combines the partials of consecutive CTAs.
-__device__ __forceinline__ int tc_split_ctas(const TcParams &p, long long total, int row_split)
+__device__ __forceinline__ int tc_split_ctas(const TcCommon &p, long long total, int row_split)
 {
     const int n = p.P / row_split;
     return (p.sched && total < n) ? (int)(total > 0 ? total : 1) : n;
@@ -239,7 +249,7 @@ struct SegPos {
 };
 
 template <bool kBatched>
-__device__ __forceinline__ SegPos seg_at(const TcParams &p, const TcSeq *seqs, long long t, long long t1, int b)
+__device__ __forceinline__ SegPos seg_at(const TcKernelParams<kBatched> &p, const TcSeq *seqs, long long t, long long t1, int b)
 {
     SegPos g;
     g.b = seq_at<kBatched>(p, t, b);
@@ -284,7 +294,7 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr)
 // second kernel.  For problems small enough that all their clusters run at
 // once (attn_tc_clusters).
 template <int kD, bool kBatched, bool kCluster>
-__global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __grid_constant__ TcParams p)
+__global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __grid_constant__ TcKernelParams<kBatched> p)
 {
     static_assert(kD == 64 || kD == 128, "head_dim 64 or 128");
     constexpr int kTile = tile_bytes(kD);
@@ -344,7 +354,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     long long total = p.total;
     if (p.sched) {
         if (threadIdx.x == 0)
-            sched_plan(p, &s_seq, &s_total);
+            sched_plan(p, p.seq[0], &s_seq, &s_total);
         __syncthreads();
         seqs = &s_seq;
         total = s_total;
@@ -950,7 +960,7 @@ struct ColVec<2> {
 };
 
 template <int kD, bool kBatched, bool kAfterStep>
-__global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__ TcParams p)
+__global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__ TcKernelParams<kBatched> p)
 {
     constexpr int kSlot = slot_floats(kD);
     constexpr int kCpl = kD / 32;  // output columns per lane
@@ -965,7 +975,7 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
     long long total = p.total;
     if (p.sched) {
         if (threadIdx.x == 0)
-            sched_plan(p, &s_seq, &s_total);
+            sched_plan(p, p.seq[0], &s_seq, &s_total);
         __syncthreads();
         seqs = &s_seq;
         total = s_total;
@@ -1071,6 +1081,17 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
 // ----------------------------------------------------------------------------
 // host side
 
+// The parameters of a launch of one sequence.
+static TcKernelParams<false> one_seq(const TcParams &p)
+{
+    TcKernelParams<false> q;
+    static_cast<TcCommon &>(q) = p;
+    q.tmap[0] = p.tmap[0];
+    q.tmap[1] = p.tmap[1];
+    q.seq[0] = p.seq[0];
+    return q;
+}
+
 // The split-unit merge of an attention launch with parameters p, for head_dim
 // kD.  after_step: see k1_merge_split.
 template <int kD>
@@ -1081,8 +1102,8 @@ static cudaError_t merge_launch_d(const TcParams &p, bool batched, cudaStream_t 
     if (batched)
         return after_step ? launch_kernel(k1_merge_split<kD, true, true>, grid, dim3(256), 0, stream, pdl, p)
                           : launch_kernel(k1_merge_split<kD, true, false>, grid, dim3(256), 0, stream, pdl, p);
-    return after_step ? launch_kernel(k1_merge_split<kD, false, true>, grid, dim3(256), 0, stream, pdl, p)
-                      : launch_kernel(k1_merge_split<kD, false, false>, grid, dim3(256), 0, stream, pdl, p);
+    return after_step ? launch_kernel(k1_merge_split<kD, false, true>, grid, dim3(256), 0, stream, pdl, one_seq(p))
+                      : launch_kernel(k1_merge_split<kD, false, false>, grid, dim3(256), 0, stream, pdl, one_seq(p));
 }
 
 // Whether a CTA range of the launch starts inside a unit (the split merge then
@@ -1126,8 +1147,12 @@ static cudaError_t attn_kernel_launch_d(const TcParams &p, cudaStream_t stream, 
     cudaError_t e;
     if ((e = allow_max_smem((const void *)k1_tree_attention_tc<kD, kBatched, kCluster>)) != cudaSuccess)
         return e;
-    return launch_kernel_cluster(k1_tree_attention_tc<kD, kBatched, kCluster>, dim3(p.P), dim3(kTcThreads),
-                                 attn_smem(kD), stream, pdl, kCluster ? p.cluster : 1, p);
+    if constexpr (kBatched)
+        return launch_kernel(k1_tree_attention_tc<kD, true, false>, dim3(p.P), dim3(kTcThreads), attn_smem(kD), stream,
+                             pdl, p);
+    else
+        return launch_kernel_cluster(k1_tree_attention_tc<kD, false, kCluster>, dim3(p.P), dim3(kTcThreads),
+                                     attn_smem(kD), stream, pdl, kCluster ? p.cluster : 1, one_seq(p));
 }
 
 static cudaError_t attn_kernel_launch(const TcParams &p, bool batched, cudaStream_t stream, bool pdl)

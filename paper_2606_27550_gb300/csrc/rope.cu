@@ -25,6 +25,7 @@
 // The queries are rotated inside the attention kernel as they are staged
 // into tensor memory (attention_tc.cu), with the same table.
 #include <cuda_bf16.h>
+#include <string.h>
 
 #include "kernels.cuh"
 
@@ -112,8 +113,16 @@ __global__ void __launch_bounds__(kRopeThreads) k0_rope_tree_k(const __grid_cons
 
 void rope_inv_freq(double theta, int d, double *inv_freq)
 {
-    for (int i = 0; i < d / 2; ++i)
-        inv_freq[i] = pow((double)theta, -2.0 * i / d);
+    // the table of the thread's last (theta, d): a model's never change
+    static thread_local double last_theta = 0.0, last[kRopeMaxHalf];
+    static thread_local int last_d = 0;
+    if (theta != last_theta || d != last_d) {
+        for (int i = 0; i < d / 2; ++i)
+            last[i] = pow(theta, -2.0 * i / d);
+        last_theta = theta;
+        last_d = d;
+    }
+    memcpy(inv_freq, last, sizeof(double) * (d / 2));
 }
 
 cudaError_t rope_launch(const RopeParams &p, int n_seq, int max_nodes, int n_layers, cudaStream_t stream)

@@ -102,3 +102,24 @@ def test_threads_share_a_bank(dev, d, structure, Hkv, L):
         assert np.array_equal(bits(wk["k"]), oracle.kv_compact(c.k, L, path))
         assert np.array_equal(bits(wk["v"]), oracle.kv_compact(c.v, L, path))
     bank.close()
+
+
+def test_calls_without_a_stream_take_the_threads_current_one():
+    """stream=None is torch's current stream of the calling thread and device,
+    whichever streams other threads have made current."""
+    seen = {}
+
+    def work(name, stream):
+        with torch.cuda.stream(stream):
+            seen[name] = (tv._stream(None), stream.cuda_stream)
+
+    torch.cuda.set_device(0)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    threads = [threading.Thread(target=work, args=(i, s)) for i, s in enumerate(streams)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert len(seen) == 3 and all(a == b for a, b in seen.values())
+    assert tv._stream(None) == torch.cuda.current_stream().cuda_stream
+    assert tv._stream(streams[0]) == streams[0].cuda_stream and tv._stream(5) == 5
