@@ -270,24 +270,6 @@ struct SegInfo {
     float m[128], l[128];      // written back by the softmax: reference maximum (log2 units) and sum of each row
 };
 
-// Loads from the shared memory of any CTA of the cluster.
-__device__ __forceinline__ float ld_cluster_f32(uint32_t addr)
-{
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr)
-{
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(addr)
-                 : "memory");
-    return v;
-}
-
 // kCluster: the p.cluster CTAs of a cluster share one unit's key tiles, leave
 // their (O, m, l) in shared memory and combine them there (log-sum-exp, in rank
 // order), every CTA a share of the rows: no partials in global memory and no

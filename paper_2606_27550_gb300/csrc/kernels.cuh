@@ -55,6 +55,7 @@ struct LmPlan {
     int R_pad, n_tiles, n_kblocks, stages, acc_cols;
     int tile_rows;    // vocab entries per tile and CTA
     int ctas_per_sm;  // 2 when two rings fit side by side, else 1
+    int split;        // > 1: clusters of that many CTAs share each tile's k-blocks
     bool pair;        // CTA pairs share each MMA (M = 256); tiles are then 256 vocab entries
     int units;        // the tile split's units: CTAs, or CTA pairs
     int P;            // persistent CTAs: ctas_per_sm per SM, at most one per vocab tile (two per pair tile)

@@ -39,6 +39,8 @@ struct LmParams {
     CUtensorMap tmap_h;  // (d_model, rows),  box (64, R_pad) (R_pad / 2 for CTA pairs), 128B swizzle
     int R, R_pad, D, V;
     int n_tiles, nk, stages, acc_cols;
+    int split;           // > 1: a cluster of that many CTAs shares each tile's k-blocks (k2_lm_head_split)
+    int w_once;          // W is too large to stay in L2 from call to call: loaded evict-first
     int tile_rows;       // vocab entries per tile and CTA: up to 128 (128 in a pair, whose tiles are two of them)
     int units;           // the tile split's units: CTAs, or CTA pairs
     int n_slots;         // per-tile partials: one per tile (two per pair tile, one per CTA)
@@ -285,7 +287,8 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
             uint32_t ph = 0;
             long long g = 0;    // the current tile's first k-block in the CTA's sequence
             long long g_end = 0;
-            const uint64_t w_policy = l2_evict_first();  // W is read once: it should not push out what is reused
+            // a W that cannot stay in L2 should not push out what is reused
+            const uint64_t w_policy = p.w_once ? l2_evict_first() : l2_evict_normal();
             bool ok = true;
             // tile scheduler (warp 0 of the even CTA): entry i + 1 of the queue is
             // published while tile i streams; its tile was fetched a tile earlier
@@ -605,6 +608,189 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
     }
 }
 
+// The LM head of a small vocabulary: a cluster of p.split CTAs shares each
+// vocab tile, every CTA a run of the tile's k-blocks.  With a whole tile per CTA
+// a vocabulary of fewer tiles than SMs leaves the others idle, and one CTA
+// streams W at about 47 GB/s however deep its ring (1 MB of a 128 x 4096 tile in
+// 22 us).  Each CTA accumulates its part of the 128 x R_pad logits in TMEM and
+// leaves it in shared memory; then rank k adds, in rank order, and reduces the
+// rows k, k + split, ..: one warp per row, four logits per lane.  Same partials
+// as k2_lm_head, merged by k2_lm_merge.
+// lm_head_stats, whole tiles / split: 26 rows x 4096 at V 1000 25.3 / 10.4 us, V
+// 4000 25.7 / 13.0, V 16000 30.5 / 28.8; 200 rows at V 3000 33.0 / 28.7.
+//   warps 0, 2   TMA producers (alternate stages); warp 1 TMEM and the MMAs;
+//   then all eight warps: TMEM -> shared memory, and the rows.
+constexpr int kSplitThreads = 256;
+constexpr int kMaxSplit = 8;
+constexpr int kSplitLd = 132;  // row stride of the parts in shared memory (floats): 16-byte rows, conflict-free writes
+
+template <bool kTyp>
+__global__ void __launch_bounds__(kSplitThreads, 2) k2_lm_head_split(const __grid_constant__ LmParams p)
+{
+    // the kernel that reads this one's outputs may be launched now
+    pdl_trigger();
+    PdlWaitOnExit pdl_exit;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[8], empty_bar[8];
+    __shared__ __align__(8) uint64_t acc_full, never_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+
+    uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    float *parts = reinterpret_cast<float *>(ring);  // [R_pad][kSplitLd], once the ring is drained
+    const int S = p.stages;
+    const uint32_t stage_bytes = 16384u + (uint32_t)p.R_pad * 128u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n_cta = p.split, tile = blockIdx.x / n_cta, rank = blockIdx.x % n_cta;
+    const int k0 = p.nk * rank / n_cta, n_k = p.nk * (rank + 1) / n_cta - k0;  // at least one k-block each
+    const uint32_t cols = (uint32_t)p.acc_cols;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full_bar[s], 1);
+            mbar_init(&empty_bar[s], 1);
+        }
+        mbar_init(&acc_full, 1);
+        mbar_init(&never_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&p.tmap_w);
+        prefetch_tmap(&p.tmap_h);
+    }
+    if (warp == 1) {
+        tmem_alloc(&tmem_slot, cols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    int issued = 0;  // k-blocks up to the last one this thread loaded
+    if ((warp == 0 || warp == 2) && lane == 0) {
+        const int mine = warp >> 1;
+        const uint64_t w_policy = p.w_once ? l2_evict_first() : l2_evict_normal();
+        for (int it = mine; it < n_k; it += 2) {
+            const int s = it % S;
+            if (!mbar_wait_bounded(&empty_bar[s], ((uint32_t)(it / S) & 1u) ^ 1u, &abort_flag, p.status))
+                break;
+            uint8_t *dst = ring + (size_t)s * stage_bytes;
+            mbar_arrive_expect_tx(&full_bar[s], stage_bytes);
+            tma_load_2d_hint(dst, &p.tmap_w, &full_bar[s], (k0 + it) * 64, tile * 128, w_policy);
+            tma_load_2d(dst + 16384, &p.tmap_h, &full_bar[s], (k0 + it) * 64, 0);
+            issued = it + 1;
+        }
+    } else if (warp == 1 && lane == 0) {
+        const uint32_t idesc = idesc_bf16_f32(128, p.R_pad);
+        for (int j = 0; j < n_k; ++j) {
+            const int s = j % S;
+            if (!mbar_wait_bounded(&full_bar[s], (uint32_t)(j / S) & 1u, &abort_flag, p.status))
+                break;
+            tc_fence_after();
+            const uint32_t a_base = smem_u32(ring + (size_t)s * stage_bytes);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                tc_mma_f16_ss(tmem, smem_desc_sw128(a_base + k * 32, 0, 1024),
+                              smem_desc_sw128(a_base + 16384u + k * 32, 0, 1024), idesc, (j != 0 || k != 0) ? 1u : 0u);
+            tc_commit(&empty_bar[s]);
+        }
+        tc_commit(&acc_full);  // arrives when every MMA issued above has retired
+    }
+    __syncwarp();
+    mbar_wait_bounded(p.expire_wait ? &never_bar : &acc_full, 0, &abort_flag, p.status);
+    __syncthreads();  // every role is done; its verdict is the same for all threads from here on
+    const bool ok = abort_flag == 0;
+    if (!ok) {
+        // given up: MMAs in flight retire before TMEM is freed, and copies in
+        // flight land before the CTA exits
+        if (threadIdx.x == 32)
+            mbar_wait_drain(&acc_full, 0);
+        for (int it = issued > S ? issued - S : 0; it < issued; ++it)
+            if ((it & 1) == ((issued - 1) & 1))
+                mbar_wait_drain(&full_bar[it % S], (uint32_t)(it / S) & 1u);
+    }
+    tc_fence_after();
+    if (ok) {
+        // 16 tree rows at a time, this thread's vocab entry of the tile
+        const int q = warp & 3, vr = 32 * q + lane;
+        for (int c0 = 16 * (warp >> 2); c0 < p.R_pad; c0 += 32) {
+            uint32_t v[16];
+            tmem_ld_32x32b_x16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                parts[(c0 + j) * kSplitLd + vr] = __uint_as_float(v[j]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, cols);
+    }
+    cluster_barrier();  // every CTA's part is in its shared memory
+    if (ok) {
+        const int v0 = tile * 128, nvalid = min(128, p.V - v0);
+        const uint32_t parts_addr = smem_u32(parts);
+        for (int r = rank + n_cta * warp; r < p.R; r += n_cta * (kSplitThreads / 32)) {
+            const uint32_t addr = parts_addr + (uint32_t)(r * kSplitLd + 4 * lane) * 4;
+            float4 part[kMaxSplit];
+#pragma unroll
+            for (int k = 0; k < kMaxSplit; ++k)
+                if (k < n_cta)
+                    part[k] = ld_cluster_f32x4(cluster_map(addr, k));
+            float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < kMaxSplit; ++k)
+                if (k < n_cta)
+                    z[0] += part[k].x, z[1] += part[k].y, z[2] += part[k].z, z[3] += part[k].w;
+            RowStat st = stat_empty();
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (4 * lane + x < nvalid && z[x] > st.m) {
+                    st.m = z[x];
+                    st.idx = v0 + 4 * lane + x;
+                }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (4 * lane + x < nvalid) {
+                    const float dz = z[x] - st.m;
+                    const float ex = ex2_approx(dz * kLog2e);
+                    st.s += ex;
+                    st.t += ex * dz;
+                    if constexpr (kTyp) {
+                        const float dT = dz * p.inv_t;
+                        const float eT = ex2_approx(dT * kLog2e);
+                        st.sT += eT;
+                        st.tT += eT * dT;
+                    }
+                }
+            st = group_merge<kTyp>(st, 32, p.inv_t);
+            if (lane == 0) {
+                p.part_tile[(size_t)tile * p.R_pad + r] = stat_pack(st);
+                if constexpr (kTyp)
+                    p.part_tile_t[(size_t)tile * p.R_pad + r] = make_float2(st.sT, st.tT);
+            }
+            if constexpr (kTyp) {
+                // the row's logits, over this CTA's part of them (which only this warp reads)
+                float *row = parts + r * kSplitLd;
+                *reinterpret_cast<float4 *>(row + 4 * lane) = make_float4(z[0], z[1], z[2], z[3]);
+                __syncwarp();
+                for (int bq = 0; bq < p.gather.n_seq; ++bq)
+                    for (int j = 1 + lane; j < p.gather.seq[bq].n; j += 32) {
+                        int er, ec;
+                        if (gather_hit(p.gather, bq, j, p.R, v0, nvalid, &er, &ec) && er == r)
+                            p.gather.seq[bq].out[j] = row[ec];
+                    }
+                if (p.logits_out)
+                    for (int j = lane; j < nvalid; j += 32)
+                        p.logits_out[(size_t)r * p.V + v0 + j] = row[j];
+            }
+        }
+    }
+    cluster_barrier();  // no CTA leaves while another reads its shared memory
+}
+
 // Final merge of the per-tile partials (K2 merge): one CTA per tree row.
 // Thread k folds slots k, k + 256, ... in order -- the row's maximum and its
 // lowest vocab index first, then the sums rescaled to that maximum -- and the
@@ -775,15 +961,28 @@ LmPlan lm_plan(int R, int D, int V, int n_sm, size_t parts_bytes, int max_pairs)
     const int st2 = half > fixed + pad ? (int)((half - fixed - pad) / stage1) : 0;
     const bool two = st2 >= 3 && 4 * cols <= 512;
     // Over many rounds of tiles one CTA with a ring twice as deep is faster: 26
-    // rows x 4096, V 128256 160 us against 166, V 100000 x 1024 39.5 against
-    // 40.0; V 80000 108 against 106, V 32000 51 against 46.
-    pl.ctas_per_sm = two && ceil_div(V, 128) <= 5 * n_sm ? 2 : 1;
+    // rows x 4096, V 128256 160 us against 166; V 103787 (13 rows) 137 against
+    // 135 with two, V 80000 108 against 106, V 32000 51 against 46.
+    pl.ctas_per_sm = two && ceil_div(V, 128) <= 6 * n_sm ? 2 : 1;
     // Otherwise (wide rows, one CTA per SM) CTA pairs share each MMA: each CTA
     // stages half of the rows, so the rows cross each SM's shared memory once
     // per 256 vocab entries instead of once per 128.
     if (max_pairs < 0)
         max_pairs = n_sm / 2;
     pl.pair = !two && max_pairs >= 1;
+    // Fewer tiles than CTA slots: clusters share each tile, with at least eight
+    // k-blocks per CTA, sixteen for wide rows (under that, the exchange costs more
+    // than it saves: 232 rows x 1024, V 5000 21.7 us split in two against 20.2).
+    const int tiles1 = ceil_div(V, 128);
+    int split = (two ? 2 : 1) * n_sm / tiles1;
+    split = split < kMaxSplit ? split : kMaxSplit;
+    const int most = pl.n_kblocks / (two ? 8 : 16);
+    split = split < most ? split : most;
+    pl.split = split > 1 ? split : 1;
+    if (pl.split > 1) {
+        pl.pair = false;
+        pl.ctas_per_sm = two ? 2 : 1;
+    }
     const size_t stage_bytes = 16384 + (size_t)(pl.pair ? pl.R_pad / 2 : pl.R_pad) * 128;
     const size_t budget = (pl.ctas_per_sm == 2 ? half : 227 * 1024) - fixed - pad;
     pl.stages = (int)(budget / stage_bytes);
@@ -791,11 +990,13 @@ LmPlan lm_plan(int R, int D, int V, int n_sm, size_t parts_bytes, int max_pairs)
         pl.stages = 8;
     if (pl.stages < 2)
         pl.stages = 2;
+    if (pl.split > 1 && pl.stages > ceil_div(pl.n_kblocks, pl.split))
+        pl.stages = ceil_div(pl.n_kblocks, pl.split);
     // tiles of 128 vocab entries (256 for a pair)
     pl.tile_rows = 128;
     pl.n_tiles = ceil_div(V, pl.pair ? 256 : 128);
     const int slots = pl.pair ? max_pairs : pl.ctas_per_sm * n_sm;
-    if (!pl.pair) {
+    if (!pl.pair && pl.split == 1) {
         // Lower tiles where they spread several rounds of the vocabulary evenly over
         // the CTAs, in as many rounds as 128-entry tiles take, and the workspace has
         // room for their partials: V 40000 59 us against 72, V 80000 106 against
@@ -811,9 +1012,17 @@ LmPlan lm_plan(int R, int D, int V, int n_sm, size_t parts_bytes, int max_pairs)
     }
     pl.units = slots < pl.n_tiles ? slots : pl.n_tiles;
     pl.P = pl.pair ? 2 * pl.units : pl.units;
+    if (pl.split > 1) {
+        pl.units = pl.n_tiles;
+        pl.P = pl.n_tiles * pl.split;
+    }
     // per-tile partials: one per tile and CTA, merged by k2_lm_merge
     pl.n_slots = pl.pair ? 2 * pl.n_tiles : pl.n_tiles;
     pl.smem_bytes = (size_t)pl.stages * stage_bytes + fixed + 1024;
+    if (pl.split > 1) {
+        const size_t ring = (size_t)pl.stages * stage_bytes, parts = (size_t)pl.R_pad * kSplitLd * 4;
+        pl.smem_bytes = (ring > parts ? ring : parts) + 1024;
+    }
     pl.n_counters = 1;  // the tile counter
     // What a call needs: the partials of 128-entry tiles (two per pair tile), or
     // of the plan without pairs, which a launch takes when no cluster of two can
@@ -866,7 +1075,12 @@ template <bool kTyp>
 static cudaError_t lm_launch_as(LmParams &p, const LmPlan &pl, cudaStream_t stream, bool pdl)
 {
     cudaError_t e;
-    if (pl.pair) {
+    if (pl.split > 1) {
+        if ((e = allow_max_smem((const void *)k2_lm_head_split<kTyp>)) != cudaSuccess)
+            return e;
+        e = launch_kernel_cluster(k2_lm_head_split<kTyp>, dim3(pl.P), dim3(kSplitThreads), pl.smem_bytes, stream, pdl,
+                                  pl.split, p);
+    } else if (pl.pair) {
         if ((e = allow_max_smem((const void *)k2_lm_head<kTyp, true>)) != cudaSuccess)
             return e;
         e = launch_kernel_cluster(k2_lm_head<kTyp, true>, dim3(pl.P), dim3(kLmThreads), pl.smem_bytes, stream, pdl,
@@ -905,6 +1119,11 @@ cudaError_t lm_head_launch(const void *hidden, int R, const void *W, int D, int 
     p.V = V;
     p.n_tiles = pl.n_tiles;
     p.tile_rows = pl.tile_rows;
+    p.split = pl.split;
+    // Half of the 129 MB L2: a smaller W is still there at the next step (a 10 MB
+    // one loaded evict-first made a scheduled step 30.3 -> 32.1 us; 262 MB evict-first
+    // made a 7B layer's step 57.3 -> 55.3 us).
+    p.w_once = (size_t)V * D * 2 > ((size_t)64 << 20);
     p.nk = pl.n_kblocks;
     p.stages = pl.stages;
     p.acc_cols = pl.acc_cols;

@@ -974,14 +974,12 @@ extern "C" tb_status typical_accept(const tb_bank *bank, int bank_id, const int3
 // size and the step runs as the same chain: both start at once, and the
 // programmatic launches hide the launch latencies (the tiny step: 60-65 k
 // verify-steps/s against 47-57 k with the LM head forked).  0: no cap.
-static int lm_sms_beside_attn(const LmPlan &lp)
-{
-    return (lp.P + lp.ctas_per_sm - 1) / lp.ctas_per_sm;
-}
-
 static int attn_ctas_beside_lm(const AttnPlan &ap, const LmPlan &lp, int d_model, int vocab, int n_sm)
 {
-    const int free_sms = n_sm - lm_sms_beside_attn(lp);
+    // the SMs a round of one 128-entry tile per CTA takes; the LM head then gets
+    // all that the attention leaves (clusters share the tiles of a small vocabulary)
+    const int lm_ctas = lp.pair ? lp.P : (vocab + 127) / 128;
+    const int free_sms = n_sm - (lm_ctas + lp.ctas_per_sm - 1) / lp.ctas_per_sm;
     if (free_sms < 1 || ap.total < 1)
         return 0;
     if (ap.P <= free_sms)
@@ -1072,7 +1070,7 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
     lt.ent_t = tr.ent_t;
     lt.logits_out = logits;
     a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
-    const int lm_sms = a.max_ctas > 0 ? lm_sms_beside_attn(lplan) : 0;
+    const int lm_sms = a.max_ctas > 0 ? sm_count(bank->device) - a.max_ctas : 0;
     // the structure of verify_step, with the walk between the LM head and the compaction
     StepStreams ss(bank, s, a.max_ctas > 0);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
@@ -1154,7 +1152,7 @@ static tb_status verify_step_impl(const tb_bank *bank, int bank_id, const tb_kv 
     }
     // the step's structure: see StepStreams
     a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
-    const int lm_sms = a.max_ctas > 0 ? lm_sms_beside_attn(lplan) : 0;
+    const int lm_sms = a.max_ctas > 0 ? sm_count(bank->device) - a.max_ctas : 0;
     StepStreams ss(bank, s, a.max_ctas > 0);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
