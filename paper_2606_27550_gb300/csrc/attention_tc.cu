@@ -117,6 +117,7 @@ struct TcCommon {
     // device memory (sched[0] = rung into rung_tree, sched[1] = L) and every
     // CTA derives the work split itself; seq[0] carries q, out and nstride
     const int32_t *sched;
+    int32_t *sched_copy;  // the attention writes sched[0..1] here; the split merge's sched is this copy
     const TreeDesc *rung_tree[8];
     int n_rungs, n_layers, L_cap;
     int max_rows;  // rows the split merge's grid covers: of the largest row block, or of both (row_split)
@@ -337,6 +338,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     if (p.sched) {
         if (threadIdx.x == 0)
             sched_plan(p, p.seq[0], &s_seq, &s_total);
+        if (threadIdx.x == 32 && c == 0) {
+            p.sched_copy[0] = p.sched[0];
+            p.sched_copy[1] = p.sched[1];
+        }
         __syncthreads();
         seqs = &s_seq;
         total = s_total;
@@ -1183,7 +1188,9 @@ static int attn_max_clusters(int size)
 static void stash_merge(const TcParams &p, bool batched, AttnMerge *m)
 {
     static_assert(sizeof(TcParams) <= sizeof(m->params), "AttnMerge holds the attention launch's parameters");
-    memcpy(m->params, &p, sizeof p);
+    TcParams q = p;
+    q.sched = p.sched ? p.sched_copy : nullptr;
+    memcpy(m->params, &q, sizeof q);
     m->batched = batched;
     m->pending = any_split(p);
 }
@@ -1404,18 +1411,20 @@ cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *
     p.part = part;
     p.status = status;
     p.sched = sc.sched;
+    p.sched_copy = sc.sched_copy;
     p.rope_tab = sc.rope_tab;
     p.n_rungs = sc.n_rungs;
     for (int r = 0; r < sc.n_rungs; ++r)
         p.rung_tree[r] = sc.rung_tree[r];
     p.max_rows = sc.N_max * p.group;
     cudaError_t e;
-    if ((e = attn_kernel_launch(p, false, stream, false)) != cudaSuccess)
+    if ((e = attn_kernel_launch(p, false, stream, merge_later != nullptr)) != cudaSuccess)
         return e;
     if (merge_later) {
         stash_merge(p, false, merge_later);
         return cudaSuccess;
     }
+    p.sched = p.sched_copy;
     return merge_launch(p, false, stream, false, false);
 }
 

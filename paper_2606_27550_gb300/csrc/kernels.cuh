@@ -170,6 +170,8 @@ struct AttnSched {
     const TreeDesc *rung_tree[8];
     int n_rungs, N_max;
     const int32_t *sched;
+    int32_t *sched_copy;     // workspace: the attention leaves sched[0..1] here for the split-unit merge, which may
+                             // run beside the acceptance kernel that advances them
     const void *q;
     void *out;
     const float2 *rope_tab;  // null, or the rotary tables (pre-rotary queries)

@@ -154,7 +154,7 @@ bool make_tmap_kv(CUtensorMap *map, const void *base, int d, int n_keys, int n_h
 
 // ------------------------------------------------------------------ workspace layout
 //
-//   [0, 256)                    status word
+//   [0, 256)                    status word; scheduled steps: arrival ticket, copy of (rung, L)
 //   [256, 256 + 4 KiB)          LM-head counters (1024 int32; the tile counter)
 //   [.., + 12 KiB)              typical acceptance: logZ_T, H_T, draft logits (3 x 1024 float)
 //   [.., + 512 KiB)             rotary tables: (cos, sin) per (depth, pair), one per sequence
@@ -162,7 +162,8 @@ bool make_tmap_kv(CUtensorMap *map, const void *base, int d, int n_keys, int n_h
 // Counters sit at fixed offsets so that calls of different shapes sharing one
 // workspace always find them zero; partials are written before they are read.
 
-constexpr size_t kTicketOff = 128;  // scheduled acceptance: arrival ticket, inside the status page
+constexpr size_t kTicketOff = 128;     // scheduled acceptance: arrival ticket, inside the status page
+constexpr size_t kSchedCopyOff = 160;  // scheduled attention: the rung and prefix length it ran with
 // (layer, kv head, row block) units of one attention launch: keeps the
 // kernels' 32-bit unit indices in range
 constexpr int kMaxAttnUnits = 1 << 24;
@@ -775,12 +776,18 @@ tb_status tv::lm_validate(const void *hidden, int R, const void *W, int D, int V
     return TB_OK;
 }
 
+// n_sm: the SMs the launch may use (0: all).  forked: it runs in the tail of an
+// attention that holds the SMs, so its CTAs start at different times and take
+// tiles as they come: even tile heights, made for CTAs that start together,
+// only add tiles there (parts_bytes 0; a 5-layer step at V 63992 102.5 us against
+// 96.7).
 static tb_status lm_enqueue(const void *hidden, int R, const void *W, int D, int V, int32_t *am, float *t1, float *en,
                             uint8_t *ws, size_t ws_bytes, size_t part_off, cudaStream_t stream, const char *fn,
-                            int expire_wait = 0, const LmTypical *typ = nullptr, bool pdl = false, int n_sm = 0)
+                            int expire_wait = 0, const LmTypical *typ = nullptr, bool pdl = false, int n_sm = 0,
+                            bool forked = false)
 {
     const char *err = "";
-    cudaError_t e = lm_head_launch(hidden, R, W, D, V, am, t1, en, ws + part_off, ws_bytes - part_off,
+    cudaError_t e = lm_head_launch(hidden, R, W, D, V, am, t1, en, ws + part_off, forked ? 0 : ws_bytes - part_off,
                                    reinterpret_cast<int *>(ws + kLmCounterOff), reinterpret_cast<int *>(ws),
                                    n_sm > 0 ? n_sm : sm_count(current_device()), stream, &err, expire_wait, typ, pdl);
     if (e == cudaErrorInvalidValue && err[0])
@@ -961,32 +968,42 @@ extern "C" tb_status typical_accept(const tb_bank *bank, int bank_id, const int3
     return ok();
 }
 
-// The attention grid beside the LM head of the same step.  The attention's
-// persistent grid normally takes one CTA per SM, each holding the whole
-// register file, so the LM head (launched once every attention CTA has
-// started) runs on the SMs that attention CTAs release.  When the LM head is the longer of the two (a
-// single layer against a large vocabulary), the attention instead gets only
-// the SMs the LM head's CTAs leave free, and both run from the start.  That
-// pays when the attention on those SMs still ends well before the LM head:
-// about 3 us per 128-key tile a CTA walks plus 6 us, against the weight
-// bytes at 5 TB/s plus 8 us (measured on GB300 at 7B shapes).  An attention
-// grid that already fits beside the LM head (a small problem) keeps its own
-// size and the step runs as the same chain: both start at once, and the
-// programmatic launches hide the launch latencies (the tiny step: 60-65 k
-// verify-steps/s against 47-57 k with the LM head forked).  0: no cap.
-static int attn_ctas_beside_lm(const AttnPlan &ap, const LmPlan &lp, int d_model, int vocab, int n_sm)
+// The attention grid beside the LM head of the same step: how many SMs the
+// attention takes, the LM head running on the others from the start (the
+// chain, see StepStreams); 0: the attention takes every SM and the LM head
+// follows in its tail (the fork).
+//
+// Its persistent grid normally takes one CTA per SM, each holding the whole
+// register file, so the LM head runs on the SMs that attention CTAs release.
+// An attention grid that fits beside one round of the LM head's CTAs keeps its
+// own size: both start at once, and the programmatic launches hide the launch
+// latencies (the tiny step: 60-65 k verify-steps/s against 47-57 k forked).
+// Otherwise the SMs are divided so that neither waits long for the other, if
+// that ends sooner than the fork.  The estimates (us, measured on GB300 at 7B
+// shapes): an attention CTA beside the LM head takes about 2.2 per 128-key
+// tile, 1.4 with every SM its own, plus 6 to 10; the LM head streams at 6.3
+// MB/us, 0.05 on one SM.  One 7B layer, 288 tiles, against V 32000, attention on
+// 12 / 16 / 20 / 24 / 27 / 32 SMs: 52.0 / 49.0 / 51.8 / 53.0 / 53.3 / 58.1 us (past
+// 27 the LM head needs a second round); forked 61.
+static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp, int d_model, int vocab, int n_sm)
 {
-    // the SMs a round of one 128-entry tile per CTA takes; the LM head then gets
-    // all that the attention leaves (clusters share the tiles of a small vocabulary)
+    // the SMs one round of the LM head's 128-entry tiles takes (a small vocabulary's
+    // clusters also use those that the attention leaves)
     const int lm_ctas = lp.pair ? lp.P : (vocab + 127) / 128;
     const int free_sms = n_sm - (lm_ctas + lp.ctas_per_sm - 1) / lp.ctas_per_sm;
-    if (free_sms < 1 || ap.total < 1)
+    if (free_sms < 1 || tiles < 1)
         return 0;
-    if (ap.P <= free_sms)
-        return ap.P;  // the same split as the uncapped plan (whole units stay whole)
-    const double t_attn = 3.0 * (double)((ap.total + free_sms - 1) / free_sms) + 6.0;
-    const double t_lm = 2.0 * (double)vocab * (double)d_model / 5.0e6 + 8.0;
-    return t_attn < 0.75 * t_lm ? free_sms : 0;
+    if (whole_grid <= free_sms)
+        return whole_grid;  // the same split as the uncapped plan (whole units stay whole)
+    const double bytes = 2.0 * (double)vocab * (double)d_model;
+    auto t_lm = [&](int sms) { return 7.0 + bytes / (5.0e4 * sms < 6.3e6 ? 5.0e4 * sms : 6.3e6); };
+    auto t_attn = [&](int sms) { return 2.2 * (double)((tiles + sms - 1) / sms) + 6.0; };
+    int a = 1;
+    while (a < free_sms && t_attn(a) > t_lm(n_sm - a))
+        ++a;
+    const double chain = t_attn(a) > t_lm(n_sm - a) ? t_attn(a) : t_lm(n_sm - a);
+    const double fork = t_lm(n_sm) + 1.4 * (double)tiles / n_sm + 10.0;
+    return chain < fork ? a : 0;
 }
 
 static tb_status sample_enqueue(const tb_bank *bank, int bank_id, const int32_t *draft, const float *logits,
@@ -1069,14 +1086,15 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
     lt.logz_t = tr.logz_t;
     lt.ent_t = tr.ent_t;
     lt.logits_out = logits;
-    a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
+    a.max_ctas = attn_ctas_beside_lm(aplan.P, aplan.total, lplan, d_model, vocab, sm_count(bank->device));
     const int lm_sms = a.max_ctas > 0 ? sm_count(bank->device) - a.max_ctas : 0;
     // the structure of verify_step, with the walk between the LM head and the compaction
     StepStreams ss(bank, s, a.max_ctas > 0);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, workspace_bytes,
-                         kPartBase + attn_bytes, ss.lm_stream(), fn, 0, &lt, ss.lm_pdl(), lm_sms)) != TB_OK)
+                         kPartBase + attn_bytes, ss.lm_stream(), fn, 0, &lt, ss.lm_pdl(), lm_sms,
+                         !ss.chain())) != TB_OK)
         return st;
     if ((st = ss.before_accept(fn)) != TB_OK)
         return st;
@@ -1151,14 +1169,14 @@ static tb_status verify_step_impl(const tb_bank *bank, int bank_id, const tb_kv 
         lt.gather.seq[0] = LmGatherSeq{bank->d_desc + bank_id, draft_tokens, tr.draft_logit, 0, N};
     }
     // the step's structure: see StepStreams
-    a.max_ctas = attn_ctas_beside_lm(aplan, lplan, d_model, vocab, sm_count(bank->device));
+    a.max_ctas = attn_ctas_beside_lm(aplan.P, aplan.total, lplan, d_model, vocab, sm_count(bank->device));
     const int lm_sms = a.max_ctas > 0 ? sm_count(bank->device) - a.max_ctas : 0;
     StepStreams ss(bank, s, a.max_ctas > 0);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, workspace_bytes,
                          kPartBase + attn_bytes, ss.lm_stream(), fn, (flags & TB_DEBUG_EXPIRE_WAIT) ? 1 : 0,
-                         typ ? &lt : nullptr, ss.lm_pdl(), lm_sms)) != TB_OK)
+                         typ ? &lt : nullptr, ss.lm_pdl(), lm_sms, !ss.chain())) != TB_OK)
         return st;
     if ((st = ss.before_accept(fn)) != TB_OK)
         return st;
@@ -1312,7 +1330,7 @@ static tb_status verify_step_batched_impl(const tb_bank *bank, int batch, const 
         // the chunks share the partials and counters: only the first overlaps the attention
         if ((st = lm_enqueue(h8 + (size_t)r0 * d_model * 2, rc, lm_head, d_model, vocab, argmax + r0, top1 + r0,
                              entropy + r0, ws, workspace_bytes, kPartBase + attn_bytes, ss.lm_stream(), fn, 0,
-                             typ ? &lt : nullptr, ss.lm_pdl() && r0 == 0)) != TB_OK)
+                             typ ? &lt : nullptr, ss.lm_pdl() && r0 == 0, 0, !ss.chain())) != TB_OK)
             return st;
     }
     if ((st = ss.before_accept(fn)) != TB_OK)
@@ -1454,7 +1472,12 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
     sc.out = attn_out;
     for (int r = 0; r < policy->n_rungs; ++r)
         sc.rung_tree[r] = bank->d_desc + policy->bank_ids[r];
-    StepStreams ss(bank, s, false);  // the scheduled attention takes every SM
+    // The step's structure (see StepStreams), for the longest prefix the cache
+    // holds: the host does not know this step's.
+    const AttnPlan aplan = attn_tc_plan(kv->L_cap - N_max, N_max, n_q_heads, kv->n_kv_heads, kv->n_layers, nsm);
+    const int attn_sms = attn_ctas_beside_lm(nsm, aplan.total, lplan, d_model, vocab, nsm);
+    StepStreams ss(bank, s, attn_sms > 0);
+    sc.sched_copy = reinterpret_cast<int32_t *>(ws + kSchedCopyOff);
     {
         if (kv->rope_theta != 0.f) {
             RopeParams rp{};
@@ -1472,15 +1495,15 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
             return st;
         const char *err = "";
         cudaError_t e = attn_tc_launch_sched(sc, n_q_heads, reinterpret_cast<float *>(ws + kPartBase),
-                                             reinterpret_cast<int *>(ws), nsm, s, &err, ss.merge_later());
+                                             reinterpret_cast<int *>(ws), attn_sms > 0 ? attn_sms : nsm, s, &err,
+                                             ss.merge_later());
         if (e == cudaErrorInvalidValue && err[0])
             return fail(TB_EINVAL, "%s: %s", fn, err);
         if (e != cudaSuccess)
             return cuda_fail(e, fn);
         if ((st = lm_enqueue(hidden, N_max, lm_head, d_model, vocab, argmax, top1, entropy, ws,
-                             workspace_bytes, kPartBase + attn_bytes, ss.lm_stream(), fn, 0, nullptr, ss.lm_pdl())) != TB_OK)
-            return st;
-        if ((st = ss.merge(fn, false)) != TB_OK)
+                             workspace_bytes, kPartBase + attn_bytes, ss.lm_stream(), fn, 0, nullptr, ss.lm_pdl(),
+                             attn_sms > 0 ? nsm - attn_sms : 0, !ss.chain())) != TB_OK)
             return st;
         if ((st = ss.before_accept(fn)) != TB_OK)
             return st;
@@ -1510,6 +1533,8 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
     cudaError_t e = accept_launch(p, nsm, s, ss.accept_pdl());
     if (e != cudaSuccess)
         return cuda_fail(e, fn);
+    if ((st = ss.merge(fn, true)) != TB_OK)
+        return st;
     return ok();
 }
 
