@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(kLmThreads, 2) k2_lm_head(const __grid_constan
 // rows k, k + split, ..: one warp per row, four logits per lane.  Same partials
 // as k2_lm_head, merged by k2_lm_merge.
 // lm_head_stats, whole tiles / split: 26 rows x 4096 at V 1000 25.3 / 10.4 us, V
-// 4000 25.7 / 13.0, V 16000 30.5 / 28.8; 200 rows at V 3000 33.0 / 28.7.
+// 4000 25.7 / 13.0, V 16000 30.5 / 28.2; 200 rows at V 3000 33.0 / 18.0.
 //   warps 0, 2   TMA producers (alternate stages); warp 1 TMEM and the MMAs;
 //   then all eight warps: TMEM -> shared memory, and the rows.
 constexpr int kSplitThreads = 256;
@@ -635,6 +635,10 @@ __global__ void __launch_bounds__(kSplitThreads, 2) k2_lm_head_split(const __gri
     __shared__ __align__(8) uint64_t acc_full, never_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    // typical mode: the tree edges whose draft token lies in this tile, packed as in k2_lm_head
+    constexpr int kHitCap = 128;
+    __shared__ int s_hit[kTyp ? kHitCap : 1];
+    __shared__ int s_nhit;
 
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     float *parts = reinterpret_cast<float *>(ring);  // [R_pad][kSplitLd], once the ring is drained
@@ -653,6 +657,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) k2_lm_head_split(const __gri
         mbar_init(&acc_full, 1);
         mbar_init(&never_bar, 1);
         abort_flag = 0;
+        s_nhit = 0;
         fence_mbar_init();
         prefetch_tmap(&p.tmap_w);
         prefetch_tmap(&p.tmap_h);
@@ -695,6 +700,18 @@ __global__ void __launch_bounds__(kSplitThreads, 2) k2_lm_head_split(const __gri
             tc_commit(&empty_bar[s]);
         }
         tc_commit(&acc_full);  // arrives when every MMA issued above has retired
+    } else if (kTyp && warp >= 3) {
+        // the warps with nothing to do yet list the tile's draft tokens
+        const int v0 = tile * 128, nvalid = min(128, p.V - v0);
+        for (int bq = 0; bq < p.gather.n_seq; ++bq)
+            for (int e = 1 + (int)threadIdx.x - 96; e < p.gather.seq[bq].n; e += kSplitThreads - 96) {
+                int r, col;
+                if (gather_hit(p.gather, bq, e, p.R, v0, nvalid, &r, &col)) {
+                    const int h = atomicAdd(&s_nhit, 1);
+                    if (h < kHitCap)
+                        s_hit[h] = (bq << 24) | (e << 16) | (r << 7) | col;
+                }
+            }
     }
     __syncwarp();
     mbar_wait_bounded(p.expire_wait ? &never_bar : &acc_full, 0, &abort_flag, p.status);
@@ -732,60 +749,117 @@ __global__ void __launch_bounds__(kSplitThreads, 2) k2_lm_head_split(const __gri
     if (ok) {
         const int v0 = tile * 128, nvalid = min(128, p.V - v0);
         const uint32_t parts_addr = smem_u32(parts);
-        for (int r = rank + n_cta * warp; r < p.R; r += n_cta * (kSplitThreads / 32)) {
-            const uint32_t addr = parts_addr + (uint32_t)(r * kSplitLd + 4 * lane) * 4;
-            float4 part[kMaxSplit];
+        // kRows rows at a time: their loads and shuffles overlap
+        constexpr int kRows = 2;
+        const int step = n_cta * (kSplitThreads / 32);
+        for (int r0 = rank + n_cta * warp; r0 < p.R; r0 += kRows * step) {
+            float z[kRows][4];
 #pragma unroll
-            for (int k = 0; k < kMaxSplit; ++k)
-                if (k < n_cta)
-                    part[k] = ld_cluster_f32x4(cluster_map(addr, k));
-            float z[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int y = 0; y < kRows; ++y) {
+                const int r = r0 + y * step;
+                const int n = r < p.R ? n_cta : 0;  // past the rows: nothing to add
+                const uint32_t addr = parts_addr + (uint32_t)(r * kSplitLd + 4 * lane) * 4;
+                float4 part[kMaxSplit];
 #pragma unroll
-            for (int k = 0; k < kMaxSplit; ++k)
-                if (k < n_cta)
-                    z[0] += part[k].x, z[1] += part[k].y, z[2] += part[k].z, z[3] += part[k].w;
-            RowStat st = stat_empty();
+                for (int k = 0; k < kMaxSplit; ++k)
+                    if (k < n)
+                        part[k] = ld_cluster_f32x4(cluster_map(addr, k));
+                z[y][0] = z[y][1] = z[y][2] = z[y][3] = 0.f;
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
-                if (4 * lane + x < nvalid && z[x] > st.m) {
-                    st.m = z[x];
-                    st.idx = v0 + 4 * lane + x;
+                for (int k = 0; k < kMaxSplit; ++k)
+                    if (k < n)
+                        z[y][0] += part[k].x, z[y][1] += part[k].y, z[y][2] += part[k].z, z[y][3] += part[k].w;
+            }
+            // the row's maximum and its lowest entry, then the sums relative to it
+            RowStat st[kRows];
+#pragma unroll
+            for (int y = 0; y < kRows; ++y) {
+                st[y] = stat_empty();
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    if (4 * lane + x < nvalid && z[y][x] > st[y].m) {
+                        st[y].m = z[y][x];
+                        st[y].idx = v0 + 4 * lane + x;
+                    }
+            }
+#pragma unroll
+            for (int m = 16; m >= 1; m >>= 1)
+#pragma unroll
+                for (int y = 0; y < kRows; ++y) {
+                    const float m2 = __shfl_xor_sync(0xffffffffu, st[y].m, m);
+                    const int i2 = __shfl_xor_sync(0xffffffffu, st[y].idx, m);
+                    if (m2 > st[y].m || (m2 == st[y].m && i2 < st[y].idx)) {
+                        st[y].m = m2;
+                        st[y].idx = i2;
+                    }
                 }
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
-                if (4 * lane + x < nvalid) {
-                    const float dz = z[x] - st.m;
-                    const float ex = ex2_approx(dz * kLog2e);
-                    st.s += ex;
-                    st.t += ex * dz;
+            for (int y = 0; y < kRows; ++y)
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    if (4 * lane + x < nvalid) {
+                        const float dz = z[y][x] - st[y].m;
+                        const float ex = ex2_approx(dz * kLog2e);
+                        st[y].s += ex;
+                        st[y].t += ex * dz;
+                        if constexpr (kTyp) {
+                            const float dT = dz * p.inv_t;
+                            const float eT = ex2_approx(dT * kLog2e);
+                            st[y].sT += eT;
+                            st[y].tT += eT * dT;
+                        }
+                    }
+#pragma unroll
+            for (int m = 16; m >= 1; m >>= 1)
+#pragma unroll
+                for (int y = 0; y < kRows; ++y) {
+                    st[y].s += __shfl_xor_sync(0xffffffffu, st[y].s, m);
+                    st[y].t += __shfl_xor_sync(0xffffffffu, st[y].t, m);
                     if constexpr (kTyp) {
-                        const float dT = dz * p.inv_t;
-                        const float eT = ex2_approx(dT * kLog2e);
-                        st.sT += eT;
-                        st.tT += eT * dT;
+                        st[y].sT += __shfl_xor_sync(0xffffffffu, st[y].sT, m);
+                        st[y].tT += __shfl_xor_sync(0xffffffffu, st[y].tT, m);
                     }
                 }
-            st = group_merge<kTyp>(st, 32, p.inv_t);
-            if (lane == 0) {
-                p.part_tile[(size_t)tile * p.R_pad + r] = stat_pack(st);
-                if constexpr (kTyp)
-                    p.part_tile_t[(size_t)tile * p.R_pad + r] = make_float2(st.sT, st.tT);
-            }
-            if constexpr (kTyp) {
-                // the row's logits, over this CTA's part of them (which only this warp reads)
-                float *row = parts + r * kSplitLd;
-                *reinterpret_cast<float4 *>(row + 4 * lane) = make_float4(z[0], z[1], z[2], z[3]);
-                __syncwarp();
-                for (int bq = 0; bq < p.gather.n_seq; ++bq)
-                    for (int j = 1 + lane; j < p.gather.seq[bq].n; j += 32) {
-                        int er, ec;
-                        if (gather_hit(p.gather, bq, j, p.R, v0, nvalid, &er, &ec) && er == r)
-                            p.gather.seq[bq].out[j] = row[ec];
+#pragma unroll
+            for (int y = 0; y < kRows; ++y) {
+                const int r = r0 + y * step;
+                if (r >= p.R)
+                    continue;
+                if (lane == 0) {
+                    p.part_tile[(size_t)tile * p.R_pad + r] = stat_pack(st[y]);
+                    if constexpr (kTyp)
+                        p.part_tile_t[(size_t)tile * p.R_pad + r] = make_float2(st[y].sT, st[y].tT);
+                }
+                if constexpr (kTyp) {
+                    // the row's logits, over this CTA's part of them (which only this warp reads)
+                    float *row = parts + r * kSplitLd;
+                    *reinterpret_cast<float4 *>(row + 4 * lane) = make_float4(z[y][0], z[y][1], z[y][2], z[y][3]);
+                    if (p.logits_out) {
+                        __syncwarp();
+                        for (int v = lane; v < nvalid; v += 32)
+                            p.logits_out[(size_t)r * p.V + v0 + v] = row[v];
                     }
-                if (p.logits_out)
-                    for (int j = lane; j < nvalid; j += 32)
-                        p.logits_out[(size_t)r * p.V + v0 + j] = row[j];
+                }
             }
+        }
+        if constexpr (kTyp) {
+            // the draft-token logits of the tree edges whose parent row is this CTA's
+            __syncthreads();
+            const int nhit = s_nhit;
+            for (int h = threadIdx.x; h < min(nhit, kHitCap); h += kSplitThreads) {
+                const int w = s_hit[h], r = (w >> 7) & 0x1ff;
+                if (r % n_cta == rank && in_bounds((w >> 24) < p.gather.n_seq &&
+                                                       ((w >> 16) & 0xff) < p.gather.seq[w >> 24].n,
+                                                   p.status))
+                    p.gather.seq[w >> 24].out[(w >> 16) & 0xff] = parts[r * kSplitLd + (w & 0x7f)];
+            }
+            if (nhit > kHitCap)
+                for (int bq = 0; bq < p.gather.n_seq; ++bq)
+                    for (int e = 1 + threadIdx.x; e < p.gather.seq[bq].n; e += kSplitThreads) {
+                        int r, col;
+                        if (gather_hit(p.gather, bq, e, p.R, v0, nvalid, &r, &col) && r % n_cta == rank)
+                            p.gather.seq[bq].out[e] = parts[r * kSplitLd + col];
+                    }
         }
     }
     cluster_barrier();  // no CTA leaves while another reads its shared memory
