@@ -11,7 +11,10 @@
 // kernel at the end of the step: nothing in the step reads the attention
 // output).  A call of its own on a small problem (one layer of a model) gives
 // each unit to a cluster of CTAs instead, which combine their (O, m, l) through
-// shared memory at the end: no partials in memory and no second kernel.
+// shared memory at the end: no partials in memory and no second kernel.  With
+// the rotary embedding such a call also rotates the tree keys (in shared memory
+// and in the cache) and the queries itself, where one CTA alone reads a unit's
+// tree tiles.
 //
 //   S   = Q K^T   tcgen05.mma kind::f16, M = 128 query rows, N = 128 keys,
 //                 K = kD = head_dim; Q (bf16) is the TMEM A operand, the K
@@ -80,6 +83,11 @@ constexpr int tile_bytes(int d)
 {
     return d / 64 * kAtom;
 }
+// bytes of the K and V rings
+constexpr int attn_ring_bytes(int d)
+{
+    return (kKStages + kVStages) * tile_bytes(d);
+}
 // floats per partial slot: O[128][kD], m[128], l[128]
 constexpr int slot_floats(int d)
 {
@@ -122,7 +130,7 @@ struct TcCommon {
     int n_rungs, n_layers, L_cap;
     int max_rows;  // rows the split merge's grid covers: of the largest row block, or of both (row_split)
     int d;         // head_dim: the kernels' kD (host side: picks the instantiation)
-    int cluster;   // > 1: a cluster of that many CTAs shares each unit (one sequence; see attn_tc_clusters)
+    int cluster;   // > 0: a cluster of that many CTAs shares each unit (one sequence; see attn_tc_clusters)
     // rotary embedding (null: the queries are already rotated): per sequence a
     // table of (cos, sin) at position L + depth for every pair of head elements
     const float2 *rope_tab;
@@ -139,6 +147,23 @@ struct TcParamsOf : TcCommon {
 using TcParams = TcParamsOf<kMaxSeqPerLaunch>;
 template <bool kBatched>
 using TcKernelParams = TcParamsOf<kBatched ? kMaxSeqPerLaunch : 1>;
+
+// A cluster launch's parameters.  rope: the kernel itself rotates the tree keys
+// (in the cache too) and the queries, at L + depth(node).
+struct TcClusterParams : TcParamsOf<1> {
+    int rope;
+    long long k_layer_stride, k_head_stride;  // of the K cache, elements
+    __nv_bfloat16 *k;
+    double inv_freq[kRopeMaxHalf];
+};
+template <bool kBatched, bool kCluster>
+struct TcKernelArg {
+    using type = TcKernelParams<kBatched>;
+};
+template <>
+struct TcKernelArg<false, true> {
+    using type = TcClusterParams;
+};
 
 // Two row blocks per kv head (grouped queries, 129 to 256 rows) and more than a
 // wave of tiles: neighbouring CTAs walk the same key tiles side by side, one
@@ -275,9 +300,16 @@ struct SegInfo {
 // their (O, m, l) in shared memory and combine them there (log-sum-exp, in rank
 // order), every CTA a share of the rows: no partials in global memory and no
 // second kernel.  For problems small enough that all their clusters run at
-// once (attn_tc_clusters).
+// once (attn_tc_clusters).  Latency bounds these calls: of the 12 us of one
+// layer of 32 heads at 1526 keys 3.5 go to the first keys and queries, 1.05 to
+// each of three tiles, 3 to the combination and its two cluster barriers.  So
+// everything that needs none of the caller's memory (the first unit's indices,
+// the rotary table, the fetch of the roles' instructions) runs before the wait
+// for the previous kernel: 0.4 to 0.7 us less per call.  With the rotary kernel
+// before it and its table in memory a layer took 17.2 us in a 16-layer pass,
+// rotating here 14.5.
 template <int kD, bool kBatched, bool kCluster>
-__global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __grid_constant__ TcKernelParams<kBatched> p)
+__global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __grid_constant__ typename TcKernelArg<kBatched, kCluster>::type p)
 {
     static_assert(kD == 64 || kD == 128, "head_dim 64 or 128");
     constexpr int kTile = tile_bytes(kD);
@@ -293,6 +325,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     __shared__ TcSeq s_seq;
     __shared__ long long s_total;
     __shared__ SegInfo s_info[2];
+    __shared__ __align__(8) uint64_t kr_full[2];  // kCluster: the tree keys of the first / second tile that holds any are rotated
 
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sK = smem;                                // K ring: kKStages tiles
@@ -316,6 +349,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             mbar_init(&o_free[b], 4);
         }
         mbar_init(&drain_bar, 2);  // one commit from each MMA issuer
+        if constexpr (kCluster) {
+            mbar_init(&kr_full[0], 4);
+            mbar_init(&kr_full[1], 4);
+        }
         abort_flag = 0;
         fence_mbar_init();
         for (int b = 0; b < (kBatched ? p.n_seq : 1); ++b) {
@@ -327,15 +364,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         tmem_alloc(&tmem_slot, 512);
         tmem_relinquish();
     }
-    // Launched as a programmatic dependent, the kernel waits here for the
-    // stream's previous work (the previous step's compaction writes the cache);
-    // only the set-up above overlaps it.  The step's LM head may then be
-    // launched: it fills the SMs that attention CTAs leave free or release.
-    pdl_wait();
-    pdl_trigger();
+    // (cos, sin) of every pair at L + depth, and the nodes' depths: they depend on
+    // the topology and L only
+    float2 *s_rope = reinterpret_cast<float2 *>(smem + attn_ring_bytes(kD));
+    int8_t *s_dep = reinterpret_cast<int8_t *>(s_rope + kMaxNodes * (kD / 2));
+    if constexpr (kCluster) {
+        if (p.rope) {
+            const TreeDesc *tree = p.seq[0].tree;
+            if (threadIdx.x < kMaxNodes)
+                s_dep[threadIdx.x] = tree->depth[threadIdx.x];
+            const int n = (min(tree->max_depth, kMaxNodes - 1) + 1) * (kD / 2);
+            for (int i = threadIdx.x; i < n; i += kTcThreads) {
+                constexpr double kTwoPi = 6.283185307179586476925286766559;
+                const double a = (double)(p.seq[0].L + i / (kD / 2)) * p.inv_freq[i % (kD / 2)];
+                const double red = a - kTwoPi * rint(a * (1.0 / kTwoPi));
+                float2 cn;
+                sincosf((float)red, &cn.y, &cn.x);
+                s_rope[i] = cn;
+            }
+        }
+    }
+    // Launched as a programmatic dependent, the kernel waits for the stream's
+    // previous work (the previous step's compaction writes the cache) before it
+    // reads or writes any of the caller's memory: each role just before its first
+    // such access (wait_previous), so that its set-up, its first unit's indices and
+    // the fetch of its instructions overlap what runs before.  From then on the
+    // step's LM head may be launched: it fills the SMs that attention CTAs leave
+    // free or release.
+    auto wait_previous = [] {
+        pdl_wait();
+        pdl_trigger();
+    };
     const TcSeq *seqs = p.seq;
     long long total = p.total;
     if (p.sched) {
+        wait_previous();  // the state is an earlier kernel's
         if (threadIdx.x == 0)
             sched_plan(p, p.seq[0], &s_seq, &s_total);
         if (threadIdx.x == 32 && c == 0) {
@@ -367,6 +430,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     if (warp < 4) {
         if (lane != 0) {
             // one thread of each warp of this warpgroup works
+            wait_previous();
         } else if (warp == 0 || warp == 3) {
             // -------------------------------------------------------- TMA producers
             // warp 0 streams the K tiles, warp 3 the V tiles, each through its own
@@ -387,6 +451,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                 const int head = (g.u / sq.row_blocks) % p.Hkv;
                 const int layer = p.layer_begin + g.u / (sq.row_blocks * p.Hkv);
                 const CUtensorMap *m = &p.tmap[2 * sb + (is_v ? 1 : 0)];
+                if (t == t0)
+                    wait_previous();
                 for (int j = 0; j < g.n; ++j) {
                     if (!mbar_wait_bounded(&empty[s], ph ^ 1u, &abort_flag, p.status)) {
                         ok = false;
@@ -410,6 +476,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                     mbar_wait_drain(&full[it % S], (uint32_t)(it / S) & 1u);
         } else if (warp == 1) {
             // -------------------------------------------------------- QK^T issuer
+            wait_previous();
             const uint32_t idesc_s = idesc_bf16_f32(128, kBN);
             long long it = 0;
             int s = 0, sb = 0, sg = 0;
@@ -430,6 +497,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                         (j == 0 && !mbar_wait_bounded(&q_full[sg & 1], (uint32_t)(sg >> 1) & 1u, &abort_flag, p.status))) {
                         ok = false;
                         break;
+                    }
+                    if constexpr (kCluster) {
+                        const int tree_tile = g.j0 + j - p.seq[0].L / kBN;  // 0 or 1: the tile holds tree keys
+                        if (p.rope && tree_tile >= 0 &&
+                            !mbar_wait_bounded(&kr_full[tree_tile & 1], 0, &abort_flag, p.status)) {
+                            ok = false;
+                            break;
+                        }
                     }
                     tc_fence_after();
                     const uint32_t k_base = smem_u32(sK + (size_t)s * kTile);
@@ -457,6 +532,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             // 100 cycles at these shapes, so P V(i) issued here runs alongside
             // QK^T(i + 1) instead of queueing behind it, and the stage is released
             // that much sooner.
+            wait_previous();
             const uint32_t idesc_pv = idesc_bf16_f32(128, kD, false, true);
             long long it = 0;
             int s = 0, sb = 0, sg = 0;
@@ -500,6 +576,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         const int q4 = warp & 3;  // TMEM lane quadrant of this warp
         const uint32_t lane_addr = tmem + ((uint32_t)(32 * q4) << 16);
         const int rloc = 4 * lane + q4;  // query row of this thread within the block
+        wait_previous();
         long long it = 0;
         bool aborted = false;
         int sg = 0;
@@ -684,7 +761,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             SegInfo &si = s_info[sg & 1];
             const uint32_t col = lane_addr + kColQ + (sg & 1) * (kD / 2);
             const uint4 *src = reinterpret_cast<const uint4 *>(g.q);
-            if (!p.rope_tab) {
+            bool rotate = p.rope_tab != nullptr;
+            const float2 *tab = p.rope_tab + (size_t)g.b * kRopeTableEntries + (size_t)g.dep * kRopeMaxHalf;
+            if constexpr (kCluster) {
+                if (p.rope) {
+                    rotate = true;
+                    tab = s_rope + g.dep * (kD / 2);
+                }
+            }
+            if (!rotate) {
                 // the whole row (2 kD bytes) in flight at once, then kD / 32 TMEM stores
                 uint4 qv[kD / 8];
 #pragma unroll
@@ -707,7 +792,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                 // pre-rotary query: element i pairs with i + kD / 2, rotated at position
                 // L + depth(node) with the sequence's (cos, sin) table
                 constexpr int kHalf = kD / 64;  // 32-element chunks per half row
-                const float2 *tab = p.rope_tab + (size_t)g.b * kRopeTableEntries + (size_t)g.dep * kRopeMaxHalf;
 #pragma unroll 1
                 for (int qc = 0; qc < kHalf; ++qc) {
                     uint32_t wl[16], wh[16];
@@ -743,10 +827,63 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             if (lane == 0)
                 mbar_arrive(&q_full[sg & 1]);
         };
+        // Rotates the tree keys of the CTA's it-th tile (key tile j of its unit) in
+        // shared memory and writes them to the cache: no other CTA reads that tile
+        // (the launch has one row block per kv head).
+        auto rotate_keys = [&](int it, int j, int head, int layer) {
+            if constexpr (kCluster) {
+                if (!mbar_wait_bounded(&k_full[it % kKStages], (uint32_t)(it / kKStages) & 1u, &abort_flag, p.status))
+                    return false;
+                uint8_t *tile = sK + (size_t)(it % kKStages) * kTile;
+                const int L = p.seq[0].L, first = max(L, j * kBN), last = min(L + p.seq[0].N, (j + 1) * kBN);
+                constexpr int kCh = kD / 16;  // 8-pair pieces of a row
+                __nv_bfloat16 *kc = p.k + (size_t)layer * p.k_layer_stride + (size_t)head * p.k_head_stride;
+                for (int x = (int)threadIdx.x - 256; x < (last - first) * kCh; x += 128) {
+                    const int slot = first + x / kCh, ch = x % kCh, row = slot - j * kBN;
+                    // elements [8 ch, 8 ch + 8) and their partners kD / 2 on
+                    const int hi_ch = ch + kD / 16;
+                    uint4 *lo = reinterpret_cast<uint4 *>(tile + (ch >> 3) * kAtom + row * 128 + (((ch & 7) ^ (row & 7)) << 4));
+                    uint4 *hi = reinterpret_cast<uint4 *>(tile + (hi_ch >> 3) * kAtom + row * 128 +
+                                                          (((hi_ch & 7) ^ (row & 7)) << 4));
+                    uint4 a = *lo, b = *hi;
+                    __nv_bfloat16 *xa = reinterpret_cast<__nv_bfloat16 *>(&a), *xb = reinterpret_cast<__nv_bfloat16 *>(&b);
+                    const float2 *cs = s_rope + s_dep[slot - L] * (kD / 2) + 8 * ch;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const float2 c0 = cs[e];
+                        const float x1 = __bfloat162float(xa[e]), x2 = __bfloat162float(xb[e]);
+                        xa[e] = __float2bfloat16_rn(x1 * c0.x - x2 * c0.y);
+                        xb[e] = __float2bfloat16_rn(x2 * c0.x + x1 * c0.y);
+                    }
+                    *lo = a;
+                    *hi = b;
+                    if (in_bounds((long long)(slot + 1) * kD <= p.k_head_stride && slot - L < kMaxNodes, p.status)) {
+                        uint4 *dst = reinterpret_cast<uint4 *>(kc + (size_t)slot * kD);
+                        dst[ch] = a;
+                        dst[hi_ch] = b;
+                    }
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(&kr_full[(j - L / kBN) & 1]);
+            }
+            return true;
+        };
         long long t = t0;
         if (t < t1) {
             Seg cur = describe(t);
+            wait_previous();
             stage(cur, 0);
+            if constexpr (kCluster) {
+                if (p.rope) {
+                    const int u = c / p.cluster, head = u % p.Hkv, layer = p.layer_begin + u / p.Hkv;
+                    const int from = max(0, cur.L / kBN - cur.j0);  // the first tile that holds a tree key
+                    for (int it = from; it < cur.n; ++it)
+                        if (!rotate_keys(it, cur.j0 + it, head, layer))
+                            break;
+                }
+            }
             t += cur.n;
             Seg nxt{};
             bool has_next = t < t1;
@@ -777,14 +914,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                 if (!mbar_wait_bounded(&pv_done[last & 1], (uint32_t)(last >> 1) & 1u, &abort_flag, p.status))
                     break;
                 tc_fence_after();
-                const bool whole = !kCluster && cur.n == cur.T;
+                const bool whole = cur.n == cur.T;
                 const bool write = cur.valid && (whole || in_bounds(c < p.P && rloc < 128, p.status));
                 const float inv = 1.f / l;
                 uint4 *dst = reinterpret_cast<uint4 *>(cur.out);
                 // a partial (O, m, l) goes to the CTA's slot; k1_merge_split finishes the unit
                 float *slot = p.part + ((size_t)c * 2 + (cur.first ? 0 : 1)) * kSlot;
                 float4 *pdst = reinterpret_cast<float4 *>(slot + rloc * kD);
-                if constexpr (kCluster)  // the rings are drained: every tile has been consumed
+                if constexpr (kCluster)  // the rings are drained: every tile has been consumed (a cluster's part)
                     pdst = reinterpret_cast<float4 *>(smem + (size_t)rloc * kClusterLd * 4);
 #pragma unroll
                 for (int c0 = 0; c0 < kD; c0 += 64) {
@@ -835,6 +972,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     }
 
     // ---------------------------------------------------------------- teardown
+    wait_previous();  // also where a role had nothing to do: the grid completes after the stream's previous work
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -844,6 +982,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         tmem_dealloc(tmem, 512);
     }
     if constexpr (kCluster) {
+        if (p.cluster == 1)
+            return;  // whole units: written
         cluster_barrier();  // every CTA's (O, m, l) is in its shared memory
         const TcSeq &sq = seqs[0];
         const int n_cta = p.cluster, rank = c % n_cta, u = c / n_cta;
@@ -851,55 +991,47 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         const int head = (u / sq.row_blocks) % p.Hkv;
         const int layer_rel = u / (sq.row_blocks * p.Hkv);
         const int rows_here = abort_flag ? 0 : min(128, sq.rows - rb * 128);
-        // this CTA's rows are rank, rank + n_cta, ..: at most 64, so that their weights
-        // (one per row and rank, then 1 / l) fit the unused second unit record
+        // This CTA's rows are rank, rank + n_cta, ..: kVec lanes per row, four columns
+        // each, the first n_cta of them also one rank's maximum and sum; all of a
+        // row's loads are in flight together.
         const int n_rows = (rows_here - rank + n_cta - 1) / n_cta;
-        float *s_w = reinterpret_cast<float *>(s_info[1].anc), *s_inv = s_info[1].l;
-        if ((int)threadIdx.x < n_rows) {
-            const int r = threadIdx.x * n_cta + rank;
-            const uint32_t m_addr = smem_u32(&s_info[0].m[r]), l_addr = smem_u32(&s_info[0].l[r]);
-            float m[kMaxCluster], l[kMaxCluster], M = -INFINITY, lsum = 0.f;
-#pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k) {
-                m[k] = k < n_cta ? ld_cluster_f32(cluster_map(m_addr, k)) : -INFINITY;
-                l[k] = k < n_cta ? ld_cluster_f32(cluster_map(l_addr, k)) : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k)
-                M = fmaxf(M, m[k]);
-#pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k) {
-                const float w = m[k] == -INFINITY ? 0.f : ex2_approx(m[k] - M);
-                lsum += w * l[k];
-                if (k < n_cta)
-                    s_w[threadIdx.x * n_cta + k] = w;
-            }
-            s_inv[threadIdx.x] = 1.f / lsum;
-        }
-        __syncthreads();
-        constexpr int kVec = kD / 4;  // 4-column pieces of a row
-        const uint32_t o_base = smem_u32(smem);
-        for (int x = threadIdx.x; x < n_rows * kVec; x += kTcThreads) {
-            const int i = x / kVec, col = 4 * (x % kVec), r = i * n_cta + rank;
-            const uint32_t o_addr = o_base + (uint32_t)(r * kClusterLd + col) * 4;
+        constexpr int kVec = kD / 4;
+        const int sub = lane % kVec, base_lane = lane - sub;
+        const uint32_t o_base = smem_u32(smem), m_base = smem_u32(s_info[0].m), l_base = smem_u32(s_info[0].l);
+        for (int x0 = warp * 32; x0 < n_rows * kVec; x0 += kTcThreads) {
+            const int i = (x0 + lane) / kVec, r = i * n_cta + rank;
+            const int n = i < n_rows ? n_cta : 0;  // at head_dim 64 a warp's second row may not exist
+            const uint32_t o_addr = o_base + (uint32_t)(r * kClusterLd + 4 * sub) * 4;
             float4 v[kMaxCluster];
 #pragma unroll
             for (int k = 0; k < kMaxCluster; ++k)
-                if (k < n_cta)
+                if (k < n)
                     v[k] = ld_cluster_f32x4(cluster_map(o_addr, k));
+            const float m = sub < n ? ld_cluster_f32(cluster_map(m_base + 4 * r, sub)) : -INFINITY;
+            const float l = sub < n ? ld_cluster_f32(cluster_map(l_base + 4 * r, sub)) : 0.f;
+            float M = m;
+#pragma unroll
+            for (int k = kMaxCluster / 2; k >= 1; k >>= 1)
+                M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, k));
+            const float w = m == -INFINITY ? 0.f : ex2_approx(m - M);  // right in the first kMaxCluster lanes
+            float lsum = w * l;
+#pragma unroll
+            for (int k = kMaxCluster / 2; k >= 1; k >>= 1)
+                lsum += __shfl_xor_sync(0xffffffffu, lsum, k);
+            const float inv = 1.f / __shfl_sync(0xffffffffu, lsum, base_lane);
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int k = 0; k < kMaxCluster; ++k)
-                if (k < n_cta) {
-                    const float w = s_w[i * n_cta + k];
-                    acc.x += w * v[k].x, acc.y += w * v[k].y, acc.z += w * v[k].z, acc.w += w * v[k].w;
-                }
-            const float inv = s_inv[i];
+            for (int k = 0; k < kMaxCluster; ++k) {
+                const float wk = __shfl_sync(0xffffffffu, w, base_lane + k);
+                if (k < n)
+                    acc.x += wk * v[k].x, acc.y += wk * v[k].y, acc.z += wk * v[k].z, acc.w += wk * v[k].w;
+            }
             const int grow = rb * 128 + r;
             const int node = grow / p.group;
             const int qh = head * p.group + grow % p.group;
-            if (in_bounds(layer_rel < p.n_layers && node < sq.nstride && qh < p.Hq, p.status))
-                *reinterpret_cast<uint2 *>(sq.out + (((size_t)layer_rel * sq.nstride + node) * p.Hq + qh) * kD + col) =
+            if (n > 0 && in_bounds(layer_rel < p.n_layers && node < sq.nstride && qh < p.Hq, p.status))
+                *reinterpret_cast<uint2 *>(sq.out + (((size_t)layer_rel * sq.nstride + node) * p.Hq + qh) * kD +
+                                           4 * sub) =
                     make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
         }
         cluster_barrier();  // no CTA leaves while another reads its shared memory
@@ -1097,7 +1229,7 @@ static cudaError_t merge_launch_d(const TcParams &p, bool batched, cudaStream_t 
 // has work).  Scheduled mode plans on the device: assumed so.
 static bool any_split(const TcParams &p)
 {
-    if (p.P <= 1 || p.cluster > 1)
+    if (p.P <= 1 || p.cluster > 0)
         return false;
     if (p.sched)
         return true;
@@ -1123,30 +1255,45 @@ static cudaError_t merge_launch(const TcParams &p, bool batched, cudaStream_t st
 }
 
 // The attention kernel for p.d, one CTA per SM (each holds 512 TMEM columns).
-static size_t attn_smem(int d)
+static size_t attn_smem(int d, bool cluster)
 {
-    return (size_t)(kKStages + kVStages) * tile_bytes(d) + 1024;
+    // a cluster launch has room for the rotary table and the depths behind the rings
+    return (size_t)attn_ring_bytes(d) + 1024 + (cluster ? (size_t)kMaxNodes * (d / 2) * sizeof(float2) + kMaxNodes : 0);
 }
 
 template <int kD, bool kBatched, bool kCluster>
-static cudaError_t attn_kernel_launch_d(const TcParams &p, cudaStream_t stream, bool pdl)
+static cudaError_t attn_kernel_launch_d(const TcParams &p, cudaStream_t stream, bool pdl, const tb_kv *kv = nullptr)
 {
     cudaError_t e;
     if ((e = allow_max_smem((const void *)k1_tree_attention_tc<kD, kBatched, kCluster>)) != cudaSuccess)
         return e;
-    if constexpr (kBatched)
-        return launch_kernel(k1_tree_attention_tc<kD, true, false>, dim3(p.P), dim3(kTcThreads), attn_smem(kD), stream,
-                             pdl, p);
-    else
-        return launch_kernel_cluster(k1_tree_attention_tc<kD, false, kCluster>, dim3(p.P), dim3(kTcThreads),
-                                     attn_smem(kD), stream, pdl, kCluster ? p.cluster : 1, one_seq(p));
+    const size_t smem = attn_smem(kD, kCluster);
+    if constexpr (kBatched) {
+        return launch_kernel(k1_tree_attention_tc<kD, true, false>, dim3(p.P), dim3(kTcThreads), smem, stream, pdl, p);
+    } else if constexpr (kCluster) {
+        TcClusterParams q;
+        static_cast<TcParamsOf<1> &>(q) = one_seq(p);
+        q.rope = kv->rope_theta != 0.f && !p.rope_tab;
+        if (q.rope) {
+            q.k = static_cast<__nv_bfloat16 *>(kv->k);
+            q.k_layer_stride = kv->layer_stride;
+            q.k_head_stride = kv->head_stride;
+            rope_inv_freq((double)kv->rope_theta, kv->head_dim, q.inv_freq);
+        }
+        return launch_kernel_cluster(k1_tree_attention_tc<kD, false, true>, dim3(p.P), dim3(kTcThreads), smem, stream,
+                                     pdl, p.cluster, q);
+    } else {
+        return launch_kernel(k1_tree_attention_tc<kD, false, false>, dim3(p.P), dim3(kTcThreads), smem, stream, pdl,
+                             one_seq(p));
+    }
 }
 
-static cudaError_t attn_kernel_launch(const TcParams &p, bool batched, cudaStream_t stream, bool pdl)
+static cudaError_t attn_kernel_launch(const TcParams &p, bool batched, cudaStream_t stream, bool pdl,
+                                      const tb_kv *kv = nullptr)
 {
-    if (p.cluster > 1)
-        return p.d == 64 ? attn_kernel_launch_d<64, false, true>(p, stream, pdl)
-                         : attn_kernel_launch_d<128, false, true>(p, stream, pdl);
+    if (p.cluster > 0)
+        return p.d == 64 ? attn_kernel_launch_d<64, false, true>(p, stream, pdl, kv)
+                         : attn_kernel_launch_d<128, false, true>(p, stream, pdl, kv);
     if (p.d == 64)
         return batched ? attn_kernel_launch_d<64, true, false>(p, stream, pdl)
                        : attn_kernel_launch_d<64, false, false>(p, stream, pdl);
@@ -1167,7 +1314,7 @@ static int attn_max_clusters(int size)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(size);
     cfg.blockDim = dim3(kTcThreads);
-    cfg.dynamicSmemBytes = attn_smem(kD);
+    cfg.dynamicSmemBytes = attn_smem(kD, true);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = size;
@@ -1258,6 +1405,27 @@ static int attn_tc_clusters(const AttnPlan &pl, int d, int n_sm)
     return longest - even <= size ? size : 1;
 }
 
+// The launch of a stand-alone call of one sequence: its cluster size (0: the
+// ordinary kernel), and whether it applies the rotary embedding itself, which
+// saves the rotary kernel.  It does where exactly one CTA reads a tree tile of a
+// unit (one row block per kv head): units shared by clusters, and units run
+// whole (then on the cluster kernel with one CTA per unit).
+static int alone_cluster(const AttnPlan &pl, int d, int n_sm, bool rope, bool *fused)
+{
+    const int size = attn_tc_clusters(pl, d, n_sm);
+    const bool whole = pl.P == pl.n_units && pl.row_split == 1;
+    *fused = rope && pl.row_blocks == 1 && (size > 1 || whole);
+    return size > 1 ? size : *fused ? 1 : 0;
+}
+
+bool attn_tc_fuses_rope(const tb_kv *kv, int N, int Hq, int n_layers, int n_sm)
+{
+    bool fused;
+    alone_cluster(attn_tc_plan(kv->L, N, Hq, kv->n_kv_heads, n_layers, n_sm), kv->head_dim, n_sm,
+                  kv->rope_theta != 0.f, &fused);
+    return fused;
+}
+
 size_t attn_tc_slot_floats(int d)
 {
     return (size_t)slot_floats(d);
@@ -1324,15 +1492,16 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     p.total = tiles;
     // a batch splits its tiles evenly (units of different lengths)
     p.P = (int)(tiles < n_sm ? tiles : n_sm);
-    p.cluster = 1;
+    p.cluster = 0;
     if (n_seq == 1) {
         // one sequence: its plan (whole units for a short one-wave problem), or in a call of its
         // own, not part of a step, clusters that share the units of a small problem
         const AttnPlan pl = attn_tc_plan(seqs[0].kv->L, seqs[0].N, Hq, Hkv, n_layers, n_sm);
         p.P = pl.P;
+        bool fused = false;
         if (alone)
-            p.cluster = attn_tc_clusters(pl, d, n_sm);
-        if (p.cluster > 1) {
+            p.cluster = alone_cluster(pl, d, n_sm, seqs[0].kv->rope_theta != 0.f, &fused);
+        if (p.cluster > 0) {
             p.P = pl.n_units * p.cluster;
         } else if (pl.row_split == 2) {
             p.seq[0].row_split = 2;
@@ -1357,7 +1526,7 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     // dependent too, and so is its merge: only the set-up overlaps what runs
     // before, each kernel waiting for the one it follows.
     const bool pdl = alone || merge_later;
-    if ((e = attn_kernel_launch(p, batched, stream, pdl)) != cudaSuccess)
+    if ((e = attn_kernel_launch(p, batched, stream, pdl, seqs[0].kv)) != cudaSuccess)
         return e;
     if (merge_later) {
         stash_merge(p, batched, merge_later);

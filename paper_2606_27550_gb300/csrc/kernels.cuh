@@ -161,6 +161,9 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
                                  const float2 *rope_tab = nullptr, AttnMerge *merge_later = nullptr,
                                  bool alone = false);
 bool attn_tc_supported(int d);
+// whether a stand-alone call applies the rotary embedding in the attention
+// kernel (no rotary launch, rope_tab null)
+bool attn_tc_fuses_rope(const tb_kv *kv, int N, int Hq, int n_layers, int n_sm);
 AttnPlan attn_tc_plan(int L, int N, int Hq, int Hkv, int n_layers, int n_sm);
 size_t attn_tc_slot_floats(int d);  // floats per partial slot (two slots per CTA)
 // scheduled mode: the tree (rung_tree[sched[0]]) and L (sched[1]) are read on

@@ -730,7 +730,9 @@ static tb_status attn_enqueue(const AttnArgs &a, uint8_t *ws, size_t part_off, c
 {
     const char *err = "";
     const int N = a.bank->h_desc[a.bank_id].n;
-    const bool rope = a.kv->rope_theta != 0.f;
+    const int nsm = sm_count(a.bank->device);
+    // a call of its own may rotate in the attention kernel
+    const bool rope = a.kv->rope_theta != 0.f && (ss || !attn_tc_fuses_rope(a.kv, N, a.Hq, a.n_layers, nsm));
     if (rope) {
         RopeParams rp{};
         rp.seq[0] = rope_seq(a.kv, a.bank->d_desc + a.bank_id);
@@ -744,7 +746,6 @@ static tb_status attn_enqueue(const AttnArgs &a, uint8_t *ws, size_t part_off, c
             return st;
     }
     AttnMerge *merge_later = ss ? ss->merge_later() : nullptr;
-    const int nsm = sm_count(a.bank->device);
     const cudaError_t e =
         attn_tc_launch(a.kv, a.bank->d_desc + a.bank_id, N, a.layer_begin, a.n_layers, a.q, a.Hq, a.out,
                        reinterpret_cast<float *>(ws + part_off), reinterpret_cast<int *>(ws),

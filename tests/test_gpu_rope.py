@@ -104,6 +104,25 @@ def test_tree_attention_rope_parity(dev, bank, parent, L, layers, Hq, Hkv, d):
     assert np.array_equal(bits(vd), v)
 
 
+FUSED_CASES = [
+    # parent, L, layers, Hq, Hkv: a call that rotates in the attention kernel, at its edges
+    (synth.chain(64), 1000, 1, 4, 4),             # the tree spans two key tiles; 64 depths
+    (synth.bank_trees()[-1], 120, 1, 4, 4),       # two tiles, a whole unit per CTA
+    (synth.bank_trees()[5], 1152, 1, 32, 32),     # the prefix ends at a tile boundary
+    (synth.chain(2), 1023, 1, 16, 8),             # one tree key in each of two tiles
+    (synth.bank_trees()[5], 1023, 1, 20, 20),     # uneven shares of the tiles
+    (synth.bank_trees()[4], 500, 4, 8, 8),        # four layers
+    (synth.bank_trees()[-1], 1040, 1, 8, 2),      # two row blocks read the tree tile: the rotary kernel
+    (synth.bank_trees()[3], 700, 20, 16, 16),     # more units than SMs: the rotary kernel
+]
+
+
+@pytest.mark.parametrize("d", [128, 64])
+@pytest.mark.parametrize("parent,L,layers,Hq,Hkv", FUSED_CASES)
+def test_tree_attention_rope_fused_edges(dev, bank, parent, L, layers, Hq, Hkv, d):
+    test_tree_attention_rope_parity(dev, bank, parent, L, layers, Hq, Hkv, d)
+
+
 def test_tree_attention_rope_layer_subset(dev, bank):
     parent = np.asarray(synth.bank_trees()[5], np.int32)
     N, L, layers, H, d = len(parent), 200, 3, 4, 128
