@@ -325,7 +325,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     __shared__ TcSeq s_seq;
     __shared__ long long s_total;
     __shared__ SegInfo s_info[2];
-    __shared__ __align__(8) uint64_t kr_full[2];  // kCluster: the tree keys of the first / second tile that holds any are rotated
+    // kCluster with rope, for the unit's first and second tile that hold tree keys:
+    // the K tile has landed; its tree keys are rotated.  Used once each.
+    __shared__ __align__(8) uint64_t kt_full[2], kr_full[2];
 
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sK = smem;                                // K ring: kKStages tiles
@@ -350,8 +352,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         }
         mbar_init(&drain_bar, 2);  // one commit from each MMA issuer
         if constexpr (kCluster) {
-            mbar_init(&kr_full[0], 4);
-            mbar_init(&kr_full[1], 4);
+            for (int b = 0; b < 2; ++b) {
+                mbar_init(&kt_full[b], 1);
+                mbar_init(&kr_full[b], 4);
+            }
         }
         abort_flag = 0;
         fence_mbar_init();
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
             const int S = is_v ? kVStages : kKStages;
             uint8_t *ring = is_v ? sV : sK;
             long long issued = 0;
-            int s = 0, sb = 0;
+            int s = 0, sb = 0, tree_issued = 0;
             uint32_t ph = 0;
             bool ok = true;
             for (long long t = t0; ok && t < t1;) {
@@ -459,10 +463,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                         break;
                     }
                     uint8_t *dst = ring + (size_t)s * kTile;
-                    mbar_arrive_expect_tx(&full[s], kTile);
+                    uint64_t *landed = &full[s];
+                    if constexpr (kCluster) {
+                        // a K tile with tree keys to rotate lands on a barrier of its own, which
+                        // the rotating warps wait for; QK^T then waits for them
+                        const int tree_tile = g.j0 + j - p.seq[0].L / kBN;
+                        if (p.rope && !is_v && tree_tile >= 0) {
+                            mbar_arrive(&full[s]);
+                            landed = &kt_full[tree_tile & 1];
+                            tree_issued |= 1 << (tree_tile & 1);
+                        }
+                    }
+                    mbar_arrive_expect_tx(landed, kTile);
 #pragma unroll
                     for (int a = 0; a < kD / 64; ++a)
-                        tma_load_4d(dst + a * kAtom, m, &full[s], 64 * a, (g.j0 + j) * kBN, head, layer);
+                        tma_load_4d(dst + a * kAtom, m, landed, 64 * a, (g.j0 + j) * kBN, head, layer);
                     ++issued;
                     if (++s == S) {
                         s = 0;
@@ -471,9 +486,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
                 }
                 t += g.n;
             }
-            if (!ok)
+            if (!ok) {
                 for (long long it = (issued > S ? issued - S : 0); it < issued; ++it)
                     mbar_wait_drain(&full[it % S], (uint32_t)(it / S) & 1u);
+                for (int b = 0; b < 2; ++b)
+                    if (kCluster && ((tree_issued >> b) & 1))
+                        mbar_wait_drain(&kt_full[b], 0);
+            }
         } else if (warp == 1) {
             // -------------------------------------------------------- QK^T issuer
             wait_previous();
@@ -832,7 +851,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         // (the launch has one row block per kv head).
         auto rotate_keys = [&](int it, int j, int head, int layer) {
             if constexpr (kCluster) {
-                if (!mbar_wait_bounded(&k_full[it % kKStages], (uint32_t)(it / kKStages) & 1u, &abort_flag, p.status))
+                if (!mbar_wait_bounded(&kt_full[(j - p.seq[0].L / kBN) & 1], 0, &abort_flag, p.status))
                     return false;
                 uint8_t *tile = sK + (size_t)(it % kKStages) * kTile;
                 const int L = p.seq[0].L, first = max(L, j * kBN), last = min(L + p.seq[0].N, (j + 1) * kBN);

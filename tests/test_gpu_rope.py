@@ -112,6 +112,9 @@ FUSED_CASES = [
     (synth.chain(2), 1023, 1, 16, 8),             # one tree key in each of two tiles
     (synth.bank_trees()[5], 1023, 1, 20, 20),     # uneven shares of the tiles
     (synth.bank_trees()[4], 500, 4, 8, 8),        # four layers
+    ([-1], 3138, 2, 32, 32),                      # the tree tile is a CTA's 12th: the K ring has gone round
+    (synth.bank_trees()[5], 3138, 1, 32, 32),     # ... its 6th
+    (synth.bank_trees()[-1], 6080, 1, 8, 8),      # the tree tiles are a CTA's last two
     (synth.bank_trees()[-1], 1040, 1, 8, 2),      # two row blocks read the tree tile: the rotary kernel
     (synth.bank_trees()[3], 700, 20, 16, 16),     # more units than SMs: the rotary kernel
 ]
