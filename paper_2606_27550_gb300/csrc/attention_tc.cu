@@ -302,10 +302,11 @@ struct SegInfo {
 // second kernel.  For problems small enough that all their clusters run at
 // once (attn_tc_clusters).  Latency bounds these calls: of the 12 us of one
 // layer of 32 heads at 1526 keys 3.5 go to the first keys and queries, 1.05 to
-// each of three tiles, 3 to the combination and its two cluster barriers.  So
-// everything that needs none of the caller's memory (the first unit's indices,
-// the rotary table, the fetch of the roles' instructions) runs before the wait
-// for the previous kernel: 0.4 to 0.7 us less per call.  With the rotary kernel
+// each of three tiles, 3 to the combination and its two cluster barriers
+// (the first is arrived at before TMEM is freed: 0.5 us less).  So everything that
+// needs none of the caller's memory (the first unit's indices, the rotary table,
+// the fetch of the roles' instructions) runs before the wait for the previous
+// kernel: 0.4 to 0.7 us less per call.  With the rotary kernel
 // before it and its table in memory a layer took 17.2 us in a 16-layer pass,
 // rotating here 14.5.
 template <int kD, bool kBatched, bool kCluster>
@@ -993,6 +994,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
     // ---------------------------------------------------------------- teardown
     wait_previous();  // also where a role had nothing to do: the grid completes after the stream's previous work
     tc_fence_before();
+    __syncwarp();
+    if constexpr (kCluster)
+        cluster_arrive();  // this warp's part of (O, m, l) is in shared memory
     __syncthreads();
     if (warp == 1) {
         if (lane == 0)
@@ -1001,9 +1005,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
         tmem_dealloc(tmem, 512);
     }
     if constexpr (kCluster) {
+        cluster_wait();  // every CTA's (O, m, l) is in its shared memory
         if (p.cluster == 1)
             return;  // whole units: written
-        cluster_barrier();  // every CTA's (O, m, l) is in its shared memory
         const TcSeq &sq = seqs[0];
         const int n_cta = p.cluster, rank = c % n_cta, u = c / n_cta;
         const int rb = u % sq.row_blocks;
@@ -1061,8 +1065,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
 // is split exactly when a CTA range starts inside it, so the grid runs over
 // the CTA boundaries c = 1 .. P-1 (x) and groups of 8 query rows (y); the
 // first boundary inside a unit handles it.  One warp per query row, each lane
-// kD / 32 of the kD output columns, four slots' loads issued together; at most
-// 64 registers per thread (four CTAs of 256 threads per SM).
+// kD / 32 of the kD output columns.  Latency bounds it: the first block's
+// maxima, sums and four rows are loaded together (one round trip for the usual
+// unit, split between two or three CTAs), then four slots' rows at a time (2
+// heads x 128 at 12000 keys, 38 slots a unit: 25.9 us a call with the maxima
+// loaded first, 22.8 now); two CTAs of 256 threads per SM, so that nothing spills.
 //
 // kAfterStep: launched as a programmatic dependent of a verification step's
 // acceptance kernel.  The attention it merges has completed by then (the
@@ -1098,7 +1105,7 @@ struct ColVec<2> {
 };
 
 template <int kD, bool kBatched, bool kAfterStep>
-__global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__ TcKernelParams<kBatched> p)
+__global__ void __launch_bounds__(256, 2) k1_merge_split(const __grid_constant__ TcKernelParams<kBatched> p)
 {
     constexpr int kSlot = slot_floats(kD);
     constexpr int kCpl = kD / 32;  // output columns per lane
@@ -1152,31 +1159,45 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
                        p.status))
             return;
     }
-    // lane j of each 32-slot block owns slot c_lo + j0 + j: its row pointer, max and weight
-    float M = -INFINITY;
-    for (int j0 = 0; j0 < nseg; j0 += 32) {
-        const int cc = c_lo + j0 + lane;
-        if (j0 + lane < nseg) {
-            const float *sl = p.part + ((size_t)(cc * rs + half) * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
-            M = fmaxf(M, __ldcg(sl + 128 * kD + r));
-        }
+    // Lane j of each 32-slot block owns slot c_lo + j0 + j: its row pointer,
+    // maximum and sum.  The first block's four first rows are loaded with them (a
+    // unit is mostly split between two or three CTAs): one round trip to memory.
+    constexpr int kEarly = 4;
+    auto slot_of = [&](int k) {
+        const int cc = c_lo + k;
+        return p.part + ((size_t)(cc * rs + half) * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
+    };
+    const float *sl = lane < nseg ? slot_of(lane) : p.part;
+    float ms = lane < nseg ? __ldcg(sl + 128 * kD + r) : -INFINITY;
+    float ls = lane < nseg ? __ldcg(sl + 128 * kD + 128 + r) : 0.f;
+    unsigned long long row_ptr = reinterpret_cast<unsigned long long>(sl + r * kD);
+    ColVec<kCpl> early[kEarly];
+#pragma unroll
+    for (int k = 0; k < kEarly; ++k) {
+        // lane's column block of slot k
+        const unsigned long long base = __shfl_sync(0xffffffffu, row_ptr, k) + 4ull * kCpl * lane;
+        if (k < nseg)
+            early[k].load(reinterpret_cast<const float *>(base));
     }
+    float M = ms;
+    for (int j0 = 32; j0 < nseg; j0 += 32)
+        if (j0 + lane < nseg)
+            M = fmaxf(M, __ldcg(slot_of(j0 + lane) + 128 * kD + r));
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1)
         M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, m));
     float lsum = 0.f;
     float acc[kCpl] = {};
     for (int j0 = 0; j0 < nseg; j0 += 32) {
-        const int cc = c_lo + j0 + lane;
-        const float *sl = p.part;
-        float w = 0.f;
-        if (j0 + lane < nseg) {
-            sl = p.part + ((size_t)(cc * rs + half) * 2 + (tc_seg_begin(total, P, cc) >= u_first ? 0 : 1)) * kSlot;
-            const float ms = __ldcg(sl + 128 * kD + r);
-            w = (ms == -INFINITY) ? 0.f : ex2_approx(ms - M);
-            lsum += w * __ldcg(sl + 128 * kD + 128 + r);
+        if (j0 > 0) {
+            const bool have = j0 + lane < nseg;
+            sl = have ? slot_of(j0 + lane) : p.part;
+            ms = have ? __ldcg(sl + 128 * kD + r) : -INFINITY;
+            ls = have ? __ldcg(sl + 128 * kD + 128 + r) : 0.f;
+            row_ptr = reinterpret_cast<unsigned long long>(sl + r * kD);
         }
-        const unsigned long long row_ptr = reinterpret_cast<unsigned long long>(sl + r * kD);
+        const float w = (ms == -INFINITY) ? 0.f : ex2_approx(ms - M);
+        lsum += w * ls;
         const int cnt = min(32, nseg - j0);
         for (int j1 = 0; j1 < cnt; j1 += 4) {
             ColVec<kCpl> v[4];
@@ -1184,21 +1205,19 @@ __global__ void __launch_bounds__(256, 4) k1_merge_split(const __grid_constant__
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int src = (j1 + k) & 31;
-                // lane's column block of slot j0 + j1 + k
                 const unsigned long long base = __shfl_sync(0xffffffffu, row_ptr, src) + 4ull * kCpl * lane;
                 wk[k] = __shfl_sync(0xffffffffu, w, src);
-                if (j1 + k < cnt)
+                if (j0 == 0 && j1 == 0)
+                    v[k] = early[k];
+                else if (j1 + k < cnt)
                     v[k].load(reinterpret_cast<const float *>(base));
-                else
-#pragma unroll
-                    for (int x = 0; x < kCpl; ++x)
-                        v[k].v[x] = 0.f;
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
+                if (j1 + k < cnt)
 #pragma unroll
-                for (int x = 0; x < kCpl; ++x)
-                    acc[x] += wk[k] * v[k].v[x];
+                    for (int x = 0; x < kCpl; ++x)
+                        acc[x] += wk[k] * v[k].v[x];
         }
     }
 #pragma unroll

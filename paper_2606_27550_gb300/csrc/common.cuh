@@ -335,6 +335,19 @@ __device__ __forceinline__ void st_cluster_s64(uint32_t addr, long long v)
     asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 
+// The two halves of a cluster barrier: every thread of every CTA arrives once,
+// then waits once; writes before the arrival are visible after the wait.  The
+// threads of a warp need not be converged.
+__device__ __forceinline__ void cluster_arrive()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+
+__device__ __forceinline__ void cluster_wait()
+{
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // All threads of every CTA of the cluster.
 __device__ __forceinline__ void cluster_barrier()
 {

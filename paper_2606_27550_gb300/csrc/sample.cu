@@ -259,16 +259,6 @@ constexpr int kWalkWarps = kWalkThreads / 32;
 // All threads of all CTAs of the cluster; orders shared and global memory at
 // cluster scope (writes before it are visible to every CTA after it).  The
 // non-.aligned form: the threads of a warp need not be converged here.
-__device__ __forceinline__ void cluster_arrive()
-{
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-}
-
-__device__ __forceinline__ void cluster_wait()
-{
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-
 __device__ __forceinline__ void cluster_sync()
 {
     cluster_arrive();

@@ -982,11 +982,12 @@ extern "C" tb_status typical_accept(const tb_bank *bank, int bank_id, const int3
 // Otherwise the SMs are divided so that neither waits long for the other, if
 // that ends sooner than the fork.  The estimates (us, measured on GB300 at 7B
 // shapes): an attention CTA beside the LM head takes about 2.2 per 128-key
-// tile, 1.4 with every SM its own, plus 6 to 10; the LM head streams at 6.3
-// MB/us, 0.05 on one SM.  One 7B layer, 288 tiles, against V 32000, attention on
+// tile, less on many SMs, 1.4 with every SM its own, plus 6 to 10; the LM head
+// streams at 6.3 MB/us, 0.05 on one SM.  One 7B layer, 288 tiles, against V 32000, attention on
 // 12 / 16 / 20 / 24 / 27 / 32 SMs: 52.0 / 49.0 / 51.8 / 53.0 / 53.3 / 58.1 us (past
 // 27 the LM head needs a second round); forked 61.
-static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp, int d_model, int vocab, int n_sm)
+static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp, int d_model, int vocab, int n_sm,
+                               bool scheduled = false)
 {
     // the SMs one round of the LM head's 128-entry tiles takes (a small vocabulary's
     // clusters also use those that the attention leaves)
@@ -994,15 +995,27 @@ static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp
     const int free_sms = n_sm - (lm_ctas + lp.ctas_per_sm - 1) / lp.ctas_per_sm;
     if (free_sms < 1 || tiles < 1)
         return 0;
+    const double bytes = 2.0 * (double)vocab * (double)d_model;
+    if (scheduled && bytes < 16.0e6 && tiles < n_sm)
+        return 0;  // all launch latency: forked, the split-unit merge does not come last
     if (whole_grid <= free_sms)
         return whole_grid;  // the same split as the uncapped plan (whole units stay whole)
-    const double bytes = 2.0 * (double)vocab * (double)d_model;
-    auto t_lm = [&](int sms) { return 7.0 + bytes / (5.0e4 * sms < 6.3e6 ? 5.0e4 * sms : 6.3e6); };
-    auto t_attn = [&](int sms) { return 2.2 * (double)((tiles + sms - 1) / sms) + 6.0; };
+    if (bytes < 16.0e6 && tiles < n_sm)
+        return 0;
+    // many CTAs per tile of a small vocabulary: the step is faster forked (d_model
+    // 4096, V 4000 and 8000, 288 to 768 tiles: 25.6-38.8 us against 27.8-40.7), the
+    // scheduled one is not (28.0-41.2 against 25.2-38.2)
+    if (!scheduled && bytes >= 16.0e6 && 2 * lm_ctas <= n_sm)
+        return 0;
+    const double per_sm = lm_ctas < n_sm ? 3.5e4 : 5.0e4;  // a small vocabulary's clusters stream less each
+    auto t_lm = [&](int sms) { return 7.0 + bytes / (per_sm * sms < 6.3e6 ? per_sm * sms : 6.3e6); };
+    auto t_attn = [&](int sms) { return (sms > 48 ? 1.6 : 2.2) * (double)((tiles + sms - 1) / sms) + 6.0; };
     int a = 1;
     while (a < free_sms && t_attn(a) > t_lm(n_sm - a))
         ++a;
-    const double chain = t_attn(a) > t_lm(n_sm - a) ? t_attn(a) : t_lm(n_sm - a);
+    // a was taken with some slack: an attention that does not hold the step up
+    const double t_a = t_attn(a) * 0.85;
+    const double chain = t_a > t_lm(n_sm - a) ? t_a : t_lm(n_sm - a);
     const double fork = t_lm(n_sm) + 1.4 * (double)tiles / n_sm + 10.0;
     return chain < fork ? a : 0;
 }
@@ -1476,7 +1489,8 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
     // The step's structure (see StepStreams), for the longest prefix the cache
     // holds: the host does not know this step's.
     const AttnPlan aplan = attn_tc_plan(kv->L_cap - N_max, N_max, n_q_heads, kv->n_kv_heads, kv->n_layers, nsm);
-    const int attn_sms = attn_ctas_beside_lm(nsm, aplan.total, lplan, d_model, vocab, nsm);
+    const int attn_grid = aplan.total < nsm ? (int)aplan.total : nsm;
+    const int attn_sms = attn_ctas_beside_lm(attn_grid, aplan.total, lplan, d_model, vocab, nsm, true);
     StepStreams ss(bank, s, attn_sms > 0);
     sc.sched_copy = reinterpret_cast<int32_t *>(ws + kSchedCopyOff);
     {
@@ -1496,7 +1510,7 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
             return st;
         const char *err = "";
         cudaError_t e = attn_tc_launch_sched(sc, n_q_heads, reinterpret_cast<float *>(ws + kPartBase),
-                                             reinterpret_cast<int *>(ws), attn_sms > 0 ? attn_sms : nsm, s, &err,
+                                             reinterpret_cast<int *>(ws), attn_sms > 0 ? attn_sms : attn_grid, s, &err,
                                              ss.merge_later());
         if (e == cudaErrorInvalidValue && err[0])
             return fail(TB_EINVAL, "%s: %s", fn, err);
