@@ -1464,6 +1464,13 @@ bool attn_tc_fuses_rope(const tb_kv *kv, int N, int Hq, int n_layers, int n_sm)
     return fused;
 }
 
+bool attn_tc_clustered(const tb_kv *kv, int N, int Hq, int n_layers, int n_sm)
+{
+    bool fused;
+    return alone_cluster(attn_tc_plan(kv->L, N, Hq, kv->n_kv_heads, n_layers, n_sm), kv->head_dim, n_sm,
+                         kv->rope_theta != 0.f, &fused) > 0;
+}
+
 size_t attn_tc_slot_floats(int d)
 {
     return (size_t)slot_floats(d);
@@ -1533,7 +1540,7 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     p.cluster = 0;
     if (n_seq == 1) {
         // one sequence: its plan (whole units for a short one-wave problem), or in a call of its
-        // own, not part of a step, clusters that share the units of a small problem
+        // own (and a step that runs it like one) clusters that share the units of a small problem
         const AttnPlan pl = attn_tc_plan(seqs[0].kv->L, seqs[0].N, Hq, Hkv, n_layers, n_sm);
         p.P = pl.P;
         bool fused = false;
@@ -1556,11 +1563,10 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     p.max_rows = max_rows;
     const bool batched = n_seq > 1;
     cudaError_t e;
-    // In a step, a grid that takes every SM starts when the stream's previous
-    // work is done, so that all its CTAs start together (its work split is
-    // static) and before the LM head's; a grid capped beside a longer LM head
-    // (merge_later) is launched as a programmatic dependent and its CTAs wait on
-    // SMs that are free already.  A call of its own is launched as a programmatic
+    // In a forked step the grid starts when the stream's previous work is done,
+    // so that all its CTAs start together (its work split is static) and before
+    // the LM head's; in a chain (merge_later) it is launched as a programmatic
+    // dependent.  A call of its own is launched as a programmatic
     // dependent too, and so is its merge: only the set-up overlaps what runs
     // before, each kernel waiting for the one it follows.
     const bool pdl = alone || merge_later;

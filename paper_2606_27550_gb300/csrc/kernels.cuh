@@ -154,7 +154,7 @@ cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream, bool afte
 // pre-rotary and are rotated at L + depth while they are staged
 // merge_later: the split-unit merge is not enqueued but kept there, and the
 // attention is launched as a programmatic dependent; alone: a call of its own,
-// not part of a verification step (clusters may share its units, and its
+// or a step's attention run like one (clusters may share its units, and its
 // launches are programmatic dependents)
 cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin, int n_layers, int Hq, float *part,
                                  int *status, int n_sm, cudaStream_t stream, const char **err,
@@ -164,6 +164,8 @@ bool attn_tc_supported(int d);
 // whether a stand-alone call applies the rotary embedding in the attention
 // kernel (no rotary launch, rope_tab null)
 bool attn_tc_fuses_rope(const tb_kv *kv, int N, int Hq, int n_layers, int n_sm);
+// whether its launch leaves no partials to merge (clusters share its units)
+bool attn_tc_clustered(const tb_kv *kv, int N, int Hq, int n_layers, int n_sm);
 AttnPlan attn_tc_plan(int L, int N, int Hq, int Hkv, int n_layers, int n_sm);
 size_t attn_tc_slot_floats(int d);  // floats per partial slot (two slots per CTA)
 // scheduled mode: the tree (rung_tree[sched[0]]) and L (sched[1]) are read on

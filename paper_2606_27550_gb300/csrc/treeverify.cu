@@ -240,15 +240,15 @@ struct tb_bank {
 };
 
 // The order in which one verification step's kernels are enqueued.  Two
-// structures:
-//  - The attention and the LM head divide the SMs (attn_ctas_beside_lm: one
-//    layer or a few against a vocabulary): one chain on the caller's stream,
-//    each kernel a programmatic dependent of the one before: [rotary embedding,]
-//    attention, LM head, acceptance + compaction, then the attention's (small)
-//    split-unit merge, beside the acceptance kernel (nothing in the step reads
-//    the attention output).  The LM head does not depend on the attention: it is
-//    launched as soon as every attention CTA has started and fills the SMs the
-//    attention is kept off; it completes only after the attention has, so the
+// structures (plan_step chooses for one sequence):
+//  - One chain on the caller's stream, each kernel a programmatic dependent of
+//    the one before: [rotary embedding,] attention, LM head, acceptance +
+//    compaction, then the attention's split-unit merge (if it leaves one), beside
+//    the acceptance kernel (nothing in the step reads the attention output).  The
+//    LM head does not depend on the attention: it is launched as soon as every
+//    attention CTA has started and fills the SMs the attention is kept off
+//    (attn_ctas_beside_lm: one layer or a few against a vocabulary) or those it
+//    releases; it completes only after the attention has, so the
 //    acceptance kernel, which waits for it, compacts the cache after the
 //    attention read it, and its launch overlaps the LM head's tail.  The
 //    attention is itself a programmatic dependent of the previous step.
@@ -260,9 +260,9 @@ struct tb_bank {
 //    join events are shared, so the bank's mutex is held from construction to
 //    the end of the step's enqueueing.
 // Measured on GB300, fork / chain: one 7B layer at 1024 keys against V 32000
-// 58.4 / 50.0 us a step, at 3000 keys 63.7 / 56.0, device-driven 66.6 / 60.3; with
-// an attention that takes every SM the chain cost 4-8 us (its split-unit merge
-// then lies on the critical path).
+// 58.4 / 50.0 us a step, at 3000 keys 63.7 / 56.0, device-driven 66.6 / 60.3.  A
+// batch whose attention takes every SM is forked: its split-unit merge would lie
+// on the critical path (4-8 us).
 class StepStreams {
   public:
     StepStreams(const tb_bank *bank, cudaStream_t s, bool chain)
@@ -653,6 +653,7 @@ struct AttnArgs {
     int Hq;
     void *out;
     int max_ctas;  // > 0: the tcgen05 attention grid takes at most this many SMs
+    bool clusters; // a step's attention that runs as a call of its own: clusters share its units, no merge
 };
 
 static tb_status check_rope(const tb_kv *kv, const char *fn);
@@ -731,7 +732,8 @@ static tb_status attn_enqueue(const AttnArgs &a, uint8_t *ws, size_t part_off, c
     const int N = a.bank->h_desc[a.bank_id].n;
     const int nsm = sm_count(a.bank->device);
     // a call of its own may rotate in the attention kernel
-    const bool rope = a.kv->rope_theta != 0.f && (ss || !attn_tc_fuses_rope(a.kv, N, a.Hq, a.n_layers, nsm));
+    const bool alone = !ss || a.clusters;
+    const bool rope = a.kv->rope_theta != 0.f && !(alone && attn_tc_fuses_rope(a.kv, N, a.Hq, a.n_layers, nsm));
     if (rope) {
         RopeParams rp{};
         rp.seq[0] = rope_seq(a.kv, a.bank->d_desc + a.bank_id);
@@ -744,12 +746,12 @@ static tb_status attn_enqueue(const AttnArgs &a, uint8_t *ws, size_t part_off, c
         if (st != TB_OK)
             return st;
     }
-    AttnMerge *merge_later = ss ? ss->merge_later() : nullptr;
+    AttnMerge *merge_later = alone ? nullptr : ss->merge_later();
     const cudaError_t e =
         attn_tc_launch(a.kv, a.bank->d_desc + a.bank_id, N, a.layer_begin, a.n_layers, a.q, a.Hq, a.out,
                        reinterpret_cast<float *>(ws + part_off), reinterpret_cast<int *>(ws),
                        a.max_ctas > 0 && a.max_ctas < nsm ? a.max_ctas : nsm, stream, &err,
-                       rope ? rope_table(ws) : nullptr, merge_later, ss == nullptr);
+                       rope ? rope_table(ws) : nullptr, merge_later, alone);
     if (e == cudaErrorInvalidValue && err[0])
         return fail(TB_EINVAL, "%s: %s", fn, err);
     if (e != cudaSuccess)
@@ -1019,6 +1021,34 @@ static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp
     return chain < fork ? a : 0;
 }
 
+// The structure of one sequence's step (see StepStreams): sets a.max_ctas and
+// a.clusters, and returns whether the step is one chain.
+//  - the attention and the LM head divide the SMs where that ends sooner
+//    (attn_ctas_beside_lm);
+//  - an attention whose units clusters share takes every SM and leaves no merge:
+//    the chain, the LM head following in the attention's tail.  Forked (with the
+//    split grid and its merge) / chained, us a step: 4 layers x 8 kv heads at
+//    6000 keys 45.8 / 43.6, with the rotary embedding (in the attention kernel
+//    then) 50.5 / 43.7; 8 layers x 8 kv heads at 3000 keys 52.5 / 46.2; 2 layers x 32
+//    at 2000 keys, V 64000 125 / 113;
+//  - otherwise the split-unit merge comes last in the chain and beside the LM
+//    head in the fork.  The chain is the faster while the merge is small: up to
+//    32 query rows a unit (6 layers x 32 kv heads, 16 rows at 1000 keys, V 32000 and
+//    128256 76.6 / 74.7 and 194 / 189; 32 layers, 26 rows 141 / 139; 64 rows 85.0 /
+//    86.9), or beside an LM head too short to hide it (W 66 MB: 64 to 128 rows, 9 to
+//    17 tiles an SM 61 to 75 / 57 to 71; 213 tiles an SM 279 / 284; W 262 MB 85 to 97 /
+//    87 to 100).
+static bool plan_step(AttnArgs &a, const AttnPlan &ap, const LmPlan &lp, int d_model, int vocab)
+{
+    const int n_sm = sm_count(a.bank->device);
+    a.max_ctas = attn_ctas_beside_lm(ap.P, ap.total, lp, d_model, vocab, n_sm);
+    a.clusters = a.max_ctas == 0 &&
+                 attn_tc_clustered(a.kv, a.bank->h_desc[a.bank_id].n, a.Hq, a.n_layers, n_sm);
+    if (a.max_ctas > 0 || a.clusters || ap.rows <= 32)
+        return true;
+    return 2.0 * (double)vocab * (double)d_model <= 128.0e6 && ap.total <= 16ll * n_sm;
+}
+
 static tb_status sample_enqueue(const tb_bank *bank, int bank_id, const int32_t *draft, const float *logits,
                                 const float *logz_t, const float *q, const float *unif, int vocab, int L,
                                 float temperature, float *scratch, tb_result *result, const int *ws_status,
@@ -1099,15 +1129,15 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
     lt.logz_t = tr.logz_t;
     lt.ent_t = tr.ent_t;
     lt.logits_out = logits;
-    a.max_ctas = attn_ctas_beside_lm(aplan.P, aplan.total, lplan, d_model, vocab, sm_count(bank->device));
+    const bool chain = plan_step(a, aplan, lplan, d_model, vocab);
     const int lm_sms = a.max_ctas > 0 ? sm_count(bank->device) - a.max_ctas : 0;
     // the structure of verify_step, with the walk between the LM head and the compaction
-    StepStreams ss(bank, s, a.max_ctas > 0);
+    StepStreams ss(bank, s, chain);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, workspace_bytes,
                          kPartBase + attn_bytes, ss.lm_stream(), fn, 0, &lt, ss.lm_pdl(), lm_sms,
-                         !ss.chain())) != TB_OK)
+                         a.max_ctas == 0)) != TB_OK)
         return st;
     if ((st = ss.before_accept(fn)) != TB_OK)
         return st;
@@ -1182,14 +1212,14 @@ static tb_status verify_step_impl(const tb_bank *bank, int bank_id, const tb_kv 
         lt.gather.seq[0] = LmGatherSeq{bank->d_desc + bank_id, draft_tokens, tr.draft_logit, 0, N};
     }
     // the step's structure: see StepStreams
-    a.max_ctas = attn_ctas_beside_lm(aplan.P, aplan.total, lplan, d_model, vocab, sm_count(bank->device));
+    const bool chain = plan_step(a, aplan, lplan, d_model, vocab);
     const int lm_sms = a.max_ctas > 0 ? sm_count(bank->device) - a.max_ctas : 0;
-    StepStreams ss(bank, s, a.max_ctas > 0);
+    StepStreams ss(bank, s, chain);
     if ((st = attn_enqueue(a, ws, kPartBase, s, fn, &ss)) != TB_OK)
         return st;
     if ((st = lm_enqueue(hidden, N, lm_head, d_model, vocab, argmax, top1, entropy, ws, workspace_bytes,
                          kPartBase + attn_bytes, ss.lm_stream(), fn, (flags & TB_DEBUG_EXPIRE_WAIT) ? 1 : 0,
-                         typ ? &lt : nullptr, ss.lm_pdl(), lm_sms, !ss.chain())) != TB_OK)
+                         typ ? &lt : nullptr, ss.lm_pdl(), lm_sms, a.max_ctas == 0)) != TB_OK)
         return st;
     if ((st = ss.before_accept(fn)) != TB_OK)
         return st;
