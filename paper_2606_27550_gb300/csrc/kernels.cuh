@@ -1,6 +1,8 @@
 // kernels.cuh -- host-side interface between the C-ABI layer and the kernels.
 #pragma once
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace tv {
@@ -49,6 +51,38 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 {
     return launch_kernel_cluster(kernel, grid, block, smem, stream, pdl, 1, static_cast<Args &&>(args)...);
 }
+
+// Clusters of `size` CTAs of `kernel`, of `threads` threads and `smem` bytes of
+// dynamic shared memory each, that the current device holds at once (0: none, or
+// the query failed).  Gives the device's copy of the kernel the attributes that
+// such a launch needs: 8 is the largest size that needs none.
+int ask_max_clusters(const void *kernel, int size, int threads, size_t smem);
+
+// What was asked of each device, by a small index: attributes and occupancy
+// belong to a device's copy of a kernel, and one process may use several devices.
+template <int kSlots>
+class PerDevice {
+  public:
+    // ask(): the answer (>= 0) for the current device, asked once per device and slot
+    template <typename F>
+    int get(int slot, F ask)
+    {
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices)
+            return ask();
+        std::atomic<int> &a = answers_[dev][slot];
+        int v = a.load(std::memory_order_acquire);
+        if (v == 0) {
+            v = ask() + 1;
+            a.store(v, std::memory_order_release);
+        }
+        return v - 1;
+    }
+
+  private:
+    static constexpr int kDevices = 32;
+    std::atomic<int> answers_[kDevices][kSlots] = {};  // 0: not asked yet, else the answer + 1
+};
 
 // LM head (lm_head.cu)
 struct LmPlan {

@@ -46,8 +46,6 @@
 // rejection.
 #include <math.h>
 
-#include <atomic>
-
 #include "kernels.cuh"
 
 namespace tv {
@@ -514,35 +512,15 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
     }
 }
 
-// Whether a cluster of kCtas CTAs can be resident (cached; 16 is above the
-// portable cluster size).
+// Whether a cluster of kCtas CTAs can be resident (16 is above the portable
+// cluster size: the query also allows it on the current device).
 template <int E, int kCtas>
 static bool walk_fits()
 {
-    static std::atomic<int> cache{0};  // 0: not queried yet, 1: no, 2: yes
-    int v = cache.load(std::memory_order_relaxed);
-    if (v == 0) {
-        int n = 0;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(kCtas);
-        cfg.blockDim = dim3(kWalkThreads);
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = kCtas;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if ((kCtas > 8 && cudaFuncSetAttribute(k4_spec_sample_cluster<E, kCtas>,
-                                               cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
-            cudaOccupancyMaxActiveClusters(&n, k4_spec_sample_cluster<E, kCtas>, &cfg) != cudaSuccess) {
-            (void)cudaGetLastError();
-            n = 0;
-        }
-        v = n >= 1 ? 2 : 1;
-        cache.store(v, std::memory_order_relaxed);
-    }
-    return v == 2;
+    static PerDevice<1> fits;
+    return fits.get(0, [] {
+        return ask_max_clusters((const void *)k4_spec_sample_cluster<E, kCtas>, kCtas, kWalkThreads, 0);
+    }) >= 1;
 }
 
 template <int E, int kCtas>
