@@ -61,8 +61,6 @@
 // the softmax).
 #include <string.h>
 
-#include <atomic>
-
 #include "kernels.cuh"
 
 namespace tv {
@@ -1340,33 +1338,15 @@ static cudaError_t attn_kernel_launch(const TcParams &p, bool batched, cudaStrea
 }
 
 // Clusters of `size` CTAs of the attention kernel that can be resident at once
-// on the current device (cached; 0 if none).
+// on the current device (0 if none).
 template <int kD>
 static int attn_max_clusters(int size)
 {
-    static std::atomic<int> cache[kMaxCluster + 1];  // 0: not queried yet, else clusters + 1
-    const int v = cache[size].load(std::memory_order_relaxed);
-    if (v > 0)
-        return v - 1;
-    int n = 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(size);
-    cfg.blockDim = dim3(kTcThreads);
-    cfg.dynamicSmemBytes = attn_smem(kD, true);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (allow_max_smem((const void *)k1_tree_attention_tc<kD, false, true>) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, k1_tree_attention_tc<kD, false, true>, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        n = 0;
-    }
-    cache[size].store(n + 1, std::memory_order_relaxed);
-    return n;
+    static PerDevice<kMaxCluster + 1> clusters;
+    return clusters.get(size, [size] {
+        return ask_max_clusters((const void *)k1_tree_attention_tc<kD, false, true>, size, kTcThreads,
+                                attn_smem(kD, true));
+    });
 }
 
 // The attention launch's parameters, kept for a split-unit merge enqueued later.

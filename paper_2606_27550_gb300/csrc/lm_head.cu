@@ -33,7 +33,6 @@
 // HBM bounds it: 262 MB (V 32000 x 4096) in 45-46 us with its merge, 1.05 GB (V
 // 128256) in 160-163 us, 6.4 TB/s.  W larger than half of L2 is loaded
 // evict-first (V 128256 168 us without).
-#include <atomic>
 #include <math.h>
 #include <stdlib.h>
 
@@ -1120,34 +1119,13 @@ size_t lm_parts_bytes(int R, int V, int n_sm)
 }
 
 // Clusters of two CTAs of k2_lm_head<kTyp, true> with `smem` bytes each that
-// can be resident at once (cached per shared-memory size; 0 if none).
+// can be resident at once on the current device (0 if none).
 template <bool kTyp>
 static int lm_max_pairs(size_t smem)
 {
-    static std::atomic<int> cache[24];  // by smem / 16 KB; 0: not queried yet, else pairs + 1
-    const size_t slot = smem / 16384 < 24 ? smem / 16384 : 23;
-    int v = cache[slot].load(std::memory_order_relaxed);
-    if (v > 0)
-        return v - 1;
-    int pairs = 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2);
-    cfg.blockDim = dim3(kLmThreads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (allow_max_smem((const void *)k2_lm_head<kTyp, true>) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&pairs, k2_lm_head<kTyp, true>, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        pairs = 0;
-    }
-    cache[slot].store(pairs + 1, std::memory_order_relaxed);
-    return pairs;
+    static PerDevice<24> pairs;  // by smem / 16 KB
+    const int slot = smem / 16384 < 24 ? (int)(smem / 16384) : 23;
+    return pairs.get(slot, [smem] { return ask_max_clusters((const void *)k2_lm_head<kTyp, true>, 2, kLmThreads, smem); });
 }
 
 // k2_lm_head, then its merge as a programmatic dependent (launched while the

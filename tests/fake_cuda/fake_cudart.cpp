@@ -7,6 +7,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -21,7 +22,7 @@ namespace {
 
 constexpr int kDevices = 2, kSms = 152, kMaxSmem = 232448, kDefaultSmem = 48 << 10;
 // clusters of 1..16 such CTAs (one per SM) that a GB300 holds at once
-constexpr int kClustersBySize[17] = {0, 152, 76, 48, 36, 28, 24, 20, 16, 15, 14, 13, 12, 11, 10, 10, 8};
+constexpr int kClustersBySize[17] = {0, 152, 76, 46, 36, 28, 23, 15, 15, 7, 7, 7, 7, 7, 7, 7, 7};
 
 struct Launch {
     std::string name;
@@ -41,6 +42,7 @@ std::set<std::pair<const void *, int>> large_smem, large_cluster;  // (function,
 std::vector<Launch> launches;
 std::string text;
 thread_local int device = 0;
+int cluster_limit[kDevices] = {kSms, kSms};  // clusters of any size that a device holds at once
 unsigned long long next_handle = 0x1000;
 
 cudaError_t check(const cudaLaunchConfig_t *cfg, const void *fn, unsigned *cluster, int *pdl)
@@ -98,6 +100,12 @@ void fake_set_device(int d)
     device = d;
 }
 
+// limits the clusters that a device holds at once
+void fake_limit_clusters(int d, int n)
+{
+    cluster_limit[d] = n;
+}
+
 void **__cudaRegisterFatBinary(void *)
 {
     static void *handle;
@@ -151,7 +159,7 @@ cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *fn, const cudaLau
     int pdl;
     const cudaError_t e = check(cfg, fn, &cluster, &pdl);
     if (e == cudaSuccess)
-        *n = kClustersBySize[cluster];
+        *n = std::min(kClustersBySize[cluster], cluster_limit[device]);
     return e;
 }
 cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute attr, int value)
