@@ -53,6 +53,7 @@ namespace tv {
 namespace {
 
 constexpr int kSampleThreads = 1024;
+constexpr int kNoToken = 0x7fffffff;
 
 // Block-wide sum over the kSampleThreads threads; every thread gets the total.
 __device__ float block_sum(float x, float *red)
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(kSampleThreads) k4_spec_sample(const __grid_co
     __shared__ float red[32];
     __shared__ int s_par[kMaxNodes];
     __shared__ int s_draft[kMaxNodes];
-    __shared__ int s_tok;
+    __shared__ int s_tok, s_last;
     pdl_wait();
     pdl_trigger();
     const TreeDesc *t = p.tree;
@@ -145,8 +146,10 @@ __global__ void __launch_bounds__(kSampleThreads) k4_spec_sample(const __grid_co
         s_par[tid] = tid < n ? t->parent[tid] : -2;
         s_draft[tid] = tid < n ? p.draft[tid] : 0;
     }
-    if (tid == 0)
-        s_tok = 0x7fffffff;
+    if (tid == 0) {
+        s_tok = kNoToken;
+        s_last = -1;
+    }
     __syncthreads();
 
     constexpr float kLog2e = 1.4426950408889634f;
@@ -204,29 +207,43 @@ __global__ void __launch_bounds__(kSampleThreads) k4_spec_sample(const __grid_co
     const int per = vec ? ((p.V / 4 + kSampleThreads - 1) / kSampleThreads) * 4 : (p.V + kSampleThreads - 1) / kSampleThreads;
     const int v0 = min(p.V, tid * per), v1 = min(p.V, v0 + per);
     float loc = 0.f;
+    int last = -1;  // the last entry of positive probability
     if (vec) {
         for (int v = v0; v < v1; v += 4) {
             const float4 x = r.at4(p.resid, v);
             loc += ((x.x + x.y) + x.z) + x.w;
+            last = x.w > 0.f ? v + 3 : x.z > 0.f ? v + 2 : x.y > 0.f ? v + 1 : x.x > 0.f ? v : last;
         }
     } else {
-        for (int v = v0; v < v1; ++v)
-            loc += r.at(p.resid, v);
+        for (int v = v0; v < v1; ++v) {
+            const float x = r.at(p.resid, v);
+            loc += x;
+            last = x > 0.f ? v : last;
+        }
     }
     float total;
     const float before = block_exclusive_scan(loc, red, &total);
     const float thr = p.unif[n + u] * total;
-    if (v1 > v0 && before <= thr && thr < before + loc) {
+    // The lowest first entry past the threshold of the chunks that end past it,
+    // else the last positive entry (see the cluster walk).
+    int pick = kNoToken;
+    if (loc > 0.f && thr < before + loc) {
+        pick = last;
         float cum = before;
-        int pick = v1 - 1;
         for (int v = v0; v < v1; ++v) {
-            cum += r.at(p.resid, v);
-            if (cum > thr) {
+            const float x = r.at(p.resid, v);
+            cum += x;
+            if (x > 0.f && cum > thr) {
                 pick = v;
                 break;
             }
         }
-        atomicMin(&s_tok, pick);  // rounding can let two neighbouring chunks claim the threshold
+    }
+    pick = __reduce_min_sync(0xffffffffu, pick);
+    last = __reduce_max_sync(0xffffffffu, last);
+    if ((tid & 31) == 0) {
+        atomicMin(&s_tok, pick);
+        atomicMax(&s_last, last);
     }
     __syncthreads();
 
@@ -241,7 +258,7 @@ __global__ void __launch_bounds__(kSampleThreads) k4_spec_sample(const __grid_co
         for (int i = pos; i < kMaxNodes; ++i)
             res->path[i] = -1;
         res->accept_len = len;
-        res->bonus_token = s_tok == 0x7fffffff ? p.V - 1 : s_tok;  // threshold at the total: the last token
+        res->bonus_token = s_tok != kNoToken ? s_tok : s_last >= 0 ? s_last : p.V - 1;
         res->new_L = p.L + len;
         const int ws = p.ws_status ? *p.ws_status : 0;
         res->status = (ws & kStatusTimeout) ? TB_ETIMEOUT
@@ -266,13 +283,6 @@ __device__ __forceinline__ void cluster_sync()
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v)
 {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-
-// Atomic minimum on a 32-bit shared variable of another CTA of the cluster
-// (ordered for the others by the next cluster barrier).
-__device__ __forceinline__ void red_min_cluster_s32(uint32_t a, int v)
-{
-    asm volatile("red.relaxed.cluster.shared::cluster.min.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
 // Hands this warp's value x to every CTA of the cluster: entry rank * 32 + warp
@@ -342,6 +352,15 @@ __device__ __forceinline__ void load_slice(const float *z, const float *q, int v
     }
 }
 
+// The first lane with a positive total that ends past thr, else the last one with
+// a positive total (-1: none).
+__device__ __forceinline__ int draw_lane(float total, float end, float thr)
+{
+    const uint32_t some = __ballot_sync(0xffffffffu, total > 0.f);
+    const uint32_t past = __ballot_sync(0xffffffffu, total > 0.f && end > thr);
+    return past ? __ffs(past) - 1 : 31 - __clz(some);
+}
+
 template <int E, int kCtas>
 __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const __grid_constant__ SampleParams p)
 {
@@ -352,7 +371,6 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
     __shared__ float l_pt[kMaxNodes];       // ... p_u(t_c), q_u(t_c) and the uniform deciding c
     __shared__ float l_qt[kMaxNodes], l_uf[kMaxNodes];
     __shared__ float l_off[kMaxNodes];      // log2(e) logZ_u of each node
-    __shared__ int s_tok;                   // rank 0: the drawn token (minimum over the claiming threads)
 
     constexpr float kLog2e = 1.4426950408889634f;
     cluster_arrive();  // every CTA has started: waited for before the first remote access
@@ -363,8 +381,6 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
     const int n = p.n;
     if (tid < kMaxNodes)
         l_kids[tid] = 0;
-    if (tid == 0)
-        s_tok = 0x7fffffff;
     __syncthreads();
     pdl_wait();
     pdl_trigger();
@@ -453,17 +469,19 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
     }
     float *vals = s_vals[nsum & 1];
     cluster_publish<kCtas>(__shfl_sync(0xffffffffu, inc, 31), rank, vals);
-    cluster_sync();
-    // lane l adds the totals of the cluster's warps [l * kCtas, (l + 1) * kCtas)
-    const int mine = static_cast<int>(rank) * kWalkWarps + warp;
-    float sum = 0.f, part = 0.f;  // part: of those before this warp
+    cluster_sync();  // no CTA touches another's shared memory after it
+    // The draw goes down in three steps: lane l stands for the cluster's warps
+    // [l * kCtas, (l + 1) * kCtas), then a lane for each of those warps, then each
+    // for a thread of the warp.  Each step takes the first lane with a positive
+    // total whose end lies past the threshold.  There is no lower bound on its
+    // begin: rounded ends and begins of neighbours need not meet, and a total may
+    // be too small to move the end.  If no end lies past it (the total was rounded
+    // up) the step takes the last positive one.  Every warp finds the same lane from
+    // the same numbers, so no CTA has to tell another.
+    float sum = 0.f;
 #pragma unroll
-    for (int r = 0; r < kCtas; ++r) {
-        const float x = vals[lane * kCtas + r];
-        if (r == mine % kCtas)
-            part = sum;
-        sum += x;
-    }
+    for (int r = 0; r < kCtas; ++r)
+        sum += vals[lane * kCtas + r];
     float incl = sum;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -472,25 +490,37 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
             incl += y;
     }
     const float grand = __shfl_sync(0xffffffffu, incl, 31);
-    const float base = __shfl_sync(0xffffffffu, incl - sum + part, mine / kCtas);
     const float thr = uf * grand;
-    const float c0 = base + (inc - loc);
-    if (loc > 0.f && c0 <= thr && thr < c0 + loc) {
-        float cum = c0;
-        int pick = -1, last = -1;
+    const int owner = draw_lane(sum, incl, thr);
+    const bool none = owner < 0 || !(grand < INFINITY);  // a residual that vanished: the last token
+    const int mine = static_cast<int>(rank) * kWalkWarps + warp;
+    if (!none && mine / kCtas == owner) {
+        const float base = __shfl_sync(0xffffffffu, incl - sum, owner);
+        const float x = lane < kCtas ? vals[owner * kCtas + lane] : 0.f;
+        float pre = x;
 #pragma unroll
-        for (int j = 0; j < E; ++j) {
-            cum += pv[j];
-            if (pv[j] > 0.f) {
-                last = v0 + j;
-                if (pick < 0 && cum > thr)
-                    pick = v0 + j;
-            }
+        for (int d = 1; d < kCtas; d <<= 1) {
+            const float y = __shfl_up_sync(0xffffffffu, pre, d);
+            if (lane >= d)
+                pre += y;
         }
-        // into rank 0's s_tok (rounding can let two neighbouring chunks claim the threshold)
-        red_min_cluster_s32(cluster_addr(&s_tok, 0), pick >= 0 ? pick : last);
+        const int w = draw_lane(x, base + pre, thr);
+        const float c0 = __shfl_sync(0xffffffffu, base + (pre - x), w);
+        if (mine % kCtas == w && lane == draw_lane(loc, c0 + inc, thr)) {
+            float cum = c0 + (inc - loc);
+            int pick = -1, last = -1;
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                cum += pv[j];
+                if (pv[j] > 0.f) {
+                    last = v0 + j;
+                    if (pick < 0 && cum > thr)
+                        pick = v0 + j;
+                }
+            }
+            p.result->bonus_token = pick >= 0 ? pick : last;
+        }
     }
-    cluster_sync();  // every claim has reached rank 0; no CTA touches another's shared memory after it
     if (rank == 0 && tid < kMaxNodes) {
         tb_result *res = p.result;
         const uint64_t anc = l_anc[u];
@@ -500,9 +530,9 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
         if (tid >= len)
             res->path[tid] = -1;
         if (tid == 0) {
-            const int tok = s_tok;
+            if (none)
+                res->bonus_token = p.V - 1;
             res->accept_len = len;
-            res->bonus_token = tok == 0x7fffffff ? p.V - 1 : tok;  // threshold at the total: the last token
             res->new_L = p.L + len;
             const int ws = p.ws_status ? *p.ws_status : 0;
             res->status = (ws & kStatusTimeout)

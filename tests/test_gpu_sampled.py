@@ -124,6 +124,32 @@ def test_walk_large_vocab_paths(dev, V):
     b.close()
 
 
+@pytest.mark.parametrize("V", [20000, 32000, 50001, 150004, 262144, 262145])
+def test_draw_in_a_flat_tail(dev, V):
+    """Thresholds inside a tail of tokens so unlikely that a thread's share of it
+    is less than half an ulp of the cumulative sum before it: the token drawn is
+    still the one whose interval holds the threshold, to the rounding of the sums
+    (about 50 of values up to 1, half an ulp of 2^-24 each, and 2^-22 of the
+    exponential: below 2^-19), and never one of the tokens of probability zero
+    that end the vocabulary."""
+    b = tv.Bank(64, 0)
+    zeros = 1000
+    z = np.full((1, V), np.float64(np.float32(T * np.log(2.0 ** -13 / (V - zeros)))))
+    z[0, 3] = 0.0
+    z[0, V - zeros:] = -2000.0
+    p = np.exp(z[0] / T)
+    p[V - zeros:] = 0.0
+    cdf = np.cumsum(p / p.sum())
+    q = np.full((1, V), 1.0 / V)
+    tol = 2.0 ** -19
+    for u in np.concatenate([1.0 - np.linspace(2.0 ** -13, 0.0, 24, endpoint=False), [1.0 - 2.0 ** -24, 0.5, 0.0]]):
+        u = float(np.float32(min(u, 1.0 - 2.0 ** -24)))
+        tok = _walk_on_gpu(dev, b, np.array([-1], np.int32), [0], z, q, np.array([0.0, u]), T)["bonus_token"]
+        assert 0 <= tok < V - zeros, (u, tok)
+        assert (cdf[tok - 1] if tok > 0 else 0.0) - tol <= u <= cdf[tok] + tol, (u, tok, cdf[tok])
+    b.close()
+
+
 def test_walk_is_lossless_on_the_gpu(dev):
     """Root with three children drawn from q: the first emitted token follows p."""
     b = tv.Bank(4, 0)
