@@ -197,3 +197,54 @@ def draw_decidable_walk(g, parent, z, q, temp, p_from_q=0.8):
         if (np.abs(tried[np.isfinite(tried)]) > WALK_MARGIN).all() and det["cdf_margin"] > WALK_MARGIN:
             return draft, unif, (k, path, tok)
     raise RuntimeError("no unambiguous uniforms")
+
+
+# One step of one sequence in each structure the host may enqueue it in (the
+# host test asserts which one a shape takes on 152 SMs): the structure, the tree,
+# prefix, layers, query and kv heads, d_model, vocabulary, rotary embedding.
+# Vocabularies from 38912 on leave no SM beside a round of the LM head's CTAs,
+# whatever d_model, so that small shapes reach the structures of large ones.
+_BANK = synth.bank_trees()
+STEP_STRUCTURES = [
+    # the attention on the SMs that a round of the LM head leaves free: the whole grid, and a share
+    ("beside", _BANK[5], 300, 1, 8, 2, 256, 1000, False),
+    ("beside", _BANK[5], 3000, 1, 8, 8, 256, 1000, False),
+    ("beside", _BANK[6], 1500, 2, 32, 8, 256, 1000, True),
+    # clusters share the attention's units, the LM head in its tail; with the rotary
+    # embedding the attention kernel rotates, unless two row blocks read the tree tiles
+    ("clusters", _BANK[5], 1500, 1, 8, 8, 64, 40000, False),
+    ("clusters", _BANK[7], 2100, 1, 32, 8, 64, 40000, False),
+    ("clusters_rotating", _BANK[5], 1500, 1, 8, 8, 64, 40000, True),
+    ("clusters_rotating", _BANK[5], 100, 2, 8, 8, 64, 40000, True),
+    ("clusters", _BANK[7], 1500, 1, 32, 8, 64, 40000, True),
+    # the even split over every SM, its merge behind the acceptance kernel: up to 32 rows, a short LM head
+    ("chain", _BANK[5], 300, 5, 32, 32, 64, 40000, False),
+    ("chain", _BANK[5], 300, 5, 32, 32, 64, 40000, True),
+    ("chain", _BANK[6], 300, 5, 32, 32, 64, 40000, False),
+    ("chain", _BANK[7], 700, 10, 32, 8, 64, 40000, False),  # two row blocks side by side
+    # ... its merge beside an LM head on the bank's helper stream: many tiles, a long LM head
+    ("fork", _BANK[6], 2100, 5, 32, 32, 64, 40000, False),
+    ("fork", _BANK[6], 2100, 5, 32, 32, 64, 40000, True),
+    ("fork", _BANK[6], 300, 5, 32, 32, 1608, 40000, False),
+]
+# the same for device-driven steps: d_model, vocabulary, prefix of the first step
+SCHEDULED_STRUCTURES = [
+    ("fork", 256, 1000, 100),
+    ("beside", 1024, 8000, 900),   # the whole grid beside the LM head
+    ("beside", 1024, 8000, 5000),  # a share of the SMs
+]
+SCHEDULED_HEADS = (2, 4, 2, 128)  # layers, query and kv heads, head_dim
+SCHEDULED_STEPS = 10
+
+
+def structure_id(case):
+    structure, parent, L, layers, Hq, Hkv, D, V, rope = case
+    return f"{structure}-{len(parent)}nodes-L{L}-{layers}x{Hq}/{Hkv}-{D}x{V}" + ("-rope" if rope else "")
+
+
+# Steps that several threads run on one bank: trees, prefix, layers, query and kv
+# heads, d_model, vocabulary
+THREAD_STEPS = {
+    "chain": ([synth.full_tree((2, 2)), _BANK[5], _BANK[7]], 300, 1, 8, 2, 256, 1000),
+    "fork": ([synth.chain(33), _BANK[6], _BANK[7]], 2000, 5, 32, 32, 64, 40000),
+}

@@ -5,6 +5,7 @@ Bit-exact: argmax, accept_len, path, bonus token, compacted KV bytes.
 Attention: max-abs <= 1e-2 and mean-abs <= 1e-3.  top-1 / entropy: <= 1e-3 abs.
 Hidden rows are drawn with an oracle top-2 logit gap > 1e-2.
 """
+import re
 import zlib
 
 import numpy as np
@@ -367,11 +368,11 @@ def test_verify_step_full_parity(dev, bank, cfg):
     assert np.array_equal(bits(vd), oracle.kv_compact(case.v, case.L, path))
 
 
-# Steps whose LM head is longer than their attention: the attention grid is then
-# capped at the SMs the LM head's CTAs leave free, so that both start at once.
-# On a 152-SM GB300 these shapes get: 73 attention CTAs over 136 tiles (units
-# of 17 tiles spread over several CTAs); 27 over 160 (units of 40 tiles); 27
-# over 64 (units of 2 tiles); 54 over 128 across two layers with GQA group 4.
+# Steps whose LM head is longer than their attention: the SMs are divided so
+# that both start at once and neither waits long for the other.  On a 152-SM GB300
+# the attention of these shapes gets (test_host_launches.py): 12 CTAs over 136 tiles
+# and 9 over 160 (units of 17 and 40 tiles spread over several CTAs); 4 over 64
+# (units of 2 tiles); 19 over 128 across two layers with GQA group 4.
 BESIDE_LM = [
     # parent, L, layers, Hq, Hkv, D, V
     (synth.shape_c2().parent, 2048, 1, 8, 8, 4096, 20000),
@@ -396,6 +397,63 @@ def test_verify_step_beside_lm_head(dev, bank, parent, L, layers, Hq, Hkv, D, V)
     assert (r["accept_len"], r["path"], r["bonus_token"], r["new_L"], r["status"]) == (k, path, bonus, L + k, 0)
     assert np.array_equal(bits(kd), oracle.kv_compact(case.k, L, path))
     assert np.array_equal(bits(vd), oracle.kv_compact(case.v, L, path))
+
+
+def _least_workspace(dev, call):
+    """The smallest workspace the call accepts (less than tb_workspace_size), zeroed."""
+    with pytest.raises(tv.TreeVerifyError) as e:
+        call(tv.make_workspace(256, dev))
+    assert e.value.status == tv.TB_ECAPACITY
+    return tv.make_workspace(int(re.search(r"(\d+) needed", str(e.value))[1]), dev)
+
+
+@pytest.mark.parametrize("R,D,V", [(26, 256, 40000), (64, 128, 100003), (200, 256, 64001), (26, 1024, 1000)])
+def test_lm_head_stats_in_the_least_workspace(dev, R, D, V):
+    """Without room for the partials of lower tiles (several rounds of them per CTA)
+    the vocabulary runs in tiles of 128 entries; the guards around the workspace
+    show that its room is enough for that, for CTA pairs and for shared tiles."""
+    W = synth.gen_lm_head(V + R, V, D)
+    hidden, am, t1, en = gap_filtered_hidden(R * 5 + D, R, W)
+    h, w = to_dev(hidden, dev), to_dev(W, dev)
+    o = (torch.full((R,), -1, dtype=torch.int32, device=dev), torch.empty(R, dtype=torch.float32, device=dev),
+         torch.empty(R, dtype=torch.float32, device=dev))
+    ws = _least_workspace(dev, lambda ws: tv.lm_head_stats(h, w, *o, ws))
+    assert ws.numel() < tv.tb_workspace_size(R, 1, 1, 1, 0, V, 0)
+    for _ in range(2):
+        tv.lm_head_stats(h, w, *o, ws)
+        torch.cuda.synchronize()
+        assert tv.tb_workspace_status(ws) == 0
+        assert np.array_equal(o[0].cpu().numpy(), am)
+        assert np.abs(o[1].cpu().numpy() - t1).max() <= STAT_TOL and np.abs(o[2].cpu().numpy() - en).max() <= STAT_TOL
+
+
+@pytest.mark.parametrize("V,L", [(1000, 300), (40000, 1500), (40000, 12000)])
+def test_verify_step_in_the_least_workspace(dev, bank, V, L):
+    """A step whose head shares the SMs with the attention, follows it, or is one of
+    several rounds, in the smallest workspace that it accepts."""
+    c = make_case(61, synth.bank_trees()[6], L, 1, 8, 8, 128, 256, V, 0.7)
+    bid, _ = bank.add(c.parent)
+    kv = tv.KvCache(to_dev(c.k, dev), to_dev(c.v, dev), L)
+    args = (to_dev(c.q, dev), to_dev(c.hidden, dev), to_dev(c.W, dev), to_dev(c.drafts.astype(np.int32), dev))
+    out = torch.empty((1, c.N, 8, 128), dtype=torch.bfloat16, device=dev)
+    am, res = torch.empty(c.N, dtype=torch.int32, device=dev), tv.make_result(dev)
+    t1, en = (torch.empty(c.N, dtype=torch.float32, device=dev) for _ in range(2))
+
+    def step(ws):
+        tv.verify_step(bank, bid, kv, *args, out, am, t1, en, res, ws, tv.TB_NO_COMPACT)
+
+    ws = _least_workspace(dev, step)
+    for _ in range(2):
+        step(ws)
+        torch.cuda.synchronize()
+        assert tv.tb_workspace_status(ws) == 0
+        check_attention(out[0].float().cpu().numpy(), oracle.tree_attention(c.q[0], c.k[0], c.v[0], L, c.parent))
+        assert np.array_equal(am.cpu().numpy(), c.argmax)
+        assert np.abs(t1.cpu().numpy() - c.top1).max() <= STAT_TOL
+        assert np.abs(en.cpu().numpy() - c.entropy).max() <= STAT_TOL
+        k, path, bonus = oracle.accept(c.parent, c.drafts, c.argmax)
+        r = tv.parse_result(res)
+        assert (r["accept_len"], r["path"], r["bonus_token"], r["status"]) == (k, path, bonus, 0)
 
 
 def test_verify_step_no_compact_flag(dev, bank):

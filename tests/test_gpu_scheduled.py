@@ -12,7 +12,8 @@ import numpy as np
 import pytest
 
 import oracle
-from helpers import STAT_TOL, bits, check_attention, gap_filtered_hidden, to_dev
+from helpers import (SCHEDULED_HEADS, SCHEDULED_STEPS, SCHEDULED_STRUCTURES, STAT_TOL, bits, check_attention,
+                     gap_filtered_hidden, to_dev)
 from paper_2606_27550_gb300 import synth
 
 torch = pytest.importorskip("torch")
@@ -20,7 +21,8 @@ tv = pytest.importorskip("paper_2606_27550_gb300")
 
 pytestmark = pytest.mark.gpu
 
-LAYERS, HQ, HKV, D_HEAD, D_MODEL, V = 2, 4, 2, 128, 256, 1000
+LAYERS, HQ, HKV, D_HEAD = SCHEDULED_HEADS
+D_MODEL, V = 256, 1000
 TREES = synth.bank_trees()
 N_MAX = max(len(t) for t in TREES)
 
@@ -39,7 +41,8 @@ class Loop:
     N_MAX nodes and one draft row per rung (drafts copy the parent's oracle
     greedy token with probability p_match)."""
 
-    def __init__(self, dev, steps, L0, seed=0, p_match=0.7, rungs=tuple(range(len(TREES))), d_head=D_HEAD):
+    def __init__(self, dev, steps, L0, seed=0, p_match=0.7, rungs=tuple(range(len(TREES))), d_head=D_HEAD,
+                 d_model=D_MODEL, vocab=V, rope_theta=0.0):
         self.dev, self.steps, self.L0 = dev, steps, L0
         self.trees = [TREES[i] for i in rungs]  # the tree of each rung; draft rows follow the rungs
         self.L_cap = L0 + steps * 7 + N_MAX + 8
@@ -47,7 +50,8 @@ class Loop:
         self.ids = [self.bank.add(t)[0] for t in self.trees]
         # every slot holds finite random K/V (the tree slots of each step are read where L lands)
         self.k, self.v = synth.gen_kv(seed, LAYERS, HKV, self.L_cap, d_head, self.L_cap)
-        self.W = synth.gen_lm_head(seed, V, D_MODEL)
+        self.W = synth.gen_lm_head(seed, vocab, d_model)
+        self.rope_theta = rope_theta
         self.q = [synth.gen_q(seed + 10 + t, LAYERS, N_MAX, HQ, d_head) for t in range(steps)]
         self.h, self.am, self.t1, self.en = [], [], [], []
         self.drafts = []
@@ -59,7 +63,7 @@ class Loop:
             self.en.append(en)
             rows = np.zeros((len(self.trees), N_MAX), np.int32)
             for r, tr in enumerate(self.trees):
-                rows[r, :len(tr)] = synth.gen_drafts(seed + 1000 * t + r, tr, am[:len(tr)], V, p_match)
+                rows[r, :len(tr)] = synth.gen_drafts(seed + 1000 * t + r, tr, am[:len(tr)], vocab, p_match)
             self.drafts.append(rows)
         self.kd, self.vd = to_dev(self.k, dev), to_dev(self.v, dev)
         self.Wd = to_dev(self.W, dev)
@@ -71,14 +75,15 @@ class Loop:
         self.g_t1 = torch.empty(N_MAX, dtype=torch.float32, device=dev)
         self.g_en = torch.empty(N_MAX, dtype=torch.float32, device=dev)
         self.res = tv.make_result(dev)
-        self.ws = tv.make_workspace(tv.tb_workspace_size(N_MAX, LAYERS, HKV, HQ, d_head, V, 0), dev)
+        self.ws = tv.make_workspace(tv.tb_workspace_size(N_MAX, LAYERS, HKV, HQ, d_head, vocab, 0), dev)
 
     def kv(self):
-        return tv.KvCache(self.kd, self.vd, 0)
+        return tv.KvCache(self.kd, self.vd, 0, rope_theta=self.rope_theta)
 
-    def step(self, t, policy, state, flags=0, stream=None):
+    def step(self, t, policy, state, flags=0, stream=None, out=None, res=None):
         tv.verify_step_scheduled(self.bank, policy, state, self.kv(), self.qd[t], self.hd[t], self.Wd, self.dd[t],
-                                 self.out, self.g_am, self.g_t1, self.g_en, self.res, self.ws, flags, stream)
+                                 self.out if out is None else out, self.g_am, self.g_t1, self.g_en,
+                                 self.res if res is None else res, self.ws, flags, stream)
 
 
 def _trace(steps, seed=3):
@@ -180,6 +185,80 @@ def test_scheduled_graph_replay_matches_eager(dev):
         assert torch.equal(lp.out.view(torch.int16), eager[3].view(torch.int16))
         assert tv.parse_result(lp.res) == eager[4]
     assert eager[0]["step"] == steps and eager[0]["L"] > lp.L0
+    lp.bank.close()
+
+
+@pytest.mark.parametrize("rope", [False, True])
+@pytest.mark.parametrize("structure,d_model,vocab,L0", SCHEDULED_STRUCTURES)
+def test_scheduled_steps_back_to_back(dev, structure, d_model, vocab, L0, rope):
+    """Steps behind one another without a wait of the host, each on another tree
+    than the one before, in both structures of a device-driven step
+    (test_host_launches.py asserts which): every step's attention is that of the
+    tree and prefix the state held when it ran, though the merge of its split units
+    runs beside the acceptance kernel that advances the state.  Then the same
+    steps as one CUDA graph, byte for byte."""
+    steps = SCHEDULED_STEPS
+    lp = Loop(dev, steps, L0=L0, seed=6, d_model=d_model, vocab=vocab, rope_theta=10000.0 if rope else 0.0)
+    up, down = 1.0, 3.0
+    trace = np.array([up, up, down, up, up, down, down, up, up, up], np.float32)
+    assert len(trace) == steps
+    tr_d = to_dev(trace, dev)
+    pol = tv.make_policy(tv.TB_POLICY_HYSTERETIC_LADDER, tv.TB_FEATURE_TRACE, lp.ids, a=1.5, b=2.5, trace=tr_d,
+                         node_stride=N_MAX)
+    k0, v0 = lp.kd.clone(), lp.vd.clone()
+    state = tv.make_state(4, L0, dev)
+
+    def run(stream=None):
+        for t in range(steps):
+            lp.step(t, pol, state, 0, stream, outs[t], ress[t])
+
+    def buffers():
+        return ([torch.zeros((LAYERS, N_MAX, HQ, D_HEAD), dtype=torch.bfloat16, device=dev) for _ in range(steps)],
+                [tv.make_result(dev) for _ in range(steps)])
+
+    outs, ress = buffers()
+    run()
+    torch.cuda.synchronize()
+    k_ref, v_ref, rung, L = lp.k.copy(), lp.v.copy(), 4, L0
+    for t in range(steps):
+        tree = np.asarray(TREES[rung], np.int32)
+        n = len(tree)
+        got = outs[t].float().cpu().numpy()
+        for layer in range(LAYERS):
+            if rope:
+                ref, k_rot = oracle.tree_attention_rope(lp.q[t][layer][:n], k_ref[layer], v_ref[layer], L, tree, 10000.0)
+                k_ref[layer][:, L:L + n] = k_rot
+            else:
+                ref = oracle.tree_attention(lp.q[t][layer][:n], k_ref[layer], v_ref[layer], L, tree)
+            check_attention(got[layer][:n], ref, f"step {t} layer {layer}")
+        ka, path, bonus = oracle.accept(tree, lp.drafts[t][rung][:n], lp.am[t][:n])
+        r = tv.parse_result(ress[t])
+        assert (r["accept_len"], r["path"], r["bonus_token"], r["new_L"], r["status"]) == (ka, path, bonus, L + ka, 0), t
+        k_ref, v_ref = oracle.kv_compact(k_ref, L, path), oracle.kv_compact(v_ref, L, path)
+        rung, L = oracle.policy_next("ladder", rung, len(TREES), float(trace[t]), 1.5, 2.5), L + ka
+    assert np.array_equal(bits(lp.vd), v_ref)
+    assert rope or np.array_equal(bits(lp.kd), k_ref)
+    want, eager, k1 = tv.parse_state(state), (outs, ress), lp.kd.clone()
+    assert (want["rung"], want["L"], want["step"]) == (rung, L, steps)
+
+    outs, ress = buffers()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        run(s)
+    for _ in range(2):
+        lp.kd.copy_(k0)
+        lp.vd.copy_(v0)
+        state.copy_(tv.make_state(4, L0, dev))
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert tv.parse_state(state) == want
+        assert torch.equal(lp.kd.view(torch.int16), k1.view(torch.int16))
+        for t in range(steps):
+            assert torch.equal(outs[t].view(torch.int16), eager[0][t].view(torch.int16)), t
+            assert torch.equal(ress[t], eager[1][t]), t
     lp.bank.close()
 
 

@@ -1,12 +1,13 @@
 """Several host threads sharing one TopologyBank, each with its own stream,
 cache, workspace and result block, calling verify_step concurrently.
 
-Two step structures: a short attention that fits beside the LM head runs as
+Two step structures: an attention that shares the SMs with the LM head runs as
 one chain on the caller's stream (each new thread's first call then encodes
-its tensor maps before any other CUDA call of that thread); a longer one
+its tensor maps before any other CUDA call of that thread); one of many tiles
 forks the LM head onto the bank's helper stream, whose fork / join events are
 shared and held under the bank's mutex, so the steps of different threads
-never interleave their fork / join sequences.  Every step of every thread
+never interleave their fork / join sequences (test_host_launches.py asserts
+that the shapes run here take them).  Every step of every thread
 must still match the fp64 oracle exactly (argmax, acceptance, path, bonus)
 and within the attention tolerance, and the compacted caches must equal the
 oracle's.
@@ -17,7 +18,7 @@ import numpy as np
 import pytest
 
 import oracle
-from helpers import STAT_TOL, bits, check_attention, make_case, to_dev
+from helpers import STAT_TOL, THREAD_STEPS, bits, check_attention, make_case, to_dev
 from paper_2606_27550_gb300 import synth
 
 torch = pytest.importorskip("torch")
@@ -36,17 +37,16 @@ def dev():
 
 
 @pytest.mark.parametrize("d", [128, 64])
-@pytest.mark.parametrize("structure,Hkv,L", [("chain", 2, 300), ("fork", 8, 3000)])
-def test_threads_share_a_bank(dev, d, structure, Hkv, L):
-    trees = [synth.full_tree((2, 2)), synth.bank_trees()[5], synth.bank_trees()[-1]]
+@pytest.mark.parametrize("structure", THREAD_STEPS)
+def test_threads_share_a_bank(dev, d, structure):
+    trees, L, layers, H, Hkv, D, V = THREAD_STEPS[structure]
     bank = tv.Bank(8, 0)
     ids = [bank.add(t)[0] for t in trees]
     n_threads, steps = 4, 12
-    H, D, V = 8, 256, 1000
     workers = []
     for w in range(n_threads):
         j = w % len(trees)
-        case = make_case(500 + 10 * w + d, trees[j], L, 1, H, Hkv, d, D, V, 0.7)
+        case = make_case(500 + 10 * w + d, trees[j], L, layers, H, Hkv, d, D, V, 0.7)
         N = case.N
         workers.append({
             "case": case, "id": ids[j], "N": N,
@@ -54,12 +54,12 @@ def test_threads_share_a_bank(dev, d, structure, Hkv, L):
             "k": to_dev(case.k, dev), "v": to_dev(case.v, dev), "q": to_dev(case.q, dev),
             "h": to_dev(case.hidden, dev), "W": to_dev(case.W, dev),
             "drafts": to_dev(case.drafts.astype(np.int32), dev),
-            "out": torch.empty((1, N, H, d), dtype=torch.bfloat16, device=dev),
+            "out": torch.empty((layers, N, H, d), dtype=torch.bfloat16, device=dev),
             "am": torch.empty(N, dtype=torch.int32, device=dev),
             "t1": torch.empty(N, dtype=torch.float32, device=dev),
             "en": torch.empty(N, dtype=torch.float32, device=dev),
             "res": tv.make_result(dev),
-            "ws": tv.make_workspace(tv.tb_workspace_size(N, 1, Hkv, H, d, V, 0), dev),
+            "ws": tv.make_workspace(tv.tb_workspace_size(N, layers, Hkv, H, d, V, 0), dev),
             "got": [], "error": None,
         })
     torch.cuda.synchronize()
@@ -90,11 +90,12 @@ def test_threads_share_a_bank(dev, d, structure, Hkv, L):
     for wk in workers:
         assert wk["error"] is None, wk["error"]
         c = wk["case"]
-        ref_o = oracle.tree_attention(c.q[0], c.k[0], c.v[0], L, c.parent)
+        ref_o = [oracle.tree_attention(c.q[i], c.k[i], c.v[i], L, c.parent) for i in range(layers)]
         ka, path, bonus = oracle.accept(c.parent, c.drafts, c.argmax)
         assert len(wk["got"]) == steps
         for t, (o, am, en, r) in enumerate(wk["got"]):
-            check_attention(o[0], ref_o, f"step {t}")
+            for i in range(layers):
+                check_attention(o[i], ref_o[i], f"step {t} layer {i}")
             assert np.array_equal(am, c.argmax), f"step {t}"
             assert np.abs(en - c.entropy).max() <= STAT_TOL
             assert (r["accept_len"], r["path"], r["bonus_token"], r["new_L"], r["status"]) == \
