@@ -1027,9 +1027,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k1_tree_attention_tc(const __gr
 #pragma unroll
             for (int k = 0; k < kMaxCluster; ++k)
                 if (k < n)
-                    v[k] = ld_cluster_f32x4(cluster_map(o_addr, k));
-            const float m = sub < n ? ld_cluster_f32(cluster_map(m_base + 4 * r, sub)) : -INFINITY;
-            const float l = sub < n ? ld_cluster_f32(cluster_map(l_base + 4 * r, sub)) : 0.f;
+                    v[k] = ld_cluster_f32x4(cluster_addr(o_addr, k));
+            const float m = sub < n ? ld_cluster_f32(cluster_addr(m_base + 4 * r, sub)) : -INFINITY;
+            const float l = sub < n ? ld_cluster_f32(cluster_addr(l_base + 4 * r, sub)) : 0.f;
             float M = m;
 #pragma unroll
             for (int k = kMaxCluster / 2; k >= 1; k >>= 1)
@@ -1248,17 +1248,13 @@ static TcKernelParams<false> one_seq(const TcParams &p)
 }
 
 // The split-unit merge of an attention launch with parameters p, for head_dim
-// kD.  after_step: see k1_merge_split.
-template <int kD>
-static cudaError_t merge_launch_d(const TcParams &p, bool batched, cudaStream_t stream, bool pdl, bool after_step)
+// kD.
+template <int kD, bool kBatched, bool kAfterStep>
+static cudaError_t merge_launch_d(const TcKernelParams<kBatched> &p, cudaStream_t stream, bool pdl)
 {
     // scheduled mode chooses row_split on the device: the grid covers both choices
     const dim3 grid((p.sched ? p.P : p.P / p.seq[0].row_split) - 1, (p.max_rows + 7) / 8);
-    if (batched)
-        return after_step ? launch_kernel(k1_merge_split<kD, true, true>, grid, dim3(256), 0, stream, pdl, p)
-                          : launch_kernel(k1_merge_split<kD, true, false>, grid, dim3(256), 0, stream, pdl, p);
-    return after_step ? launch_kernel(k1_merge_split<kD, false, true>, grid, dim3(256), 0, stream, pdl, one_seq(p))
-                      : launch_kernel(k1_merge_split<kD, false, false>, grid, dim3(256), 0, stream, pdl, one_seq(p));
+    return launch_kernel(k1_merge_split<kD, kBatched, kAfterStep>, grid, dim3(256), 0, stream, pdl, p);
 }
 
 // Whether a CTA range of the launch starts inside a unit (the split merge then
@@ -1281,13 +1277,16 @@ static bool any_split(const TcParams &p)
     return false;
 }
 
-// The split-unit merge, when the launch split a unit (nothing to do otherwise).
-static cudaError_t merge_launch(const TcParams &p, bool batched, cudaStream_t stream, bool pdl, bool after_step)
+// The split-unit merge right behind the attention, when the launch split a unit
+// (nothing to do otherwise).
+static cudaError_t merge_launch(const TcParams &p, bool batched, cudaStream_t stream, bool pdl)
 {
     if (!any_split(p))
         return cudaSuccess;
-    return p.d == 64 ? merge_launch_d<64>(p, batched, stream, pdl, after_step)
-                     : merge_launch_d<128>(p, batched, stream, pdl, after_step);
+    if (batched)
+        return p.d == 64 ? merge_launch_d<64, true, false>(p, stream, pdl) : merge_launch_d<128, true, false>(p, stream, pdl);
+    const TcKernelParams<false> one = one_seq(p);
+    return p.d == 64 ? merge_launch_d<64, false, false>(one, stream, pdl) : merge_launch_d<128, false, false>(one, stream, pdl);
 }
 
 // The attention kernel for p.d, one CTA per SM (each holds 512 TMEM columns).
@@ -1350,13 +1349,12 @@ static int attn_max_clusters(int size)
 }
 
 // The attention launch's parameters, kept for a split-unit merge enqueued later.
-static void stash_merge(const TcParams &p, bool batched, AttnMerge *m)
+static void stash_merge(const TcParams &p, AttnMerge *m)
 {
-    static_assert(sizeof(TcParams) <= sizeof(m->params), "AttnMerge holds the attention launch's parameters");
-    TcParams q = p;
+    TcKernelParams<false> q = one_seq(p);
+    static_assert(sizeof q <= sizeof(m->params), "AttnMerge holds the attention launch's parameters");
     q.sched = p.sched ? p.sched_copy : nullptr;
     memcpy(m->params, &q, sizeof q);
-    m->batched = batched;
     m->pending = any_split(p);
 }
 
@@ -1468,7 +1466,7 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
                                  int *status, int n_sm, cudaStream_t stream, const char **err,
                                  const float2 *rope_tab, AttnMerge *merge_later, bool alone)
 {
-    if (n_seq < 1 || n_seq > kMaxSeqPerLaunch) {
+    if (n_seq < 1 || n_seq > kMaxSeqPerLaunch || (n_seq > 1 && merge_later)) {
         *err = "too many sequences for one attention launch";
         return cudaErrorInvalidValue;
     }
@@ -1553,14 +1551,14 @@ cudaError_t attn_tc_launch_batch(const AttnSeq *seqs, int n_seq, int layer_begin
     if ((e = attn_kernel_launch(p, batched, stream, pdl, seqs[0].kv)) != cudaSuccess)
         return e;
     if (merge_later) {
-        stash_merge(p, batched, merge_later);
+        stash_merge(p, merge_later);
         return cudaSuccess;
     }
     // In a step, a plain dependent of the attention: launched as a programmatic
     // one, its CTAs would take the SMs that attention CTAs release and hold them until
     // the whole grid is done, away from an LM head beside it on another stream
     // (measured on GB300: the ragged batch's step 20 us longer).
-    return merge_launch(p, batched, stream, alone, false);
+    return merge_launch(p, batched, stream, alone);
 }
 
 cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *status, int n_sm,
@@ -1614,11 +1612,11 @@ cudaError_t attn_tc_launch_sched(const AttnSched &sc, int Hq, float *part, int *
     if ((e = attn_kernel_launch(p, false, stream, merge_later != nullptr)) != cudaSuccess)
         return e;
     if (merge_later) {
-        stash_merge(p, false, merge_later);
+        stash_merge(p, merge_later);
         return cudaSuccess;
     }
     p.sched = p.sched_copy;
-    return merge_launch(p, false, stream, false, false);
+    return merge_launch(p, false, stream, false);
 }
 
 cudaError_t attn_tc_launch(const tb_kv *kv, const TreeDesc *d_tree, int N, int layer_begin, int n_layers,
@@ -1631,13 +1629,13 @@ cudaError_t attn_tc_launch(const tb_kv *kv, const TreeDesc *d_tree, int N, int l
                                 merge_later, alone);
 }
 
-cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream, bool after_step)
+cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream)
 {
     if (!m.pending)
         return cudaSuccess;
-    TcParams p;
+    TcKernelParams<false> p;
     memcpy(&p, m.params, sizeof p);
-    return merge_launch(p, m.batched, stream, true, after_step);
+    return p.d == 64 ? merge_launch_d<64, false, true>(p, stream, true) : merge_launch_d<128, false, true>(p, stream, true);
 }
 
 TB_BOUNDS_COUNTER(bounds_violations_attention_tc)

@@ -247,20 +247,18 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
     return r;
 }
 
-// The shared::cluster address of `p`'s counterpart in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-    return r;
-}
-
-// As cluster_addr, from a shared::cta address.
-__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank)
+// The shared::cluster address of the counterpart, in CTA `rank` of the cluster,
+// of a shared::cta address or of `p`.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
 {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
+}
+
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank)
+{
+    return cluster_addr(smem_u32(p), rank);
 }
 
 // Loads from the shared memory of any CTA of the cluster.

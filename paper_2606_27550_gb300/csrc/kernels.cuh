@@ -174,16 +174,14 @@ struct AttnSeq {
     void *out;
 };
 int attn_tc_units(const AttnSeq *seqs, int n_seq, int Hq, int Hkv, int n_layers);
-// The split-unit merge of an attention launch, kept to be enqueued later in a
-// verification step by attn_merge_launch, as a programmatic dependent of the
-// stream's previous kernel: after the LM head, or (after_step) after the
-// acceptance kernel, beside which it runs.
+// The split-unit merge of an attention launch of one sequence, kept to be
+// enqueued later in a verification step by attn_merge_launch, as a programmatic
+// dependent of the acceptance kernel, beside which it runs.
 struct AttnMerge {
     bool pending;
-    bool batched;
-    alignas(64) unsigned char params[8192];
+    alignas(64) unsigned char params[1024];
 };
-cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream, bool after_step);
+cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream);
 // rope_tab: null, or the (cos, sin) tables of rope.cu: the queries are then
 // pre-rotary and are rotated at L + depth while they are staged
 // merge_later: the split-unit merge is not enqueued but kept there, and the

@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) k2_lm_head_split(const __gri
 #pragma unroll
                 for (int k = 0; k < kMaxSplit; ++k)
                     if (k < n)
-                        part[k] = ld_cluster_f32x4(cluster_map(addr, k));
+                        part[k] = ld_cluster_f32x4(cluster_addr(addr, k));
                 z[y][0] = z[y][1] = z[y][2] = z[y][3] = 0.f;
 #pragma unroll
                 for (int k = 0; k < kMaxSplit; ++k)
@@ -900,9 +900,10 @@ __global__ void __launch_bounds__(kMergeThreads) k2_lm_merge(const __grid_consta
         return;
     if (!in_bounds(r < p.R, p.status))
         return;
-    // A thread's slots k = tid + 256 u.  Up to 256 x kInFlight slots (every
-    // vocabulary up to 131072) its partials are loaded once and both passes
-    // read registers; beyond that pass 2 reads them again.
+    // A thread's slots k = tid + 256 u.  Up to 256 x kInFlight slots its partials
+    // are loaded once and both passes read registers; beyond that (131072
+    // vocabulary entries in 128-entry tiles, less in lower ones: 1060 slots of 121
+    // entries at V 128256) pass 2 reads them again, from L2.
     const bool held = p.n_slots <= kMergeThreads * kInFlight;
     float4 v[kInFlight];
     float2 w[kInFlight];

@@ -322,10 +322,10 @@ class StepStreams {
         return e == cudaSuccess ? TB_OK : fail(TB_ECUDA, "%s: join: %s", fn, cudaGetErrorString(e));
     }
     bool accept_pdl() const { return chain_; }
-    // the kept split-unit merge; after_step: behind the acceptance kernel (see k1_merge_split)
-    tb_status merge(const char *fn, bool after_step)
+    // the kept split-unit merge, enqueued behind the acceptance kernel (see k1_merge_split)
+    tb_status merge(const char *fn)
     {
-        cudaError_t e = chain_ ? attn_merge_launch(merge_, s_, after_step) : cudaSuccess;
+        cudaError_t e = chain_ ? attn_merge_launch(merge_, s_) : cudaSuccess;
         return e == cudaSuccess ? TB_OK : fail(TB_ECUDA, "%s: split-unit merge: %s", fn, cudaGetErrorString(e));
     }
 
@@ -1177,7 +1177,7 @@ extern "C" tb_status verify_step_sampled(const tb_bank *bank, int bank_id, const
         if (e != cudaSuccess)
             return cuda_fail(e, fn);
     }
-    if ((st = ss.merge(fn, true)) != TB_OK)
+    if ((st = ss.merge(fn)) != TB_OK)
         return st;
     return ok();
 }
@@ -1255,7 +1255,7 @@ static tb_status verify_step_impl(const tb_bank *bank, int bank_id, const tb_kv 
     cudaError_t e = accept_launch(p, sm_count(bank->device), s, ss.accept_pdl());
     if (e != cudaSuccess)
         return cuda_fail(e, fn);
-    if ((st = ss.merge(fn, true)) != TB_OK)
+    if ((st = ss.merge(fn)) != TB_OK)
         return st;
     return ok();
 }
@@ -1365,8 +1365,7 @@ static tb_status verify_step_batched_impl(const tb_bank *bank, int batch, const 
             return st;
         const char *err = "";
         e = attn_tc_launch_batch(as, batch, 0, kv0.n_layers, n_q_heads, reinterpret_cast<float *>(ws + kPartBase),
-                                 reinterpret_cast<int *>(ws), nsm, s, &err, rope ? rope_table(ws) : nullptr,
-                                 ss.merge_later());
+                                 reinterpret_cast<int *>(ws), nsm, s, &err, rope ? rope_table(ws) : nullptr);
         if (e == cudaErrorInvalidValue && err[0])
             return fail(TB_EINVAL, "%s: %s", fn, err);
         if (e != cudaSuccess)
@@ -1393,10 +1392,10 @@ static tb_status verify_step_batched_impl(const tb_bank *bank, int batch, const 
                 sr += Ns[b];
             }
         }
-        // the chunks share the partials and counters: only the first overlaps the attention
+        // the chunks share the partials and counters: each runs after the one before
         if ((st = lm_enqueue(h8 + (size_t)r0 * d_model * 2, rc, lm_head, d_model, vocab, argmax + r0, top1 + r0,
                              entropy + r0, ws, workspace_bytes, kPartBase + attn_bytes, ss.lm_stream(), fn, 0,
-                             typ ? &lt : nullptr, ss.lm_pdl() && r0 == 0, 0, !ss.chain())) != TB_OK)
+                             typ ? &lt : nullptr, false, 0, true)) != TB_OK)
             return st;
     }
     if ((st = ss.before_accept(fn)) != TB_OK)
@@ -1413,11 +1412,9 @@ static tb_status verify_step_batched_impl(const tb_bank *bank, int batch, const 
             add_compaction(ps[b], &seqs[b].kv);
         r0 += Ns[b];
     }
-    e = accept_launch_batch(ps, batch, nsm, s, ss.accept_pdl());
+    e = accept_launch_batch(ps, batch, nsm, s, false);
     if (e != cudaSuccess)
         return cuda_fail(e, fn);
-    if ((st = ss.merge(fn, true)) != TB_OK)
-        return st;
     return ok();
 }
 
@@ -1600,7 +1597,7 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
     cudaError_t e = accept_launch(p, nsm, s, ss.accept_pdl());
     if (e != cudaSuccess)
         return cuda_fail(e, fn);
-    if ((st = ss.merge(fn, true)) != TB_OK)
+    if ((st = ss.merge(fn)) != TB_OK)
         return st;
     return ok();
 }
