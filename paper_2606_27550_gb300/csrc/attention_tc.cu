@@ -51,8 +51,9 @@
 // then weights): a masked tile's extra code, unrolled over the whole row, ran
 // once per unit from cold instruction memory and took 2 to 3 us.  Measured,
 // before and now: the 32-layer step at 1063 keys and 40 nodes (rotary
-// embedding, typical acceptance) 182 -> 159 us, at 16448 keys 1228 -> 1222 us;
-// 16 single-layer calls at 1526 keys with their head 549 -> 491 us.
+// embedding, typical acceptance) 182 -> 159 us; at 16448 keys, where the stream
+// takes all of the time, no change (1229 / 1227 us on one device, 1237 / 1244 on
+// another); 16 single-layer calls at 1526 keys with their head 549 -> 491 us.
 // TMEM columns: S0 [0,128), S1 [128,256) with P0 / P1 aliased onto their first
 // halves, O [256,256+kD), Q0 [384,384+kD/2), Q1 behind it.  Both QK^T and P V take their A operand
 // from TMEM, so each MMA reads only the 128 x 16 B operand from shared memory.
@@ -1284,9 +1285,11 @@ static cudaError_t merge_launch(const TcParams &p, bool batched, cudaStream_t st
     if (!any_split(p))
         return cudaSuccess;
     if (batched)
-        return p.d == 64 ? merge_launch_d<64, true, false>(p, stream, pdl) : merge_launch_d<128, true, false>(p, stream, pdl);
+        return p.d == 64 ? merge_launch_d<64, true, false>(p, stream, pdl)
+                         : merge_launch_d<128, true, false>(p, stream, pdl);
     const TcKernelParams<false> one = one_seq(p);
-    return p.d == 64 ? merge_launch_d<64, false, false>(one, stream, pdl) : merge_launch_d<128, false, false>(one, stream, pdl);
+    return p.d == 64 ? merge_launch_d<64, false, false>(one, stream, pdl)
+                     : merge_launch_d<128, false, false>(one, stream, pdl);
 }
 
 // The attention kernel for p.d, one CTA per SM (each holds 512 TMEM columns).
@@ -1635,7 +1638,8 @@ cudaError_t attn_merge_launch(const AttnMerge &m, cudaStream_t stream)
         return cudaSuccess;
     TcKernelParams<false> p;
     memcpy(&p, m.params, sizeof p);
-    return p.d == 64 ? merge_launch_d<64, false, true>(p, stream, true) : merge_launch_d<128, false, true>(p, stream, true);
+    return p.d == 64 ? merge_launch_d<64, false, true>(p, stream, true)
+                     : merge_launch_d<128, false, true>(p, stream, true);
 }
 
 TB_BOUNDS_COUNTER(bounds_violations_attention_tc)

@@ -31,7 +31,7 @@
 // that share each tile's k-blocks (k2_lm_head_split).
 //
 // HBM bounds it: 262 MB (V 32000 x 4096) in 45-46 us with its merge, 1.05 GB (V
-// 128256) in 160-163 us, 6.4 TB/s.  W larger than half of L2 is loaded
+// 128256, 64 rows) in 163-167 us, 6.3-6.5 TB/s.  W larger than half of L2 is loaded
 // evict-first (V 128256 168 us without).
 #include <math.h>
 #include <stdlib.h>
@@ -1126,7 +1126,9 @@ static int lm_max_pairs(size_t smem)
 {
     static PerDevice<24> pairs;  // by smem / 16 KB
     const int slot = smem / 16384 < 24 ? (int)(smem / 16384) : 23;
-    return pairs.get(slot, [smem] { return ask_max_clusters((const void *)k2_lm_head<kTyp, true>, 2, kLmThreads, smem); });
+    return pairs.get(slot, [smem] {
+        return ask_max_clusters((const void *)k2_lm_head<kTyp, true>, 2, kLmThreads, smem);
+    });
 }
 
 // k2_lm_head, then its merge as a programmatic dependent (launched while the

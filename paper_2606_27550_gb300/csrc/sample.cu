@@ -477,7 +477,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) k4_spec_sample_cluster(const 
     // begin: rounded ends and begins of neighbours need not meet, and a total may
     // be too small to move the end.  If no end lies past it (the total was rounded
     // up) the step takes the last positive one.  Every warp finds the same lane from
-    // the same numbers, so no CTA has to tell another.
+    // the same numbers, so no CTA has to tell another (V 150004: 14.7 us with an offer
+    // per CTA and a barrier behind it, 14.4 so).
     float sum = 0.f;
 #pragma unroll
     for (int r = 0; r < kCtas; ++r)

@@ -1009,7 +1009,8 @@ extern "C" tb_status typical_accept(const tb_bank *bank, int bank_id, const int3
 // tile, less on many SMs, 1.4 with every SM its own, plus 6 to 10; the LM head
 // streams at 6.3 MB/us, 0.05 on one SM.  One 7B layer, 288 tiles, against V 32000, attention on
 // 12 / 16 / 20 / 24 / 27 / 32 SMs: 52.0 / 49.0 / 51.8 / 53.0 / 53.3 / 58.1 us (past
-// 27 the LM head needs a second round); forked 61.
+// 27 the LM head needs a second round); forked 61.  The rates are those of 7B
+// shapes on 152 SMs; at other shapes they only order the two structures.
 static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp, int d_model, int vocab, int n_sm,
                                bool scheduled = false)
 {
@@ -1060,7 +1061,8 @@ static int attn_ctas_beside_lm(int whole_grid, long long tiles, const LmPlan &lp
 //    128256 76.6 / 74.7 and 194 / 189; 32 layers, 26 rows 141 / 139; 64 rows 85.0 /
 //    86.9), or beside an LM head too short to hide it (W 66 MB: 64 to 128 rows, 9 to
 //    17 tiles an SM 61 to 75 / 57 to 71; 213 tiles an SM 279 / 284; W 262 MB 85 to 97 /
-//    87 to 100).
+//    87 to 100).  Between 17 and 213 tiles an SM, and between 66 and 262 MB, nothing was
+//    measured: the lines at 16 tiles and 128 MB lie there for want of a closer one.
 static bool plan_step(AttnArgs &a, const AttnPlan &ap, const LmPlan &lp, int d_model, int vocab)
 {
     const int n_sm = sm_count(a.bank->device);
@@ -1536,7 +1538,9 @@ extern "C" tb_status verify_step_scheduled(const tb_bank *bank, const tb_policy 
     for (int r = 0; r < policy->n_rungs; ++r)
         sc.rung_tree[r] = bank->d_desc + policy->bank_ids[r];
     // The step's structure (see StepStreams), for the longest prefix the cache
-    // holds: the host does not know this step's.
+    // holds: the host does not know this step's.  So a cache with room for a long
+    // prefix is forked at a short one too: one 7B layer against V 32000 divides the
+    // SMs up to 3456 slots (57 us a step at prefix 2048) and forks from 3520 up (67).
     const AttnPlan aplan = attn_tc_plan(kv->L_cap - N_max, N_max, n_q_heads, kv->n_kv_heads, kv->n_layers, nsm);
     const int attn_grid = aplan.total < nsm ? (int)aplan.total : nsm;
     const int attn_sms = attn_ctas_beside_lm(attn_grid, aplan.total, lplan, d_model, vocab, nsm, true);
