@@ -12,7 +12,7 @@ from dataclasses import dataclass
 from paper_2606_27550_gb300 import build as tvbuild
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(tvbuild.nvcc())), "include")
+CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(tvbuild.nvcc()))), "include")
 
 
 def build_lib(out_dir: str) -> str:
